@@ -1,4 +1,5 @@
-"""ctypes binding of libtman.so: same names as the C ABI, argument marshalling only.
+"""Python binding of libtman.so: same names as the C ABI, argument marshalling only (ctypes; the calls a program makes
+per token or per prompt go through the _marshal extension instead, see csrc/marshal.cpp).
 
 Tensors are torch CUDA tensors (PyTorch supplies device memory and streams); every step of the
 path runs in the library's kernels.  There is no CPU fallback: if the shared library is missing
@@ -28,6 +29,7 @@ EXPORTS = [
 ]
 
 _lib = None
+_fast = None            # the _marshal extension, bound to the loaded library
 
 
 class TmanError(RuntimeError):
@@ -38,7 +40,7 @@ class TmanError(RuntimeError):
 
 def lib() -> C.CDLL:
     """Load libtman.so (built by paper_2511_11248_b200.build); raises if it is missing."""
-    global _lib
+    global _lib, _fast
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise FileNotFoundError(
@@ -76,8 +78,24 @@ def lib() -> C.CDLL:
         L.tman_debug_mpgemm_variant.argtypes = [i, vp, sz, vp, vp, i, i, i, i, i, vp, vp, sz, vp]
         for name in EXPORTS[2:]:
             getattr(L, name).restype = C.c_int
+        try:
+            from . import _marshal
+        except ImportError as e:
+            raise ImportError(f"the _marshal extension is missing or broken ({e}): build it with "
+                              "`python -m paper_2511_11248_b200.build`; there is no fallback path") from e
+        _marshal.bind(*[C.cast(getattr(L, name), vp).value for name in (
+            "tman_mpgemv", "tman_mpgemv_grouped", "tman_mpgemm", "tman_quantize_rows", "tman_quantize_rows_i8",
+            "tman_mpgemv_ternary", "tman_mpgemm_ternary_i8", "tman_pack_weights")])
+        _fast = _marshal
         _lib = L
     return _lib
+
+
+def _hot():
+    """The _marshal extension (loads the library on first use)."""
+    if _fast is None:
+        lib()
+    return _fast
 
 
 def _check(st: int, where: str) -> None:
@@ -89,11 +107,19 @@ def _ptr(t) -> int:
     return 0 if t is None else int(t.data_ptr())
 
 
+_current_device = _raw_stream = None
+
+
 def _stream(stream) -> int:
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    global _current_device, _raw_stream
+    if stream is not None:
+        return int(stream.cuda_stream)
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()                    # initialises CUDA in torch if nothing has yet
+        # the two lookups torch.cuda.current_stream() makes, without the Stream object around the result
+        _current_device, _raw_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+    return _raw_stream(_current_device())
 
 
 def tman_version() -> int:
@@ -128,9 +154,9 @@ def tman_read_status(workspace, stream=None) -> int:
 
 
 def tman_pack_weights(codes, scales, zeros, K, N, bits, group, packed, stream=None) -> None:
-    _check(lib().tman_pack_weights(_ptr(codes), _ptr(scales), _ptr(zeros), K, N, bits, group,
-                                   _ptr(packed), packed.numel() * packed.element_size(),
-                                   _stream(stream)), "tman_pack_weights")
+    st = _hot().pack_weights(codes, scales, zeros, K, N, bits, group, packed, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_pack_weights")
 
 
 def tman_unpack_weights(packed, K, N, bits, group, codes, scales, zeros, workspace, stream=None) -> None:
@@ -141,9 +167,9 @@ def tman_unpack_weights(packed, K, N, bits, group, codes, scales, zeros, workspa
 
 
 def tman_mpgemv(packed, x, y, M, K, N, bits, group, workspace, stream=None) -> None:
-    _check(lib().tman_mpgemv(_ptr(packed), packed.numel() * packed.element_size(), _ptr(x), _ptr(y), M, K, N, bits, group, _ptr(workspace),
-                             workspace.numel() * workspace.element_size(), _stream(stream)),
-           "tman_mpgemv")
+    st = _hot().mpgemv(packed, x, y, M, K, N, bits, group, workspace, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_mpgemv")
 
 
 def tman_mpgemv_static(packed, x, y, M, K, N, bits, group, status=None, stream=None) -> None:
@@ -156,20 +182,15 @@ def tman_mpgemv_static(packed, x, y, M, K, N, bits, group, status=None, stream=N
 
 def tman_mpgemv_grouped(packed_list, x, y_list, M, K, N_list, bits, group, workspace, stream=None) -> None:
     """Decode for several weight matrices that share the activations x, in one launch."""
-    n = len(packed_list)
-    pk = (C.c_void_p * n)(*[_ptr(t) for t in packed_list])
-    pb = (C.c_size_t * n)(*[t.numel() * t.element_size() for t in packed_list])
-    ys = (C.c_void_p * n)(*[_ptr(t) for t in y_list])
-    ns = (C.c_int * n)(*[int(v) for v in N_list])
-    _check(lib().tman_mpgemv_grouped(n, pk, pb, _ptr(x), ys, M, K, ns, bits, group, _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _stream(stream)),
-           "tman_mpgemv_grouped")
+    st = _hot().mpgemv_grouped(packed_list, x, y_list, M, K, N_list, bits, group, workspace, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_mpgemv_grouped")
 
 
 def tman_mpgemm(packed, x, y, M, K, N, bits, group, workspace, stream=None) -> None:
-    _check(lib().tman_mpgemm(_ptr(packed), packed.numel() * packed.element_size(), _ptr(x), _ptr(y), M, K, N, bits, group, _ptr(workspace),
-                             workspace.numel() * workspace.element_size(), _stream(stream)),
-           "tman_mpgemm")
+    st = _hot().mpgemm(packed, x, y, M, K, N, bits, group, workspace, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_mpgemm")
 
 
 def tman_debug_indices(packed, K, N, bits, group, idx, workspace, stream=None) -> None:
@@ -205,23 +226,27 @@ def tman_dequant_ternary_int8(packed, K, N, group, w8, ws, stream=None) -> None:
 
 
 def tman_quantize_rows_i8(x, M, K, a, row_scale, stream=None) -> None:
-    _check(lib().tman_quantize_rows_i8(_ptr(x), M, K, _ptr(a), _ptr(row_scale), _stream(stream)), "tman_quantize_rows_i8")
+    st = _hot().quantize_rows_i8(x, M, K, a, row_scale, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_quantize_rows_i8")
 
 
 def tman_mpgemm_ternary_i8(packed, a, row_scale, w_scale, y, M, K, N, group, ws, stream=None) -> None:
-    _check(lib().tman_mpgemm_ternary_i8(_ptr(packed), packed.numel() * packed.element_size(), _ptr(a), _ptr(row_scale),
-                                        float(w_scale), _ptr(y), M, K, N, group, _ptr(ws), ws.numel() * ws.element_size(),
-                                        _stream(stream)), "tman_mpgemm_ternary_i8")
+    st = _hot().mpgemm_ternary_i8(packed, a, row_scale, w_scale, y, M, K, N, group, ws, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_mpgemm_ternary_i8")
 
 
 def tman_quantize_rows(x, M, K, qmax, a, row_scale, stream=None) -> None:
-    _check(lib().tman_quantize_rows(_ptr(x), M, K, qmax, _ptr(a), _ptr(row_scale), _stream(stream)), "tman_quantize_rows")
+    st = _hot().quantize_rows(x, M, K, qmax, a, row_scale, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_quantize_rows")
 
 
 def tman_mpgemv_ternary(packed, a, row_scale, w_scale, y, acc, M, K, N, group, ws, stream=None) -> None:
-    _check(lib().tman_mpgemv_ternary(_ptr(packed), packed.numel() * packed.element_size(), _ptr(a), _ptr(row_scale),
-                                     float(w_scale), _ptr(y), _ptr(acc), M, K, N, group, _ptr(ws),
-                                     ws.numel() * ws.element_size(), _stream(stream)), "tman_mpgemv_ternary")
+    st = _hot().mpgemv_ternary(packed, a, row_scale, w_scale, y, acc, M, K, N, group, ws, _stream(stream))
+    if st:
+        raise TmanError(st, "tman_mpgemv_ternary")
 
 
 GEMM_VARIANTS = {"product": 0, "convert_dq": 1, "load_full": 2, "sequential": 3}

@@ -1,15 +1,18 @@
-"""Build step: compile the CUDA sources into libtman.so next to this file (sm_100a only)."""
+"""Build step: compile the CUDA sources into libtman.so (sm_100a only) and the argument marshalling of the Python
+binding into _marshal, both next to this file."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtman.so")
 LIB_STAMPS = os.path.join(HERE, "libtman_stamps.so")   # the same library with role time stamps in the prefill kernel
+MARSHAL = os.path.join(HERE, "_marshal" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 SOURCES = ["api.cu", "pack.cu", "mpgemv.cu", "mpgemv_static.cu", "mpgemm.cu", "mpgemm_i8.cu", "microbench.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -25,8 +28,23 @@ def _stale(lib: str = LIB) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_marshal(force: bool = False) -> str:
+    """The CPython extension that binding.py calls the hot entry points through."""
+    src = os.path.join(CSRC, "marshal.cpp")
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= os.path.getmtime(src):
+        return MARSHAL
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"],
+           "-I", os.path.join(ROOT, "include"), src, "-o", MARSHAL]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("building the argument marshalling failed")
+    return MARSHAL
+
+
 def build(force: bool = False, verbose: bool = False, stamps: bool = False) -> str:
     """stamps: build libtman_stamps.so (-DTMAN_ROLE_STAMPS) instead of libtman.so."""
+    build_marshal(force)
     lib = LIB_STAMPS if stamps else LIB
     if not force and not _stale(lib):
         return lib

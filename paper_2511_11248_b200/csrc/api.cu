@@ -11,6 +11,28 @@ static bool aligned_to(const void *p, uintptr_t a) { return (reinterpret_cast<ui
 static bool buffers_aligned(const void *packed, const void *workspace) { return aligned_to(packed, 256) && aligned_to(workspace, 256); }
 static bool matrices_aligned(const void *x, const void *y) { return aligned_to(x, 16) && aligned_to(y, 16); }
 
+namespace tman {
+
+DeviceInfo *device_info(int *dev_out)
+{
+    static DeviceInfo info[kMaxDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    if (dev_out) *dev_out = dev;
+    DeviceInfo &d = info[dev];
+    if (d.sms.load(std::memory_order_acquire) == 0) {
+        int sms = 0, reserved = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0 ||
+            cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess)
+            return nullptr;
+        d.reserved_smem.store(reserved, std::memory_order_relaxed);
+        d.sms.store(sms, std::memory_order_release);
+    }
+    return &d;
+}
+
+}  // namespace tman
+
 extern "C" {
 
 const char *tman_status_string(int status)

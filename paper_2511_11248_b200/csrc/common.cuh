@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <atomic>
 
 #include "tman.h"
 
@@ -78,13 +79,36 @@ inline tman_status launch_status()
     return cudaGetLastError() == cudaSuccess ? TMAN_OK : TMAN_ERR_CUDA;
 }
 
-// number of SMs of the current device (queried per call; cheap attribute read)
+// Properties of the current device that launches are planned from.  They never change, so they are asked once per
+// device (two attribute queries a call otherwise).
+constexpr int kMaxDevices = 64;
+struct DeviceInfo {
+    std::atomic<int> sms;             // 0: not asked yet
+    std::atomic<int> reserved_smem;   // shared memory the system keeps per CTA (valid once sms is set)
+};
+DeviceInfo *device_info(int *dev = nullptr);      // nullptr: the query failed
+
 inline int sm_count()
 {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    return n;
+    const DeviceInfo *d = device_info();
+    return d ? d->sms.load(std::memory_order_acquire) : 0;
+}
+
+// Launches `launch()` (cudaSuccess or an error) of a kernel that needs `bytes` of dynamic shared memory.  The kernel's
+// limit is raised once per device, `raised[device]` remembers it; a launch that fails all the same (the context may have
+// been reset in between) raises the limit again and tries once more.
+template <typename Kernel, typename Launch>
+inline tman_status launch_with_smem(Kernel kern, int bytes, int dev, std::atomic<bool> *raised, const Launch &launch)
+{
+    if (raised[dev].load(std::memory_order_relaxed)) {
+        if (launch() == cudaSuccess) return TMAN_OK;
+        (void)cudaGetLastError();
+        raised[dev].store(false, std::memory_order_relaxed);
+    }
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return TMAN_ERR_CUDA;
+    if (launch() != cudaSuccess) return TMAN_ERR_CUDA;
+    raised[dev].store(true, std::memory_order_relaxed);
+    return TMAN_OK;
 }
 
 // ---- table building block (device) -------------------------------------------------------

@@ -944,8 +944,9 @@ tman_status launch_cfg(const CUtensorMap &tmap_x, const CUtensorMap &tmap_w, con
 {
     using C = Cfg<MH, PAIR>;
     auto kern = mpgemm_kernel<BITS, MH, PAIR, V>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem_bytes(BITS)) != cudaSuccess)
-        return TMAN_ERR_CUDA;
+    static std::atomic<bool> raised[kMaxDevices];
+    int dev = 0;
+    if (!device_info(&dev)) return TMAN_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(workers * C::NCTA));
     cfg.blockDim = dim3(GEMM_THREADS);
@@ -958,8 +959,8 @@ tman_status launch_cfg(const CUtensorMap &tmap_x, const CUtensorMap &tmap_w, con
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kern, tmap_x, tmap_w, tmap_y, tmap_wf, p) != cudaSuccess) return TMAN_ERR_CUDA;
-    return TMAN_OK;
+    return launch_with_smem(kern, C::smem_bytes(BITS), dev, raised,
+                            [&] { return cudaLaunchKernelEx(&cfg, kern, tmap_x, tmap_w, tmap_y, tmap_wf, p); });
 }
 
 template <int BITS, int V>
@@ -997,11 +998,10 @@ int resident_cfg(int sms)
 
 int resident_workers(int M, int bits, int sms)
 {
-    constexpr int kMaxDevices = 64;
     static std::mutex lock;
     static int cache[kMaxDevices][3][3];     // [device][bits - 2][variant], 0 = not asked yet
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || bits < 2 || bits > 4) return -1;
+    if (!device_info(&dev) || bits < 2 || bits > 4) return -1;
     const int variant = !gemm_pair(M) ? 0 : (gemm_mh(M) == 1 ? 1 : 2);
     std::lock_guard<std::mutex> guard(lock);
     int &slot = cache[dev][bits - 2][variant];

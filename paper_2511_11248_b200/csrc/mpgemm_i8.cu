@@ -255,10 +255,16 @@ tman_status launch_i8(const CUtensorMap &tmap_a, const CUtensorMap &tmap_w, Gemm
     p.tiles_n = (p.N + BN - 1) / BN;
     const int tiles = p.tiles_m * p.tiles_n;
     auto kern = mpgemm_i8_kernel<BN>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess) return TMAN_ERR_CUDA;
     const int grid = tiles < sms ? tiles : sms;
-    kern<<<(unsigned)grid, C::THREADS, C::SMEM_BYTES, s>>>(tmap_a, tmap_w, p);
-    return launch_status();
+    static std::atomic<bool> raised[kMaxDevices];
+    int dev = 0;
+    if (!device_info(&dev)) return TMAN_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(C::THREADS);
+    cfg.dynamicSmemBytes = C::SMEM_BYTES;
+    cfg.stream = s;
+    return launch_with_smem(kern, C::SMEM_BYTES, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, tmap_a, tmap_w, p); });
 }
 }  // namespace
 

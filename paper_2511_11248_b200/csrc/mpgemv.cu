@@ -35,8 +35,6 @@
 // kernels of the caller's own.
 #include "common.cuh"
 
-#include <atomic>
-
 namespace tman {
 
 constexpr int kGemvThreads = 512;
@@ -783,24 +781,21 @@ static tman_status launch_one(GemvParams p, int sms, cudaStream_t s)
     if (p.P > p.units) p.P = p.units;
     // every CTA must be resident while it polls for the others' partial sums
     if ((long long)p.nkappa * p.P > (long long)sms) return TMAN_ERR_UNSUPPORTED;
-    int dev = 0, reserved = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess)
-        return TMAN_ERR_CUDA;
-    if ((uint32_t)reserved != kGemvSmemBase) return TMAN_ERR_UNSUPPORTED;
+    int dev = 0;
+    const DeviceInfo *info = device_info(&dev);
+    if (!info) return TMAN_ERR_CUDA;
+    if ((uint32_t)info->reserved_smem.load(std::memory_order_relaxed) != kGemvSmemBase) return TMAN_ERR_UNSUPPORTED;
     auto kern = mpgemv_kernel<BITS, MT, S, PRE, HALF, GROUPED, ROLL, HR, INT>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
-        return TMAN_ERR_CUDA;
+    static std::atomic<bool> raised[kMaxDevices];
     // the grid has at most one CTA per SM; the occupancy query says whether an SM can hold one at all
     // (asked once per device and variant)
     {
-        constexpr int kMaxDevices = 64;
         static std::atomic<int> fits[kMaxDevices];          // 0 = not asked, 1 = fits, -1 = does not
-        if (dev < 0 || dev >= kMaxDevices) return TMAN_ERR_CUDA;
         int f = fits[dev].load(std::memory_order_relaxed);
         if (f == 0) {
             int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGemvThreads, kSmem) != cudaSuccess)
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGemvThreads, kSmem) != cudaSuccess)
                 return TMAN_ERR_CUDA;
             f = per_sm >= 1 ? 1 : -1;
             fits[dev].store(f, std::memory_order_relaxed);
@@ -819,8 +814,7 @@ static tman_status launch_one(GemvParams p, int sms, cudaStream_t s)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = packed_write_pending(s, /*clear=*/true) ? 0 : 1;
-    if (cudaLaunchKernelEx(&cfg, kern, p) != cudaSuccess) return TMAN_ERR_CUDA;
-    return TMAN_OK;
+    return launch_with_smem(kern, kSmem, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, p); });
 }
 
 template <int BITS, int MT, int PRE, int HR>

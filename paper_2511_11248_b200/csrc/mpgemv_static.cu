@@ -17,7 +17,6 @@ namespace tman {
 namespace {
 
 constexpr size_t kStaticWsBytes = 4u << 20;          // 4 MiB per GPU
-constexpr int    kMaxDevices = 64;
 
 // The scratch itself.  In host code this name is only a handle for cudaGetSymbolAddress: it is
 // not a device address and must never be passed to a kernel.

@@ -2,6 +2,8 @@
 // clusters, TMA copies, tensor memory and tcgen05 MMA / commit / load, shared-memory descriptors.
 #pragma once
 
+#include <atomic>
+
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -224,12 +226,16 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                   CUtensorMapFloatOOBfill);
 
+// (the driver's address does not change: asked once)
 inline EncodeTiledFn encode_fn()
 {
-    void *fn = nullptr;
+    static std::atomic<void *> known;
+    void *fn = known.load(std::memory_order_relaxed);
+    if (fn) return reinterpret_cast<EncodeTiledFn>(fn);
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess) return nullptr;
     if (q != cudaDriverEntryPointSuccess) return nullptr;
+    known.store(fn, std::memory_order_relaxed);
     return reinterpret_cast<EncodeTiledFn>(fn);
 }
 

@@ -195,3 +195,33 @@ def test_decode_plan_choices_and_limits(lib):
     costs = [B.tman_debug_gemv_plan(M, K, N, bits, G)["cost_us"] for M in range(1, 9)]
     assert all(a <= b + 1e-9 for a, b in zip(costs, costs[1:]))
     assert B.tman_debug_gemv_plan(4, K, N, 2, G)["cost_us"] < B.tman_debug_gemv_plan(4, K, N, 4, G)["cost_us"]
+
+
+def test_marshalled_calls_report_status_and_bad_arguments(lib):
+    """The hot entry points go through the _marshal extension: statuses come back as TmanError, sizes and addresses are
+    read from the tensors, and arguments of the wrong kind raise instead of reaching the library."""
+    torch = pytest.importorskip("torch")
+    from paper_2511_11248_b200 import binding as B
+    fast = B._hot()
+    whole = torch.zeros((1 << 16) + 256, dtype=torch.uint8)
+    t = whole[(-whole.data_ptr()) % 256:][:1 << 16]       # host memory: every call below is refused before it is read
+    assert fast.mpgemv(t, t, t, 9, 128, 8, 4, 64, t, 0) == 2
+    assert fast.mpgemv(t[:300], t, t, 1, 128, 8, 4, 64, t, 0) == 4
+    assert fast.mpgemv(t, t, t[8:], 1, 128, 8, 4, 64, t, 0) == 2
+    assert fast.mpgemv(t, None, t, 1, 128, 8, 4, 64, t, 0) == 1
+    assert fast.mpgemm(t, t, t, 0, 128, 8, 4, 64, t, 0) == 2
+    assert fast.mpgemv_grouped([t] * 5, t, [t] * 5, 1, 128, [8] * 5, 4, 64, t, 0) == 2
+    assert fast.mpgemv_grouped([t, t], t, [t, t], 1, 128, [8, 12], 4, 64, t, 0) == 2
+    assert fast.quantize_rows(t, 1, 128, 5, t, t, 0) == 2
+    assert fast.quantize_rows_i8(t, 0, 128, t, t, 0) == 2
+    assert fast.mpgemv_ternary(t, t, t, 1.0, t, None, 9, 128, 8, 64, t, 0) == 2
+    assert fast.mpgemm_ternary_i8(t, t, None, 1.0, t, 1, 128, 8, 64, t, 0) == 1
+    assert fast.pack_weights(t, t, t, 128, 8, 4, 64, t[:16], 0) == 4
+    with pytest.raises(TypeError):
+        fast.mpgemv(t, t, t, 1, 128, 8, 4, 64, t)         # an argument short
+    with pytest.raises(TypeError):
+        fast.mpgemv(t, t, t, 1.5, 128, 8, 4, 64, t, 0)
+    with pytest.raises(AttributeError):
+        fast.mpgemv(t, 3, t, 1, 128, 8, 4, 64, t, 0)
+    with pytest.raises(IndexError):
+        fast.mpgemv_grouped([t, t], t, [t], 1, 128, [8, 8], 4, 64, t, 0)
