@@ -23,6 +23,25 @@ def test_pack_is_bit_exact(K, N, bits, G):
     assert np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("K,N,bits,G", [(128, 128, 1, 32), (256, 136, 2, 64), (1152, 264, 3, 128), (640, 120, 4, 32)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_pack_tile_edges_and_misaligned_inputs(K, N, bits, G, shift):
+    # whole and ragged tiles of 32 strips x 8 words, and inputs that do not start on 4 (codes, zero-points) or 8 bytes
+    # (scales): read element by element
+    c = synth.small_case(1, K, N, bits, G, seed=7 * K + N + bits)
+    def moved(a, by):
+        flat = torch.from_numpy(np.ascontiguousarray(a).view(np.uint8).reshape(-1))
+        buf = torch.zeros(flat.numel() + 16, dtype=torch.uint8, device="cuda")
+        buf[by:by + flat.numel()] = flat.cuda()
+        return buf[by:by + flat.numel()]
+    packed = H.alloc_packed(K, N, bits, G)
+    packed.fill_(0xA5)                                     # padding must be written too
+    B.tman_pack_weights(moved(c.codes, shift), moved(c.scales, 2 * shift), moved(c.zeros, shift), K, N, bits, G, packed)
+    torch.cuda.synchronize()
+    H.check_guards()
+    assert np.array_equal(packed.cpu().numpy(), orc.pack(c.codes, c.scales, c.zeros, bits, G))
+
+
 @pytest.mark.parametrize("K,N,bits,G", SHAPES)
 def test_unpack_roundtrip_and_indices(K, N, bits, G):
     c = synth.small_case(1, K, N, bits, G, seed=3 * K + N + bits)
