@@ -62,6 +62,8 @@ mpgemm_i8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
     constexpr int I8_DEQ_WARPS = C::DEQ_WARPS, I8_TMEM_COLS = 2 * I8_BN;     // two accumulator sets: the epilogue of a tile
                                                                              // overlaps the multiplications of the next
     extern __shared__ __align__(1024) uint8_t smem[];
+    // Launched so that it may start while the row quantization before it drains; nothing is read or written before this.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!header_matches(p.packed, p.K, p.N, 2, p.group)) {          // same answer in every CTA
         if (threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)TMAN_ERR_BAD_PACKED);
         return;
@@ -264,6 +266,11 @@ tman_status launch_i8(const CUtensorMap &tmap_a, const CUtensorMap &tmap_w, Gemm
     cfg.blockDim = dim3(C::THREADS);
     cfg.dynamicSmemBytes = C::SMEM_BYTES;
     cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     return launch_with_smem(kern, C::SMEM_BYTES, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, tmap_a, tmap_w, p); });
 }
 }  // namespace

@@ -1016,24 +1016,98 @@ tman_status launch_mpgemv_grouped(int count, const void *const *packed, const vo
 // Per-row symmetric quantization of the activations (paper Sec. 6.1, A_INT16; 8 bits for the matrix unit):
 // s_a = max|x| / qmax and a = round(x / s_a), both in single precision with correctly rounded division and
 // rounding to nearest even, so that the integers are the same on any IEEE machine.  One CTA per row.
-template <typename OUT>      // int16_t or int8_t
+//
+// quantize_rows_regs_kernel: the row (K % 8 == 0, 16-byte aligned rows) is read once and kept in registers, VPT vectors of
+// eight values a thread; one barrier; the quotient is the row's reciprocal times x, corrected to the correctly rounded
+// quotient with two remainder steps (Markstein, "Computation of elementary functions on the IBM RISC System/6000
+// processor", IBM J. Res. Dev. 34, 1990, division by a correctly rounded reciprocal: q' = q + (x - q s) y, the remainder
+// exact by fused multiply-add; the first step brings q, off by at most 1.5 units in the last place, to a neighbour of the
+// quotient, the second rounds it).  No intermediate leaves the normal range: 2^-24 <= |x| < 2^16 and 2^-40 < s < 2^10.
+// Launched so that it may start while its predecessor drains, and lets its successor do the same.
+// Against two passes with a full division per value in one CTA of 512 threads a row: 2048 rows of 2560 and the INT8
+// product with 6912 channels after them 61.3 -> 50.2 us; one row and its decode, mean of 2560 x 6912 and 6912 x 2560,
+// 7.6 -> 6.1 us.
+template <typename OUT>
+__device__ __forceinline__ void store_eight(OUT *out, const int (&q)[8])
+{
+    if constexpr (sizeof(OUT) == 2)
+        *reinterpret_cast<uint4 *>(out) =
+            make_uint4(__byte_perm((uint32_t)q[0], (uint32_t)q[1], 0x5410), __byte_perm((uint32_t)q[2], (uint32_t)q[3], 0x5410),
+                       __byte_perm((uint32_t)q[4], (uint32_t)q[5], 0x5410), __byte_perm((uint32_t)q[6], (uint32_t)q[7], 0x5410));
+    else {
+        const uint32_t a = __byte_perm((uint32_t)q[0], (uint32_t)q[1], 0x0040), b = __byte_perm((uint32_t)q[2], (uint32_t)q[3], 0x0040);
+        const uint32_t c = __byte_perm((uint32_t)q[4], (uint32_t)q[5], 0x0040), d = __byte_perm((uint32_t)q[6], (uint32_t)q[7], 0x0040);
+        *reinterpret_cast<uint2 *>(out) = make_uint2(__byte_perm(a, b, 0x5410), __byte_perm(c, d, 0x5410));
+    }
+}
+
+template <typename OUT, int VPT>      // int16_t or int8_t
+__global__ void __launch_bounds__(1024) quantize_rows_regs_kernel(const __half *__restrict__ x, int nvec, int qmax,
+                                                                  OUT *__restrict__ a, float *__restrict__ s_a)
+{
+    __shared__ float red[32];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint4 *row = reinterpret_cast<const uint4 *>(x) + (size_t)blockIdx.x * nvec;
+    OUT *out = a + (size_t)blockIdx.x * nvec * 8;
+    uint4 v[VPT];
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const int at = threadIdx.x + i * blockDim.x;
+        v[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (at < nvec) v[i] = __ldg(row + at);
+    }
+    __half2 mx = __floats2half2_rn(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const __half2 *h = reinterpret_cast<const __half2 *>(&v[i]);
+        mx = __hmax2(mx, __hmax2(__hmax2(__habs2(h[0]), __habs2(h[1])), __hmax2(__habs2(h[2]), __habs2(h[3]))));
+    }
+    float amax = fmaxf(__low2float(mx), __high2float(mx));
+    for (int mask = 16; mask > 0; mask >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, mask));
+    const int warps = blockDim.x >> 5;
+    if (warps > 1) {
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = amax;
+        __syncthreads();
+        amax = (int)(threadIdx.x & 31) < warps ? red[threadIdx.x & 31] : 0.f;
+        for (int mask = 16; mask > 0; mask >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, mask));
+    }
+    const float scale = amax > 0.f ? __fdiv_rn(amax, (float)qmax) : 1.f;
+    const float inv = __frcp_rn(scale);
+    if (threadIdx.x == 0) s_a[blockIdx.x] = scale;
+    auto quant = [&](float f) {
+        float q = f * inv;
+        q = fmaf(fmaf(-q, scale, f), inv, q);
+        q = fmaf(fmaf(-q, scale, f), inv, q);
+        return (int)max(-qmax, min(qmax, __float2int_rn(q)));
+    };
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        const int at = threadIdx.x + i * blockDim.x;
+        if (at < nvec) {
+            const __half2 *h = reinterpret_cast<const __half2 *>(&v[i]);
+            int q[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float2 f = __half22float2(h[e]);
+                q[2 * e] = quant(f.x);
+                q[2 * e + 1] = quant(f.y);
+            }
+            store_eight<OUT>(out + (size_t)at * 8, q);
+        }
+    }
+}
+
+// Any K and rows longer than the registers of a CTA hold: two passes over the row, element by element.
+template <typename OUT>
 __global__ void __launch_bounds__(1024) quantize_rows_kernel(const __half *__restrict__ x, int K, int qmax,
                                                              OUT *__restrict__ a, float *__restrict__ s_a)
 {
     __shared__ float red[32];
     const __half *row = x + (size_t)blockIdx.x * K;
     OUT *out = a + (size_t)blockIdx.x * K;
-    // eight values per thread and step when the row allows 16-byte accesses (K % 8 == 0, checked by the host)
-    const bool vec = (K & 7) == 0;
-    const int nvec = vec ? K >> 3 : 0;
     float amax = 0.f;
-    for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(row) + i);
-        const __half2 *h = reinterpret_cast<const __half2 *>(&q);
-        __half2 m = __hmax2(__hmax2(__habs2(h[0]), __habs2(h[1])), __hmax2(__habs2(h[2]), __habs2(h[3])));
-        amax = fmaxf(amax, fmaxf(__low2float(m), __high2float(m)));
-    }
-    for (int k = 8 * nvec + threadIdx.x; k < K; k += blockDim.x) amax = fmaxf(amax, fabsf(__half2float(row[k])));
+    for (int k = threadIdx.x; k < K; k += blockDim.x) amax = fmaxf(amax, fabsf(__half2float(row[k])));
     for (int mask = 16; mask > 0; mask >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, mask));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = amax;
     __syncthreads();
@@ -1046,44 +1120,48 @@ __global__ void __launch_bounds__(1024) quantize_rows_kernel(const __half *__res
     amax = red[0];
     const float scale = amax > 0.f ? __fdiv_rn(amax, (float)qmax) : 1.f;
     if (threadIdx.x == 0) s_a[blockIdx.x] = scale;
-    auto quant = [&](__half v) {
-        const int r = __float2int_rn(__fdiv_rn(__half2float(v), scale));
-        return (int)max(-qmax, min(qmax, r));
-    };
-    for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(row) + i);        // second read: from L1/L2
-        const __half *h = reinterpret_cast<const __half *>(&q);
-        if constexpr (sizeof(OUT) == 2) {
-            uint4 o;
-            o.x = (uint32_t)(quant(h[0]) & 0xFFFF) | ((uint32_t)quant(h[1]) << 16);
-            o.y = (uint32_t)(quant(h[2]) & 0xFFFF) | ((uint32_t)quant(h[3]) << 16);
-            o.z = (uint32_t)(quant(h[4]) & 0xFFFF) | ((uint32_t)quant(h[5]) << 16);
-            o.w = (uint32_t)(quant(h[6]) & 0xFFFF) | ((uint32_t)quant(h[7]) << 16);
-            reinterpret_cast<uint4 *>(out)[i] = o;
-        } else {
-            uint2 o;
-            o.x = (uint32_t)(quant(h[0]) & 0xFF) | ((uint32_t)(quant(h[1]) & 0xFF) << 8) |
-                  ((uint32_t)(quant(h[2]) & 0xFF) << 16) | ((uint32_t)quant(h[3]) << 24);
-            o.y = (uint32_t)(quant(h[4]) & 0xFF) | ((uint32_t)(quant(h[5]) & 0xFF) << 8) |
-                  ((uint32_t)(quant(h[6]) & 0xFF) << 16) | ((uint32_t)quant(h[7]) << 24);
-            reinterpret_cast<uint2 *>(out)[i] = o;
-        }
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        const int r = __float2int_rn(__fdiv_rn(__half2float(row[k]), scale));
+        out[k] = (OUT)max(-qmax, min(qmax, r));
     }
-    for (int k = 8 * nvec + threadIdx.x; k < K; k += blockDim.x) out[k] = (OUT)quant(row[k]);
+}
+
+template <typename OUT>
+static tman_status launch_quantize(const void *x, int M, int K, int qmax, OUT *a, float *s_a, cudaStream_t s)
+{
+    const __half *xh = static_cast<const __half *>(x);
+    const int nvec = K / 8;
+    // Few rows: the latency of one row counts, every vector its own thread.  Many rows: four vectors a thread, so that a
+    // row's reduction is spread over fewer threads (2048 rows of 2560: 96 threads; the limit of 1024 threads holds 8 x 4
+    // values each, longer rows go element by element).
+    const bool few = M <= 2 * kGemvPlanSms && nvec <= 1024;
+    const int vpt = few ? 1 : 4;
+    if (K % 8 != 0 || nvec > 1024 * 4) {
+        const int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
+        quantize_rows_kernel<OUT><<<(unsigned)M, threads, 0, s>>>(xh, K, qmax, a, s_a);
+        return launch_status();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)M);
+    cfg.blockDim = dim3((unsigned)(((nvec + vpt - 1) / vpt + 31) / 32 * 32));
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto kern = few ? quantize_rows_regs_kernel<OUT, 1> : quantize_rows_regs_kernel<OUT, 4>;
+    return cudaLaunchKernelEx(&cfg, kern, xh, nvec, qmax, a, s_a) == cudaSuccess ? TMAN_OK : TMAN_ERR_CUDA;
 }
 
 tman_status launch_quantize_rows(const void *x, int M, int K, int qmax, int16_t *a, float *s_a, cudaStream_t s)
 {
-    const int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
-    quantize_rows_kernel<int16_t><<<(unsigned)M, threads, 0, s>>>(static_cast<const __half *>(x), K, qmax, a, s_a);
-    return launch_status();
+    return launch_quantize<int16_t>(x, M, K, qmax, a, s_a, s);
 }
 
 tman_status launch_quantize_rows_i8(const void *x, int M, int K, int8_t *a, float *s_a, cudaStream_t s)
 {
-    const int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
-    quantize_rows_kernel<int8_t><<<(unsigned)M, threads, 0, s>>>(static_cast<const __half *>(x), K, 127, a, s_a);
-    return launch_status();
+    return launch_quantize<int8_t>(x, M, K, 127, a, s_a, s);
 }
 
 // Rows of 16-bit integer activations times ternary weights packed as 2-bit codes (zero-point 1; the

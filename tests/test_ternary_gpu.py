@@ -44,6 +44,46 @@ def test_row_quantization_is_bit_exact(M, K, qmax, spread):
     assert np.array_equal(s.cpu().numpy().astype(np.float64), want_s)
 
 
+@pytest.mark.parametrize("qmax", [32767, 127])
+@pytest.mark.parametrize("M,K", [(1, 8), (300, 8192 + 8), (300, 2560), (2, 8192), (1, 32768), (1, 32776), (300, 1000)])
+def test_row_quantization_at_the_edges_of_its_variants(M, K, qmax):
+    # one and four vectors a thread, whole and ragged last vectors, rows beyond the registers; every row has another
+    # magnitude, so that quotients fall on all kinds of ties and neighbours of ties: the integers have to be exact
+    rng = np.random.default_rng(K + qmax)
+    x = (rng.standard_normal((M, K)) * 2.0 ** rng.uniform(-16, 11, size=(M, 1))).astype(np.float16)
+    x[M // 2, ::3] = np.float16(6e-8)                         # the smallest subnormal beside ordinary values
+    want_a, want_s = oi.quantize_rows(x, qmax)
+    xd = torch.from_numpy(x.view(np.int16)).cuda().view(torch.float16)
+    wide = qmax > 127
+    a = H.guarded_bytes(M * K * (2 if wide else 1), "a").view(torch.int16 if wide else torch.int8).view(M, K)
+    s = H.guarded_bytes((M * 4 + 255) // 256 * 256, "row_scale").view(torch.float32)
+    if wide:
+        B.tman_quantize_rows(xd, M, K, qmax, a, s)
+    else:
+        B.tman_quantize_rows_i8(xd, M, K, a, s)
+    torch.cuda.synchronize()
+    H.check_guards()
+    assert np.array_equal(a.cpu().numpy().astype(np.int32), want_a)
+    assert np.array_equal(s[:M].cpu().numpy().astype(np.float64), want_s)
+
+
+@pytest.mark.parametrize("qmax", [32767, 127])
+def test_row_quantization_of_every_fp16_value(qmax):
+    # all finite values up to a row's largest magnitude, for several magnitudes: the quotient is the correctly rounded one
+    for top in (65504.0, 1000.0, 3.1415, 1.0, 0.07, 6e-5, 3e-7):
+        v = np.arange(1 << 16, dtype=np.uint16).view(np.float16)
+        v = v[np.isfinite(v) & (np.abs(v) <= np.float16(top))]
+        x = np.resize(v, ((v.size + 4095) // 4096, 4096))
+        x[:, 0] = np.float16(top)
+        want_a, want_s = oi.quantize_rows(x, qmax)
+        xd = torch.from_numpy(x.view(np.int16)).cuda().view(torch.float16)
+        a = torch.empty(x.shape, dtype=torch.int16, device="cuda")
+        s = torch.empty(x.shape[0], dtype=torch.float32, device="cuda")
+        B.tman_quantize_rows(xd, x.shape[0], 4096, qmax, a, s)
+        assert np.array_equal(a.cpu().numpy().astype(np.int32), want_a), top
+        assert np.array_equal(s.cpu().numpy().astype(np.float64), want_s)
+
+
 # the paper's BitNet kernel sizes {2560, 6912} x {2560, 6912}, ragged column counts, one-slice K, both pairings
 SHAPES = [(128, 8, 128), (512, 40, 32), (2560, 2560, 128), (2560, 6912, 64), (6912, 2560, 128), (6912, 6912, 128),
           (1152, 264, 64), (16384, 72, 128)]
