@@ -121,8 +121,9 @@ tman_status tman_unpack_weights(const void *packed, size_t packed_bytes,
 /* Decode (paper Sec. 2.2 "Bit-serial table lookup", Fig. 2; Sec. 4.3): activation tables are
  * built in shared memory, packed bit-plane bytes index them, partial sums are
  * shift-accumulated per quantization block, scaled, and summed across blocks in fp32.
- * M in [1, 8], normally in one pass over the weights.  Precision: one row -- fp32 table entries and
- * sums.  Two to eight rows -- each row of a K-slice is scaled by a power of two into [1, 2) (exactly
+ * M in [1, 8], normally in one pass over the weights.  Five rows and more (three and more for 3- and 4-bit weights in groups of
+ * 64 or 128) are multiplied on the tensor cores instead: codes and activations exact in fp16, sums in fp32.  Precision: one row --
+ * fp32 table entries and sums; on the tensor cores as for one row.  Two to four rows by lookup -- each row of a K-slice is scaled by a power of two into [1, 2) (exactly
  * undone at the end), table entries are rounded to fp16 and the bits x 4 lookups of a 32-activation word
  * are added in fp16, everything after in fp32 (the paper's 16-bit table entries and low-precision
  * aggregation inside a block, Sec. 4.3, Sec. 5): error at most about 1.5e-3 of the largest output,
@@ -298,7 +299,8 @@ tman_status tman_debug_gemm_plan_for(int M, int K, int N, int bits, int group, i
  * of the lookup kernel is searched under the hardware's limits; here the searched space is the kernel
  * variants the library carries).  Host arithmetic only, nothing is launched, needs no GPU.  A variant
  * carries 1, 2, 4 or 8 activation rows per pass over the weights (table entries of one fp32 row or of
- * 1, 2 or 4 fp16 row pairs) in K-slices of 16, 32, 16 or 8 plane words.  A variant is admitted when its
+ * 1 or 2 fp16 row pairs; from five rows, or three, the tensor cores) and is admitted for K-slices of 16, 32, 16 or 8 plane words
+ * (a pass on the tensor cores then takes fewer and longer ones).  A variant is admitted when its
  * K-slices can all be resident (`sms` multiprocessors), its tables fit an SM's shared memory and its
  * partial sums fit `ws_limit` bytes (0: no limit); among the admitted ones the passes with the least
  * modelled time (fixed cost per pass + per-megabyte cost of the bit planes, fitted to measurements) are

@@ -308,7 +308,7 @@ tman_status tman_debug_gemv_plan(int M, int K, int N, int bits, int group, int s
     if (st != TMAN_OK) return st;
     if (M < 1 || M > kGemvMaxRows || sms < 1) return TMAN_ERR_SHAPE;
     if (bits < 2) return TMAN_ERR_UNSUPPORTED;
-    const GemvPlan g = plan_gemv(M, K, N, bits, sms, ws_limit ? ws_limit : (size_t)-1);
+    const GemvPlan g = plan_gemv(M, K, N, bits, group, sms, ws_limit ? ws_limit : (size_t)-1);
     for (int i = 0; i < 4 + 6 * kGemvMaxRows; ++i) out[i] = 0;
     out[0] = g.npass;
     out[1] = (int)((g.ws_bytes + 1023) / 1024);

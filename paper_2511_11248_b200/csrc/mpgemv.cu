@@ -1,8 +1,11 @@
 // Decode path: bit-serial table-lookup mpGEMV (paper Sec. 2.2 "Bit-serial table lookup", Fig. 2;
 // Sec. 4.3 "Mapping of LUT-based Decoding").
 //
-// Work split.  The reduction dimension is cut into K-slices of 8 to 32 plane words (16 for one
-// activation row; 32, 16, 8 for 2, 3-4, 5-8 rows, whose table entries carry the rows as fp16 pairs).  One
+// One to four activation rows by table lookup, described here; more rows (and four where that is faster, uses_mma below) on
+// the tensor cores (decode_mma.cuh).
+//
+// Work split.  The reduction dimension is cut into K-slices of 16 or 32 plane words (16 for one
+// activation row; 32, 16 for 2, 3-4 rows, whose table entries carry the rows as fp16 pairs).  One
 // CTA owns one K-slice: it builds that slice's
 // activation tables in shared memory once and reuses them for every output column it visits
 // (the paper's "maximise reuse of cached lookup tables").  Inside a warp a lane owns ONE plane
@@ -23,17 +26,15 @@
 // "ready" flag, so no fence and no counter sits between the last lookup and the output; the poll
 // is bounded and reports TMAN_ERR_TIMEOUT.
 //
-// Streaming.  A warp works through units (a few strips of four columns).  With up to four activation
-// rows every strip's registers are refilled with the next unit's strip as soon as its lookups are done;
-// with more rows the next unit sits in a second set of registers.  Either way HBM reads overlap the
-// lookups.  The first
+// Streaming.  A warp works through units (a few strips of four columns).  Every strip's registers are
+// refilled with the next unit's strip as soon as its lookups are done, so HBM reads overlap the lookups.  The first
 // loads (header words, first unit) are issued before the kernel waits for the previous kernel in
 // the stream (programmatic dependent launch); the host has checked that every read derived from
 // (K, N, bits, group) is in bounds.  That is only sound while the previous kernel does not write the
 // packed buffer: the host launches the call that follows a tman_pack_weights on the same stream
 // in plain stream order instead (packed_write_pending below), and the header states the rule for
 // kernels of the caller's own.
-#include "common.cuh"
+#include "decode_mma.cuh"
 
 namespace tman {
 
@@ -41,14 +42,10 @@ constexpr int kGemvThreads = 512;
 constexpr int kGemvWarps = kGemvThreads / 32;
 constexpr int kGemvTableBytes = 128 * 1024;   // 4 groups x 256 entries x 32 slots x 4 B
 
-// "No sum pending": a NaN bit pattern that no floating-point operation returns.
-constexpr uint32_t kGemvSentinel = 0x7FA5A5A5u;
-constexpr uint32_t kGemvPollLimit = 1u << 21;  // polls of ~0.5 us each: about a second
 
 // Up to kGemvMaxGroup weight matrices that share the activations (same K, bits, group) go through
 // one launch: their output columns are concatenated, the tables are built once (paper Sec. 5:
 // one table precomputation shared by the projections that read the same input).
-constexpr int kGemvMaxGroup = 4;
 
 struct GemvParams {
     const uint8_t  *packed[kGemvMaxGroup];
@@ -123,38 +120,6 @@ __device__ __forceinline__ void load_rows(const uint8_t *p, float (&out)[MT])
     if constexpr (MT == 1) { out[0] = t; }
     else if constexpr (MT == 2) { out[0] = t.x; out[1] = t.y; }
     else { out[0] = t.x; out[1] = t.y; out[2] = t.z; out[3] = t.w; }
-}
-
-__device__ __forceinline__ float4 ld_volatile_f4(const float4 *p)
-{
-    float4 v;
-    asm volatile("ld.volatile.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ bool has_sentinel(const float4 &v)
-{
-    return __float_as_uint(v.x) == kGemvSentinel || __float_as_uint(v.y) == kGemvSentinel ||
-           __float_as_uint(v.z) == kGemvSentinel || __float_as_uint(v.w) == kGemvSentinel;
-}
-
-// Bounded wait of the split-K combine: polls up to four partial-sum quads (slices kp, kp + SP, ... below
-// nkappa) until none of them holds the "no sum pending" pattern, at most `limit` times.  Returns
-// whether they all arrived; the caller reports TMAN_ERR_TIMEOUT otherwise.
-__device__ __forceinline__ bool wait_for_sums(const float4 *src, size_t stride4, int kp, int SP, int nkappa,
-                                              uint32_t limit, float4 (&t)[4])
-{
-    bool ready = false;
-    for (uint32_t tries = 0; !ready && tries < limit; ++tries) {
-        ready = true;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (kp + q * SP < nkappa) t[q] = ld_volatile_f4(src + (size_t)(kp + q * SP) * stride4);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (kp + q * SP < nkappa) ready = ready && !has_sentinel(t[q]);
-    }
-    return ready;
 }
 
 // byte offset of table entry (group c of the lane's word, index p, slot) inside the table area
@@ -821,9 +786,9 @@ template <int BITS, int MT, int PRE, int HR>
 static tman_status launch_mt(GemvParams p, int sms, cudaStream_t s)
 {
     // one row: fp32 tables over half-warp slices, large units; more rows: fp16 row pairs, smaller units
-    // (measured: 2 strips per unit for up to four rows, 1 for eight).  All on one rolling set of registers.
+    // (measured: 2 strips per unit).  All on one rolling set of registers.
     constexpr int ROLL = 1;
-    constexpr int S = (HR && MT == 4) ? 1 : (HR && MT == 2) ? 2 : ((BITS == 2) ? 4 : 2);
+    constexpr int S = (HR && MT == 2) ? 2 : ((BITS == 2) ? 4 : 2);
     constexpr int HALF = HR ? 0 : 1;
     if (p.count > 1) return launch_one<BITS, MT, S, PRE, HALF, 1, ROLL, HR>(p, sms, s);
     return launch_one<BITS, MT, S, PRE, HALF, 0, ROLL, HR>(p, sms, s);
@@ -831,19 +796,24 @@ static tman_status launch_mt(GemvParams p, int sms, cudaStream_t s)
 
 // ---- the plan: which kernel variants serve a call (host arithmetic only) -------------------------
 // A variant carries up to `rows` activation rows per pass over the weights in K-slices of `words` plane
-// words; its table entries have `slots` 32-bit slots (one fp32 row, or two fp16 rows each).  The time of a
-// pass is modelled as fixed + per_mb x megabytes of bit planes; the constants were fitted to calls timed
-// in a CUDA graph on a B200 (K = 4096, N = 14336; 2- and 4-bit for one row, 4-bit for the others):
-//   rows 1: 6.9 / 9.7 us   rows 2: 10.7 us   rows 4: 14.9 us   rows 8: 23.6 us.
-// The slope grows with the rows because an entry of 2 / 4 / 8 fp16 rows takes 1 / 2 / 4 shared-memory
-// wavefronts per lookup.
+// words; its table entries have `slots` 32-bit slots (one fp32 row, or two fp16 rows each; 0: no tables, the tensor-core
+// kernel).  The time of a pass is modelled as fixed + per_mb x megabytes of bit planes; the constants were fitted to calls
+// timed in a CUDA graph on a B200 (4-bit, group 128, 4096 x 4096 and 4096 x 28672; one row also 2-bit 4096 x 14336).
 struct GemvVariant { int rows, words, slots, half_slices; double fixed_us, us_per_mb; };
 static const GemvVariant kGemvVariants[kGemvVariantCount] = {
     {1, 16, 1, 1, 4.10, 0.190},
     {2, 32, 1, 0, 4.35, 0.216},
-    {4, 16, 2, 0, 4.85, 0.341},
-    {8, 8, 4, 0, 5.85, 0.605},
+    {4, 16, 2, 0, 4.54, 0.272},
+    {8, 8, 0, 0, 4.60, 0.316},
 };
+
+// Whether a pass of `rows` rows goes to the tensor-core kernel (decode_mma.cuh) instead of the table lookups.  From five
+// rows always: an entry of eight fp16 rows costs four shared-memory wavefronts a lookup (4-bit 4096 x 28672, group 128:
+// 42.0 us by lookup, 23.1 us here; 2-bit, group 64: 29.8 / 22.4; 4-bit, group 32: 42.5 / 32.9).  With three and four rows
+// (two wavefronts) where a lookup per plane is many of them and the blocks are no shorter than two words: 4-bit, group 128
+// 23.8 / 20.5, 3-bit, group 64 20.2 / 20.0 (4096 x 4096: 7.4 / 6.8), but 2-bit, group 64 17.3 / 18.3 and 4-bit, group 32
+// 24.0 / 31.6.  One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.3 / 20.1).
+static bool uses_mma(int bits, int group, int rows) { return rows >= 5 || (rows >= 3 && bits >= 3 && group >= 64); }
 
 static size_t variant_ws_bytes(const GemvVariant &v, int K, int N)
 {
@@ -862,7 +832,30 @@ static bool variant_feasible(const GemvVariant &v, int K, int N, int sms, size_t
     return nkappa <= sms && smem <= kGemvSmemLimit && variant_ws_bytes(v, K, N) <= ws_limit;
 }
 
-GemvPlan plan_gemv(int M, int K, int N, int bits, int sms, size_t ws_limit)
+// How the tensor-core kernel cuts a pass: warps of a team (each one 128-deep chunk of k), teams per CTA, K-slices, CTAs per
+// K-slice.  16 warps of a team give the fewest partial sums; 8 and 4 are for short K or few columns, where more CTAs get work.
+struct MmaSplit { int tk, tc, nkappa, ctas; };
+static MmaSplit split_mma(int M, int K, int N, int groups, int sms, size_t ws_limit)
+{
+    const int chunks = K / 128;
+    MmaSplit best = {0, 0, 0, 0};
+    double best_us = 1e300;
+    for (int tk = 16; tk >= 4; tk >>= 1) {
+        const int parts = (chunks + tk - 1) / tk;
+        if (parts > sms) continue;                          // every CTA must be resident while it polls
+        if (parts > 1 && kWsStatusBytes + (size_t)parts * M * N * sizeof(float) > ws_limit) continue;
+        int tc = 16 / tk, ctas = sms / parts;
+        while (tc > 1 && (groups + tc - 1) / tc < ctas) tc >>= 1;
+        if (ctas > (groups + tc - 1) / tc) ctas = (groups + tc - 1) / tc;
+        const int steps = (groups + ctas * tc - 1) / (ctas * tc);
+        // a step costs half its time in latency however many warps take part; the partial sums are written and read back
+        const double us = steps * 0.5 * (tk * tc / 16.0 + 1) + (parts > 1 ? 1.0 : 0.0) + (double)parts * M * N * 8e-6 / 3.0;
+        if (us < best_us) { best_us = us; best = {tk, tc, parts, ctas}; }
+    }
+    return best;
+}
+
+GemvPlan plan_gemv(int M, int K, int N, int bits, int group, int sms, size_t ws_limit)
 {
     // best[m]: least modelled time for m rows; a pass with variant v takes min(rows_v, m) of them
     const double plane_mb = (double)K * (double)N * bits / 8.0 / 1e6;
@@ -903,21 +896,82 @@ GemvPlan plan_gemv(int M, int K, int N, int bits, int sms, size_t ws_limit)
         ps.ctas_per_slice = sms / ps.nkappa;
         ps.smem_bytes = v.half_slices ? kGemvTableBytes / 2 : kGemvTableBytes + 64;
         const size_t need = variant_ws_bytes(v, K, N);
+        ps.mma = uses_mma(bits, group, take);
+        if (ps.mma) {
+            const MmaSplit sp = split_mma(take, K, N, (N + 31) / 32, sms, need);
+            ps.words = 4 * sp.tk;
+            ps.nkappa = sp.nkappa;
+            ps.ctas_per_slice = sp.ctas;
+            ps.smem_bytes = MmaCfg<4, 4>::SMEM;             // at most
+        }
         if (need > g.ws_bytes) g.ws_bytes = need;
         left -= take;
     }
     return g;
 }
 
-template <int BITS>
-static tman_status launch_rows(GemvParams p, int rows, int variant, int sms, cudaStream_t s)
+template <int BITS, int R, int NB, int NE>
+static tman_status launch_mma(MmaParams p, int sms, size_t ws_limit, cudaStream_t s)
 {
-    p.M = rows;
+    const MmaSplit sp = split_mma(p.M, p.K, p.N, p.groups, sms, ws_limit);
+    if (!sp.ctas) return TMAN_ERR_UNSUPPORTED;
+    p.chunks = p.K / 128;
+    p.tk = sp.tk; p.tc = sp.tc; p.nkappa = sp.nkappa;
+    constexpr int smem = MmaCfg<BITS, R>::SMEM;
+    auto kern = decode_mma_kernel<BITS, R, NB, NE>;
+    static std::atomic<bool> raised[kMaxDevices];
+    int dev = 0;
+    if (!device_info(&dev)) return TMAN_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)sp.ctas, (unsigned)sp.nkappa);
+    cfg.blockDim = dim3((unsigned)(32 * sp.tk * sp.tc));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = packed_write_pending(s, /*clear=*/true) ? 0 : 1;      // as in launch_one
+    return launch_with_smem(kern, smem, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, p); });
+}
+
+template <int BITS>
+static tman_status launch_mma_rows(const GemvParams &g, int rows, int sms, size_t ws, cudaStream_t s)
+{
+    MmaParams p = {};
+    p.count = g.count;
+    for (int i = 0; i < kGemvMaxGroup; ++i) {
+        p.packed[i] = g.packed[i];
+        p.planes[i] = reinterpret_cast<const uint8_t *>(g.planes[i]);
+        p.scales[i] = g.scales[i];
+        p.zeros[i] = g.zeros[i];
+        p.y[i] = g.y[i];
+        p.Ng[i] = g.Ng[i];
+        p.col0[i] = g.col0[i];
+        p.grp0[i] = p.groups;
+        if (i < g.count) p.groups += (g.Ng[i] + 31) / 32;
+    }
+    p.x = g.x;
+    p.partials = g.partials; p.status = g.status;
+    p.M = rows; p.K = g.K; p.N = g.N;
+    p.bits = g.bits; p.group = g.group; p.group_shift = g.group_shift; p.nblk = g.nblk;
+    // the columns of B hold the blocks of a chunk as long as there are enough of them for the rows
+    if constexpr (BITS > 2) {
+        if (p.group >= 64 && rows <= 4) return p.group == 128 ? launch_mma<BITS, 1, 1, 1>(p, sms, ws, s) : launch_mma<BITS, 1, 2, 2>(p, sms, ws, s);
+    }
+    if (p.group == 128) return launch_mma<BITS, 1, 1, 2>(p, sms, ws, s);
+    return p.group == 64 ? launch_mma<BITS, 2, 1, 2>(p, sms, ws, s) : launch_mma<BITS, 4, 1, 2>(p, sms, ws, s);
+}
+
+template <int BITS>
+static tman_status launch_rows(GemvParams p, const GemvPass &ps, int sms, cudaStream_t s)
+{
+    p.M = ps.rows;
     const bool pre = p.group >= 64;
-    if (variant == 0) return pre ? launch_mt<BITS, 1, 1, 0>(p, sms, s) : launch_mt<BITS, 1, 0, 0>(p, sms, s);
-    if (variant == 1) return pre ? launch_mt<BITS, 1, 1, 1>(p, sms, s) : launch_mt<BITS, 1, 0, 1>(p, sms, s);
-    if (variant == 2) return pre ? launch_mt<BITS, 2, 1, 1>(p, sms, s) : launch_mt<BITS, 2, 0, 1>(p, sms, s);
-    return pre ? launch_mt<BITS, 4, 1, 1>(p, sms, s) : launch_mt<BITS, 4, 0, 1>(p, sms, s);
+    if (ps.mma) return launch_mma_rows<BITS>(p, ps.rows, sms, variant_ws_bytes(kGemvVariants[ps.variant], p.K, p.N), s);
+    if (ps.variant == 0) return pre ? launch_mt<BITS, 1, 1, 0>(p, sms, s) : launch_mt<BITS, 1, 0, 0>(p, sms, s);
+    if (ps.variant == 1) return pre ? launch_mt<BITS, 1, 1, 1>(p, sms, s) : launch_mt<BITS, 1, 0, 1>(p, sms, s);
+    return pre ? launch_mt<BITS, 2, 1, 1>(p, sms, s) : launch_mt<BITS, 2, 0, 1>(p, sms, s);
 }
 
 __global__ void ws_fill_kernel(uint32_t *ws, size_t words)
@@ -958,7 +1012,7 @@ size_t mpgemv_workspace_bytes(int M, int K, int N, int bits)
     // what the preferred plan needs (on the reference device size: the choice of variants depends on the
     // SM count only through the limit on K-slices); a smaller workspace makes the call fall back to
     // variants with fewer rows per pass, down to what one row needs
-    const GemvPlan g = plan_gemv(M, K, N, bits, kGemvPlanSms, (size_t)-1);
+    const GemvPlan g = plan_gemv(M, K, N, bits, 128, kGemvPlanSms, (size_t)-1);      // (the group has no part in the size)
     return g.npass ? g.ws_bytes : (size_t)-1;
 }
 
@@ -969,7 +1023,7 @@ tman_status launch_mpgemv_grouped(int count, const void *const *packed, const vo
     if (sms <= 0) return TMAN_ERR_CUDA;
     int ntot = 0;
     for (int g = 0; g < count; ++g) ntot += Ns[g];
-    const GemvPlan plan = plan_gemv(M, K, ntot, bits, sms, ws_bytes);
+    const GemvPlan plan = plan_gemv(M, K, ntot, bits, group, sms, ws_bytes);
     if (plan.npass == 0) return TMAN_ERR_UNSUPPORTED;
     uint8_t *w8 = static_cast<uint8_t *>(ws);
     GemvParams p;
@@ -998,14 +1052,14 @@ tman_status launch_mpgemv_grouped(int count, const void *const *packed, const vo
     // a table entry carries up to eight rows (four fp16 pairs): normally one pass over the weights
     int m0 = 0;
     for (int ps = 0; ps < plan.npass; ++ps) {
-        const int rows = plan.pass[ps].rows, variant = plan.pass[ps].variant;
+        const int rows = plan.pass[ps].rows;
         p.x = static_cast<const __half *>(x) + (size_t)m0 * K;
         for (int g = 0; g < kGemvMaxGroup; ++g)
             p.y[g] = static_cast<__half *>(y[g < count ? g : 0]) + (size_t)m0 * p.Ng[g];
         tman_status st;
-        if (bits == 2) st = launch_rows<2>(p, rows, variant, sms, s);
-        else if (bits == 3) st = launch_rows<3>(p, rows, variant, sms, s);
-        else st = launch_rows<4>(p, rows, variant, sms, s);
+        if (bits == 2) st = launch_rows<2>(p, plan.pass[ps], sms, s);
+        else if (bits == 3) st = launch_rows<3>(p, plan.pass[ps], sms, s);
+        else st = launch_rows<4>(p, plan.pass[ps], sms, s);
         if (st != TMAN_OK) return st;
         m0 += rows;
     }

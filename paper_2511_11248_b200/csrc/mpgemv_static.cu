@@ -72,7 +72,7 @@ extern "C" tman_status tman_mpgemv_static(const void *packed, size_t packed_byte
     // partial-sum area must say "no sum pending" everywhere this call will look.
     st = launch_workspace_init(ws, need, s);
     if (st != TMAN_OK) return st;
-    st = launch_mpgemv(packed, x_f16, y_f16, M, K, N, bits, group, ws, kStaticWsBytes, s);
+    st = launch_mpgemv(packed, x_f16, y_f16, M, K, N, bits, group, ws, need, s);
     if (st != TMAN_OK) return st;
     if (status_dev &&
         cudaMemcpyAsync(status_dev, ws, sizeof(unsigned int), cudaMemcpyDeviceToDevice, s) != cudaSuccess)

@@ -110,6 +110,28 @@ def test_rows_in_fp16_tables_stay_near_the_predicted_error(M, factor):
     assert rel_err(got, ref) <= 2e-3
 
 
+@pytest.mark.parametrize("M,bits,G", [(3, 3, 64), (4, 4, 128), (5, 2, 32), (5, 3, 64), (6, 2, 64), (7, 4, 32), (8, 2, 128), (8, 3, 128), (8, 4, 64)])
+@pytest.mark.parametrize("K,Ns", [(128, (8,)), (640, (32, 40)), (2176, (264,)), (4096, (2056, 8, 40))])
+def test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, Ns):
+    # one chunk of 128 k; a team with idle warps; a second K-slice of a single chunk; ragged groups of 32 columns and a
+    # matrix narrower than one.  Codes and activations are exact operands and sums fp32, so what is left is the rounding of
+    # the result to fp16, 2^-11 = 4.9e-4 of it, and fp32 sums of up to 4096 terms, below 1e-5.
+    cases = [synth.small_case(M, K, N, bits, G, seed=800 + 10 * i + M, outliers=True) for i, N in enumerate(Ns)]
+    for c in cases[1:]:
+        c.x[:] = cases[0].x
+    devs = [H.device_case(c) for c in cases]
+    packed = [H.pack_case(c, d) for c, d in zip(cases, devs)]
+    ws = H.alloc_workspace(B.OP_GEMV, M, K, sum(Ns), bits, G)
+    for _ in range(2):                                       # the second call finds the workspace as the first left it
+        ys = [H.alloc_y(M, N) for N in Ns]
+        B.tman_mpgemv_grouped(packed, devs[0]["x"], ys, M, K, Ns, bits, G, ws)
+        assert B.tman_read_status(ws) == 0
+        H.check_guards()
+        for c, y in zip(cases, ys):
+            ref = orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)
+            assert rel_err(H.to_f64(y), ref) <= 5.1e-4
+
+
 def test_repeat_calls_share_workspace_and_agree():
     c = synth.small_case(2, 2048, 264, 4, 64, seed=21)
     dev = H.device_case(c)
