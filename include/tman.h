@@ -195,9 +195,9 @@ tman_status tman_mpgemm_ternary_i8(const void *packed, size_t packed_bytes, cons
 tman_status tman_dequant_ternary_int8(const void *packed, size_t packed_bytes, int K, int N, int group,
                                       int8_t *w8_nk, void *workspace, size_t ws_bytes, tman_stream_t stream);
 
-/* Prefill (paper Sec. 4.1 two-level LUT dequantization, Fig. 7; Sec. 4.2 three-stage pipeline,
- * Fig. 9): packed tiles are staged in shared memory, rebuilt into fp16 tiles through the
- * repack step and the per-(block, column) conversion table, and multiplied on the tensor
+/* Prefill (paper Sec. 4.1 two-level dequantization, Fig. 7; Sec. 4.2 three-stage pipeline,
+ * Fig. 9): packed tiles are staged in shared memory, rebuilt as fp16 weights in tensor memory (bit repacking, then
+ * fp16(s * (q - z)), rounded once), and multiplied on the tensor
  * cores with fp32 accumulation.  M >= 1.
  *   - The output is cut into tiles dealt to the SMs; when the tiles do not go round evenly, or
  *     are too few to fill the machine, the k-range of tiles is divided among the SMs and summed,
@@ -253,13 +253,13 @@ tman_status tman_debug_luts(const void *x_f16, int M, int K, float *lut, tman_st
  * full-precision weights; "Gain from pipelined execution": against doing load, dequantization and
  * multiplication in turn).  Every variant returns the same y as tman_mpgemm (same bits); only the time
  * differs.  Arguments as tman_mpgemm, plus
- *   variant 0  the product path (two-level lookup dequantization, pipelined)
+ *   variant 0  the product path (bit repacking, codes to fp16 by exact mantissa arithmetic, pipelined)
  *           1  ConvertDQ: every code converted to fp16 with an integer-to-float instruction, zero-point
  *              subtracted, scale multiplied
  *           2  LoadFull: no dequantization; fp16 weights wt_f16 [N][K] (device, 16-byte aligned, row n =
  *              fp16(s * (q - z)) of channel n) are loaded by TMA in place of the packed tiles
- *           3  Sequential: the product's dequantization with a ring of one stage, so that the load, the
- *              dequantization and the multiplication of a k-block follow one another
+ *           3  Sequential: the product's dequantization, but a k-block's activations are loaded when the block before it
+ *              has been multiplied and its weights rebuilt when they are there, so that the three follow one another
  *   wt_f16  used by variant 2 only (else may be NULL).
  * Variants 1-3 exist for bits == 4 (TMAN_ERR_UNSUPPORTED otherwise); variant 2 additionally wants N to be a
  * multiple of 32 (TMAN_ERR_UNSUPPORTED otherwise). */
@@ -281,7 +281,7 @@ tman_status tman_debug_role_stamps(const void *workspace, size_t ws_bytes, int c
 
 /* How tman_mpgemm would cut a call's work on the current device (host-side decision, nothing is
  * launched; no counterpart in the paper).  out8 (host) receives: 1 if pairs of CTAs work on a tile
- * else 0; 128-token row blocks per CTA; row tiles; column tiles; 1 if every tile is dealt whole
+ * else 0; tokens of a tile in units of 128, rounded up; row tiles; column tiles (of 128 or, in pairs, 256 channels); 1 if every tile is dealt whole
  * else 0; workers (CTAs or pairs) launched; number of last tiles whose k-blocks are dealt as equal
  * spans (0: none); pieces every tile's k-blocks are split into (0: not split).  Tests use it to
  * know which path a shape takes. */

@@ -64,6 +64,22 @@ def test_pair_kernel_cases(M, K, N, bits, G):
     check_full(synth.small_case(M, K, N, bits, G, seed=M + K + N + bits, outliers=(bits == 4)))
 
 
+# Where the transposed kernel's parts have their edges: a single CTA and a pair of one and of two tokens more, one activation
+# row per load stage of 4, 2 and 1 k-blocks (64 / 128 rows of a CTA), tiles of 16 to 256 tokens, one packed stage and a ragged
+# last one (K = 128, 384, 640), channels that end inside a strip group, a CTA and a pair.
+EDGES = [(16, 128, 8, 2, 32), (17, 384, 136, 3, 64), (33, 640, 264, 4, 128), (128, 1152, 120, 2, 128), (129, 384, 392, 4, 32),
+         (256, 640, 248, 3, 32), (257, 1280, 264, 2, 64), (1, 4096, 2056, 4, 64)]
+
+
+@pytest.mark.parametrize("M,K,N,bits,G", EDGES)
+def test_edges_of_the_transposed_kernel(M, K, N, bits, G):
+    # weights rounded to fp16 once (2^-12 each, adding up like a random walk), fp32 sums, the result rounded to fp16
+    # (2^-11 = 4.9e-4 of it): 1e-3 holds both
+    c = synth.small_case(M, K, N, bits, G, seed=11 * M + K + N + bits)
+    got = H.to_f64(run_gemm(c))
+    assert rel_err(got, orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)) <= 1e-3
+
+
 # Long K and few tiles: every tile's k-blocks go to several workers, which exchange fp32 chunks through
 # the workspace and share the summing.  Pairs of CTAs with two and one row block, a single CTA, ragged
 # M and N, every bit width; compared element by element.
