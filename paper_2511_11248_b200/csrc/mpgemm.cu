@@ -9,14 +9,14 @@
 // memory as TMA leaves them.
 // The output is cut into tiles of 128 channels (a CTA) or 256 (a pair of CTAs on two SMs, tcgen05.mma.cta_group::2: each CTA
 // holds half of the tokens' rows and rebuilds its own 128 channels, so that an activation is fetched once per 256 channels).
-// A tile's work is its K/64 k-blocks.  The host chooses the tokens of a tile and deals the tiles to the workers (CTAs or
+// A tile's work is its K/128 units of 128 k.  The host chooses the tokens of a tile and deals the tiles to the workers (CTAs or
 // pairs, at most one per SM or SM pair), whole as far as they go round; where whole tiles would leave SMs idle, the
-// k-blocks of the last tiles are laid end to end and dealt in equal spans, and a tile whose k-blocks fall into several
+// units of the last tiles are laid end to end and dealt in equal spans, and a tile whose units fall into several
 // spans is summed through fp32 partial tiles in the workspace (see "split of the work").
 // Four kinds of agents run concurrently, guarded by mbarriers (the paper's DMA / vector-core / matrix-core stages):
-//   * warp 0, one lane : TMA loads of the activations (a ring of 64-deep blocks, 128-byte swizzle) and, running ahead on a ring
-//                        of its own, of the packed bit-plane words (256-deep boxes: runs of 128 bytes per strip and plane);
-//   * warps 2..17      : four groups of four warps, each group every fourth k-block of the walk: read the plane words of their channel,
+//   * warp 0, one lane : TMA loads of the activations (a ring of units, 128-byte swizzle) and, running ahead on a ring of its own, of the
+//                        packed bit-plane words (runs of 128 bytes per strip and plane);
+//   * warps 2..17      : four groups of four warps, each group every fourth unit of the walk: read the plane words of their channel,
 //                        merge them into codes (level 1: bit-serial -> bit-parallel), turn codes into fp16 weights (level 2)
 //                        and store them to tensor memory;
 //   * warp 1, one lane : tcgen05.mma (fp16 x fp16 -> fp32 in tensor memory), one per 16 k; tcgen05.commit hands the
@@ -37,25 +37,29 @@
 namespace tman {
 namespace {
 
-constexpr int BK = 64;                          // k-block
+constexpr int BK = 64;                          // k of a 128-byte row of activations in shared memory
+constexpr int UK = 128;                         // k of a unit: what a group of warps rebuilds at a time
 constexpr int CH = 128;                         // channels a CTA rebuilds = lanes of tensor memory
 constexpr int MAX_TOKENS = 256;                 // columns of an accumulator
 constexpr int NUM_DEQ_WARPS = 16, DEQ_GROUPS = 4;
 constexpr int NUM_EPI_WARPS = 8;                // two per quarter of the tensor-memory lanes (alternate 32-token chunks)
 constexpr int GEMM_THREADS = 32 * (2 + NUM_DEQ_WARPS + NUM_EPI_WARPS);
-constexpr int P_KB = 4;                         // k-blocks of a packed stage: one 128-byte run per strip and plane
-constexpr int P_PLANE_BYTES = (CH / 4) * 128;   // one plane of a packed stage
-constexpr int P_RING_BYTES = 64 * 1024;         // packed ring: 8 / 5 / 4 stages for 2 / 3 / 4 bits
-constexpr int X_RING_BYTES = 128 * 1024;        // activation ring: stages of 4, 2 or 1 k-blocks (up to 64, 128, 256 rows of a CTA)
-constexpr int W_TILE_BYTES = CH * BK * 2;       // a k-block of fp16 weights (LoadFull variant only)
-constexpr int TMEM_COLS = 512, TMEM_W = 256;    // accumulator in columns [0, 256), weight buffers from 256 on
+constexpr int P_PLANE_BYTES = (CH / 4) * 128;   // one plane of a packed stage (two units): a 128-byte run per strip
+constexpr int P_RING_BYTES = 64 * 1024;         // 8 stages for 2 bits, 4 for 3 and 4
+constexpr int X_RING_BYTES = 128 * 1024;        // activation ring: stages of two units (8 of up to 32 rows, 4 of up to 64) or one (4 of up to 128)
+constexpr int W_TILE_BYTES = CH * BK * 2;       // half a unit of fp16 weights in shared memory (LoadFull variant only)
+constexpr int TMEM_COLS = 512;                  // accumulator from column 0, weight buffers of 64 columns behind it
+constexpr int W_COLS = UK / 2;
 constexpr int kMaxGemmCtas = 160;               // the workspace is sized for at most this many CTAs
 constexpr int GEMM_SMEM = P_RING_BYTES + X_RING_BYTES + 512;
 
-// Workspace: status word (kWsStatusBytes), one flag per epilogue warp of every CTA, a reserved area, then one fp32 partial
-// tile per CTA (a worker writes at most one per launch).
+// Workspace: status word (kWsStatusBytes), one flag per epilogue warp of every CTA (spans), one per (epilogue warp of a
+// CTA, sending piece) (even pieces), then one fp32 partial tile per CTA (a worker writes at most one per launch): per
+// epilogue warp [token][channel], its 32 channels x half of the tokens.
+constexpr int kMaxSplit = 32;                   // even pieces of a tile
 constexpr size_t kGemmFlagsOff = kWsStatusBytes;
-constexpr size_t kGemmPartialOff = kWsStatusBytes + 8192 + 40960;
+constexpr size_t kGemmPieceFlagsOff = kWsStatusBytes + 8192;
+constexpr size_t kGemmPartialOff = kGemmPieceFlagsOff + (size_t)kMaxGemmCtas * NUM_EPI_WARPS * kMaxSplit * sizeof(uint32_t);
 constexpr uint32_t kFlagEmpty = 0x7FA5A5A5u;    // what tman_workspace_init leaves behind
 // Role time stamps (only in a library built with -DTMAN_ROLE_STAMPS; the workspace has room for them in
 // every build so that its layout does not depend on the flag): per CTA and warp four 64-bit words --
@@ -70,7 +74,7 @@ constexpr size_t kStampBytesPerCta = (size_t)kGemmWarps * kStampWordsPerWarp * s
 #else
 #define TMAN_STAMPED_WAIT(acc, call) (call)
 #endif
-constexpr size_t kPartialBytesPerCta = 256 * 1024;
+constexpr size_t kPartialBytesPerCta = (size_t)MAX_TOKENS * CH * sizeof(float);
 
 struct GemmParams {
     const uint8_t  *packed;
@@ -78,14 +82,15 @@ struct GemmParams {
     const uint16_t *zeros;
     __half         *y;
     uint32_t       *status;
-    uint32_t       *flags;
+    uint32_t       *flags, *piece_flags;
     float          *partial;
     int M, K, N, bits, group;
     int nt;                    // tokens of a tile (a multiple of 16, of 32 in a pair)
-    int wbufs;                 // weight buffers in tensor memory (8 or 4)
-    int xkb_sh, xst_sh;        // activation ring: log2 of the k-blocks of a stage and of the stages
+    int wbufs, wcol;           // weight buffers in tensor memory and their first column
+    int xu_sh, xst_sh;         // activation ring: log2 of the units of a stage and of the stages
     int tiles_m, tiles_n;
-    int span_tiles;            // the last span_tiles tiles are dealt as equal spans of k-blocks (0: every tile whole)
+    int span_tiles;            // the last span_tiles tiles are dealt as equal spans of units (0: every tile whole)
+    int split_s;               // even pieces of every tile (0: not split so)
     int col_fastest;           // tile number = row tile * tiles_n + column tile (else column tile * tiles_m + row tile)
     long long *stamps;         // role time stamps (written only by a build with TMAN_ROLE_STAMPS)
 };
@@ -95,7 +100,9 @@ struct GemmParams {
 constexpr int kGemmProduct = 0;      // the product path, pipelined
 constexpr int kGemmConvertDq = 1;    // codes converted to floating point one by one, then subtract and multiply
 constexpr int kGemmLoadFull = 2;     // fp16 weights prepared in memory and loaded by TMA, no dequantization
-constexpr int kGemmSequential = 3;   // the product's dequantization; a k-block is loaded when the one before it has been multiplied, and dequantized when it is loaded
+constexpr int kGemmSequential = 3;   // the product's dequantization; a unit is loaded when the one before it has been multiplied, and dequantized when it is loaded
+
+template <int I> struct IntC { static constexpr int value = I; };
 
 // ---- level 2: codes to fp16 weights ---------------------------------------------------------------
 // w = fp16( s * (c - z) ), rounded once.  A code in the mantissa of an fp16 number between 1024 and 2048 is 1024 + c
@@ -107,9 +114,8 @@ struct BlockConsts {
     __device__ __forceinline__ void set(__half s, uint32_t z)
     {
         s2 = __half2half2(s);
-        const __half zh = __ushort2half_rn((unsigned short)z);
-        sub = __hsub2(__halves2half2(__ushort2half_rn(0), __ushort2half_rn(0)),
-                      __hadd2(__halves2half2(__ushort2half_rn(1024), __ushort2half_rn(64)), __half2half2(zh)));
+        const uint32_t u = z * 0x00100001u + 0xD400E400u;        // the two constants with z in their mantissas
+        sub = *reinterpret_cast<const __half2 *>(&u);
     }
 };
 
@@ -170,12 +176,13 @@ __device__ __forceinline__ void dequant_word(const uint32_t (&w)[BITS], const Bl
     // level 2: byte b of X holds the codes of two adjacent weights; copied into both halves of a register, the low
     // half keeps the low nibble and the high half the high one
     constexpr uint32_t M1 = (1u << BITS) - 1u, MASK = M1 | (M1 << 20);
+    const uint32_t magic = opaque_u32<0x64006400u>();
     const __half2 mul = __halves2half2(__ushort2half_rn(1), __float2half_rn(0.0625f));
 #pragma unroll
     for (int ph = 0; ph < 4; ++ph)
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const uint32_t c = (__byte_perm(X[ph], 0u, 0x1111u * b) & MASK) | 0x64006400u;
+            const uint32_t c = and_or(__byte_perm(X[ph], 0u, 0x1111u * b), MASK, magic);
             const __half2 e = __hmul2(t.s2, __hfma2(*reinterpret_cast<const __half2 *>(&c), mul, t.sub));
             out[4 * ph + b] = *reinterpret_cast<const uint32_t *>(&e);
         }
@@ -183,16 +190,17 @@ __device__ __forceinline__ void dequant_word(const uint32_t (&w)[BITS], const Bl
 
 // ---- split of the work ----------------------------------------------------------------------
 // T tiles (row tile fastest), W workers.  The first `whole` tiles (a multiple of W) are dealt whole,
-// round-robin.  The k-blocks of the remaining tiles (fewer than 2 W), laid end to end in units of two
-// k-blocks (a 128-wide quantization block is never cut), are dealt in equal contiguous spans, so
+// round-robin.  The units of the remaining tiles (fewer than 2 W), laid end to end (a unit is as deep as the
+// longest quantization block), are dealt in equal contiguous spans, so
 // every worker is busy to the end whatever the shape.  A span is shorter than two tiles: at most
 // the end of one tile, one whole tile and the start of the next.  A tile cut into several pieces
 // ("split tile") is summed by the worker that owns its last unit: the others, which all have lower
 // numbers, write their fp32 accumulators to the workspace and raise a flag.  A worker's walk: first
 // the piece that it only contributes (so that it is ready long before it is needed), then its whole
 // tiles, last the piece of the tile that it finishes.
-// Even pieces (outputs with few tiles): as many workers as tiles x pieces, so that the spans are the pieces.
-struct Segment { int tile, kb0, kb1; bool whole, finishes; };
+// Even pieces (outputs with few tiles): as many workers as tiles x pieces, so that the spans are the pieces.  They finish
+// together and share the summing: every piece sends the accumulators of the tokens that others sum, and adds up its own.
+struct Segment { int tile, u0, u1; bool whole, finishes; };
 
 struct Span {
     int full, Ur;              // tiles dealt whole round-robin; units of the remaining tiles (Ur x workers fits 31 bits, host)
@@ -201,7 +209,7 @@ struct Span {
     Segment early, mid, late;  // the piece this worker only contributes; a whole tile of its span; the piece it finishes
     bool has_early, has_mid, has_late;
     __device__ Span(const GemmParams &p, int worker, int nworkers)
-        : full(p.tiles_m * p.tiles_n - p.span_tiles), Ur(0), next_whole(worker), nu(p.K / (2 * BK)), W(nworkers),
+        : full(p.tiles_m * p.tiles_n - p.span_tiles), Ur(0), next_whole(worker), nu(p.K / UK), W(nworkers),
           has_early(false), has_mid(false), has_late(false)
     {
         if (p.span_tiles == 0) return;
@@ -213,8 +221,8 @@ struct Span {
             const int k0 = (lo > t0) ? lo - t0 : 0, k1 = hi - t0;
             Segment s;
             s.tile = full + tile;
-            s.kb0 = 2 * k0;
-            s.kb1 = 2 * k1;
+            s.u0 = k0;
+            s.u1 = k1;
             s.whole = (k0 == 0 && k1 == nu);
             s.finishes = (k1 == nu);
             if (s.whole) { mid = s; has_mid = true; }
@@ -228,8 +236,8 @@ struct Span {
         if (has_early) { s = early; has_early = false; return true; }
         if (next_whole < full) {
             s.tile = next_whole;
-            s.kb0 = 0;
-            s.kb1 = 2 * nu;
+            s.u0 = 0;
+            s.u1 = nu;
             s.whole = s.finishes = true;
             next_whole += W;
             return true;
@@ -252,20 +260,19 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
               const __grid_constant__ CUtensorMap tmap_wf, const GemmParams p)
 {
     constexpr int NCTA = PAIR ? 2 : 1;
-    constexpr int PST = V == kGemmSequential ? 1 : P_RING_BYTES / (BITS * P_PLANE_BYTES);
-    constexpr int P_STAGE_BYTES = BITS * P_PLANE_BYTES;
+    constexpr int P_STAGE_BYTES = BITS * P_PLANE_BYTES, P_STAGES = BITS == 2 ? 8 : 4;
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;   // in a pair, CTA 0 issues the MMAs and owns the shared barriers
     uint8_t *p_tiles = smem, *x_tiles = smem + P_RING_BYTES;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + P_RING_BYTES + X_RING_BYTES);
-    // packed stage loaded (TMA) / free (dequantization warps); activation stage loaded (TMA) / free (MMA commit); weights of a
+    // packed stage loaded (TMA) / free (the four warps of the groups of its two units); activation stage loaded (TMA) / free (MMA commit); weights of a
     // buffer ready (the four warps of a group; in a pair both CTAs' in CTA 0) / free (MMA commit); accumulator full (commit) /
     // empty (epilogue warps; in a pair both CTAs' in CTA 0)
     const uint32_t ploaded0 = smem_u32(bars), pempty0 = smem_u32(bars + 8), xloaded0 = smem_u32(bars + 16), xempty0 = smem_u32(bars + 24),
                    full0 = smem_u32(bars + 32), empty0 = smem_u32(bars + 40), accf = smem_u32(bars + 48), acce = smem_u32(bars + 49);
+    const uint32_t sums0 = smem_u32(bars + 52);            // partial sums of an epilogue warp loaded
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 50);
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (the shuffle tells the compiler that it is uniform)
-    const bool base_ok = (smem_u32(smem) & 1023u) == 0u;   // the swizzled tiles need 1 KB alignment (same in every CTA)
 
     // The next kernel of the stream may set itself up while this one runs, as this one does now; nothing below the wait
     // starts before the previous kernel has ended.
@@ -273,16 +280,20 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
     if (threadIdx.x == 0) {
         for (int s = 0; s < 8; ++s) {
             mbar_init(ploaded0 + 8 * s, 1);
-            mbar_init(pempty0 + 8 * s, NUM_DEQ_WARPS);
+            mbar_init(pempty0 + 8 * s, 2 * (NUM_DEQ_WARPS / DEQ_GROUPS));
             mbar_init(xloaded0 + 8 * s, 1);
             mbar_init(xempty0 + 8 * s, 1);
             mbar_init(full0 + 8 * s, NCTA * (NUM_DEQ_WARPS / DEQ_GROUPS));
             mbar_init(empty0 + 8 * s, 1);
+            mbar_init(sums0 + 8 * s, 1);
         }
         mbar_init(accf, 1);
         mbar_init(acce, NCTA * NUM_EPI_WARPS);
         *tmem_slot = 0xFFFFFFFFu;
         fence_barrier_init();
+    } else if (threadIdx.x == 32 * 2) {
+        prefetch_tensormap(&tmap_x);
+        prefetch_tensormap(V == kGemmLoadFull ? &tmap_wf : &tmap_w);
     }
     __syncthreads();
     if (warp == 1) {
@@ -304,9 +315,8 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     bool ok = tmem_base != 0xFFFFFFFFu;
-    const bool hdr_ok = header_matches(p.packed, p.K, p.N, p.bits, p.group);   // same answer in every CTA
-    const bool run = hdr_ok && base_ok;
-    if (!run && threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)(hdr_ok ? TMAN_ERR_LAYOUT : TMAN_ERR_BAD_PACKED));
+    const bool run = (smem_u32(smem) & 1023u) == 0u;       // the swizzled tiles need 1 KB alignment (same in every CTA)
+    if (!run && threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)TMAN_ERR_LAYOUT);
     long long wait_a = 0, wait_b = 0;                  // clocks in this thread's waits (time-stamp builds only)
 #ifdef TMAN_ROLE_STAMPS
     const long long role_t0 = clock64();
@@ -330,59 +340,59 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         // nothing to do: every output stays untouched
     } else if (warp == 0) {
         // ---- stage 1: activations and packed words by TMA -----------------------------------------------
-        // The warp walks as one (uniform registers: operands of the copies), an elected lane issues both streams: the packed stage an activation stage needs, further packed stages as far as their
-        // ring has room, the activation stage.  What a load needs is worked out once a segment: a division per load made this
-        // thread the slowest agent (0.6 us a k-block).
-        {
-            const bool lead = elect_one();
-            const uint32_t x_kb_bytes = (uint32_t)rows_cta * 128u, x_stage_bytes = x_kb_bytes << p.xkb_sh;
-            const uint32_t p_base = smem_u32(p_tiles), x_base = smem_u32(x_tiles);
-            const int xkb = 1 << p.xkb_sh, xst_mask = (1 << p.xst_sh) - 1;
-            Span ps = span;
-            Segment pg;
-            int pkb = 0, pend = 0, pstrip = 0, pslot = 0, ahead = 0;        // ahead: packed stages issued beyond the ones the activations have reached
-            uint32_t pph = 1u;                         // parity of "free" for this turn of the ring
-            bool pmore = V != kGemmLoadFull;
-            auto packed_next = [&]() {
-                pmore = ps.next(pg);
-                if (pmore) { pkb = pg.kb0; pend = pg.kb1; pstrip = tile_ch0(pg.tile) / 4; }
-            };
-            auto packed_issue = [&]() {
-                const uint32_t bar = ploaded0 + 8 * pslot, dst = p_base + (uint32_t)pslot * P_STAGE_BYTES;
-                if (lead) {
-                    mbar_expect_tx(bar, P_STAGE_BYTES);
+        // The warp walks as one (uniform registers: operands of the copies), an elected lane issues both streams: the packed
+        // stage a unit needs, further packed stages as far as their ring has room, the activations.  What a load needs
+        // is worked out once a segment: a division per load made this thread the slowest agent (0.6 us per 64 k).
+        const bool lead = elect_one();
+        const uint32_t x_stage_bytes = (uint32_t)rows_cta * 256u << p.xu_sh;
+        const uint32_t p_base = smem_u32(p_tiles), x_base = smem_u32(x_tiles), xst_mask = (1u << p.xst_sh) - 1u;
+        const int xu = 1 << p.xu_sh;
+        Span ps = span;
+        Segment pg;
+        int pu = 0, pend = 0, pstrip = 0, ahead = 0;       // ahead: packed stages issued beyond the one the activations have reached
+        uint32_t pc = 0;                                   // packed stages issued
+        bool pmore = V != kGemmLoadFull;
+        auto packed_next = [&]() {
+            pmore = ps.next(pg);
+            if (pmore) { pu = pg.u0; pend = pg.u1; pstrip = tile_ch0(pg.tile) / 4; }
+        };
+        auto packed_issue = [&]() {
+            const uint32_t st = pc % P_STAGES, bar = ploaded0 + 8 * st, dst = p_base + st * P_STAGE_BYTES;
+            if (lead) {
+                mbar_expect_tx(bar, P_STAGE_BYTES);
 #pragma unroll
-                    for (int i = 0; i < BITS; ++i) tma_load_3d(dst + i * P_PLANE_BYTES, &tmap_w, pkb * (BK / 8), i, pstrip, bar);
-                }
-                if (++pslot == PST) { pslot = 0; pph ^= 1u; }
-                ++ahead;
-                pkb += P_KB;
-                if (pkb >= pend) packed_next();
-            };
-            if (pmore) packed_next();
-            uint32_t xc = 0;                           // activation stages issued
-            while (ok && span.next(sg)) {
-                const int row0 = tile_tm(sg.tile) * p.nt + (int)rank * rows_cta, ch0 = tile_ch0(sg.tile);
-                for (int kb = sg.kb0; kb < sg.kb1; kb += xkb, ++xc) {
-                    if constexpr (V != kGemmLoadFull) {
-                        if (((kb - sg.kb0) & (P_KB - 1)) == 0) {
-                            // the activations reach another packed stage: it has to be on its way
-                            if (ahead == 0) {
-                                if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(pempty0 + 8 * pslot, pph)))) { ok = false; break; }
-                                packed_issue();
-                            }
-                            --ahead;
-                        }
-                        while (pmore && warp_all(mbar_test(pempty0 + 8 * pslot, pph))) packed_issue();
+                for (int i = 0; i < BITS; ++i) tma_load_3d(dst + i * P_PLANE_BYTES, &tmap_w, pu * (UK / 8), i, pstrip, bar);
+            }
+            ++pc;
+            ++ahead;
+            pu += 2;
+            if (pu >= pend) packed_next();
+        };
+        auto packed_bar = [&]() { return pempty0 + 8 * (pc % P_STAGES); };
+        auto packed_par = [&]() { return ((pc / P_STAGES) & 1u) ^ 1u; };
+        if (pmore) packed_next();
+        uint32_t xc = 0;                                   // activation stages issued
+        while (ok && span.next(sg)) {
+            const int row0 = tile_tm(sg.tile) * p.nt + (int)rank * rows_cta, ch0 = tile_ch0(sg.tile);
+            for (int u = sg.u0; u < sg.u1; u += xu, ++xc) {
+                if (V != kGemmLoadFull && ((u - sg.u0) & 1) == 0) {
+                    if (ahead == 0) {
+                        if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(packed_bar(), packed_par())))) { ok = false; break; }
+                        packed_issue();
                     }
-                    const uint32_t st = xc & (uint32_t)xst_mask, bar = xloaded0 + 8 * st;
-                    if constexpr (V == kGemmSequential)
-                        if (xc > 0 && !warp_all(mbar_wait(xempty0 + 8 * ((xc - 1) & (uint32_t)xst_mask), ((xc - 1) >> p.xst_sh) & 1u))) { ok = false; break; }
-                    if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(xempty0 + 8 * st, ((xc >> p.xst_sh) & 1u) ^ 1u)))) { ok = false; break; }
-                    if (lead) {
-                        mbar_expect_tx(bar, x_stage_bytes + (V == kGemmLoadFull ? W_TILE_BYTES : 0));
-                        tma_load_3d(x_base + st * x_stage_bytes, &tmap_x, 0, row0, kb, bar);
-                        if constexpr (V == kGemmLoadFull) tma_load_2d(p_base + st * W_TILE_BYTES, &tmap_wf, kb * BK, ch0, bar);
+                    --ahead;
+                    while (pmore && warp_all(mbar_test(packed_bar(), packed_par()))) packed_issue();
+                }
+                const uint32_t st = xc & xst_mask, bar = xloaded0 + 8 * st;
+                if constexpr (V == kGemmSequential)
+                    if (xc > 0 && !warp_all(mbar_wait(xempty0 + 8 * ((xc - 1) & xst_mask), ((xc - 1) >> p.xst_sh) & 1u))) { ok = false; break; }
+                if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(xempty0 + 8 * st, ((xc >> p.xst_sh) & 1u) ^ 1u)))) { ok = false; break; }
+                if (lead) {
+                    mbar_expect_tx(bar, x_stage_bytes + (V == kGemmLoadFull ? 2 * W_TILE_BYTES : 0));
+                    tma_load_3d(x_base + st * x_stage_bytes, &tmap_x, 0, row0, 2 * u, bar);
+                    if constexpr (V == kGemmLoadFull) {
+                        tma_load_2d(p_base + st * (2 * W_TILE_BYTES), &tmap_wf, u * UK, ch0, bar);
+                        tma_load_2d(p_base + st * (2 * W_TILE_BYTES) + W_TILE_BYTES, &tmap_wf, u * UK + BK, ch0, bar);
                     }
                 }
             }
@@ -395,42 +405,45 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
             const uint32_t idesc = (1u << 4) | ((uint32_t)(p.nt >> 3) << 17) | ((uint32_t)((NCTA * CH) >> 4) << 24);
             // descriptors in 16-byte units: only the low word (start address) changes
             const uint64_t bdesc0 = make_kmajor_sw128_desc(smem_u32(x_tiles)), adesc0 = make_kmajor_sw128_desc(smem_u32(p_tiles));
-            const uint32_t kb_units = (uint32_t)rows_cta * 8u;
-            const int xkb_mask = (1 << p.xkb_sh) - 1;
+            const uint32_t half_units = (uint32_t)rows_cta * 8u, xst_mask = (1u << p.xst_sh) - 1u;
+            const int xu_mask = (1 << p.xu_sh) - 1;
             uint32_t ti = 0, ph = 0u, s = 0, xst = 0;
             while (ok && span.next(sg)) {
                 if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(acce, (ti & 1u) ^ 1u)))) { ok = false; break; }
                 tcgen05_fence_after();
-                const int nkb = sg.kb1 - sg.kb0;
                 uint32_t acc = 0u;
-                for (int i = 0; i < nkb; ++i) {
+                for (int u = sg.u0; u < sg.u1; ++u) {
                     if (!TMAN_STAMPED_WAIT(wait_b, warp_all(mbar_wait(full0 + 8 * s, ph)))) { ok = false; break; }
                     tcgen05_fence_after();
-                    const uint64_t bdesc = bdesc0 + ((xst << p.xkb_sh) + (uint32_t)(i & xkb_mask)) * kb_units;
-                    const uint64_t adesc = adesc0 + s * (W_TILE_BYTES / 16);
-                    const uint32_t wt = tmem_base + TMEM_W + 32u * s;
-                    const bool xlast = (i & xkb_mask) == xkb_mask || i == nkb - 1;
+                    const int xi = (u - sg.u0) & xu_mask;                  // unit of the activation stage
+                    const bool xlast = xi == xu_mask || u == sg.u1 - 1;
+                    const uint64_t bdesc = bdesc0 + 2u * ((xst << p.xu_sh) + (uint32_t)xi) * half_units;
+                    const uint64_t adesc = adesc0 + xst * (2 * W_TILE_BYTES / 16);
+                    const uint32_t wt = tmem_base + (uint32_t)p.wcol + (uint32_t)W_COLS * s;
                     if (lead) {
 #pragma unroll
-                        for (int j = 0; j < BK / 16; ++j) {
+                        for (int j = 0; j < UK / 16; ++j) {
+                            const uint64_t bd = bdesc + 2 * (j & 3) + (j >> 2) * half_units;
                             if constexpr (V == kGemmLoadFull) {
-                                if constexpr (PAIR) tcgen05_mma2_f16(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc, acc);
-                                else tcgen05_mma_f16(tmem_base, adesc + 2 * j, bdesc + 2 * j, idesc, acc);
+                                const uint64_t ad = adesc + 2 * (j & 3) + (j >> 2) * (W_TILE_BYTES / 16);
+                                if constexpr (PAIR) tcgen05_mma2_f16(tmem_base, ad, bd, idesc, acc);
+                                else tcgen05_mma_f16(tmem_base, ad, bd, idesc, acc);
                             } else {
-                                if constexpr (PAIR) tcgen05_mma2_f16_ts(tmem_base, wt + 8 * j, bdesc + 2 * j, idesc, acc);
-                                else tcgen05_mma_f16_ts(tmem_base, wt + 8 * j, bdesc + 2 * j, idesc, acc);
+                                if constexpr (PAIR) tcgen05_mma2_f16_ts(tmem_base, wt + 8 * j, bd, idesc, acc);
+                                else tcgen05_mma_f16_ts(tmem_base, wt + 8 * j, bd, idesc, acc);
                             }
                             acc = 1u;
                         }
-                        if constexpr (PAIR) tcgen05_commit2_both(empty0 + 8 * s);
-                        else tcgen05_commit(empty0 + 8 * s);
-                        if (xlast) {
-                            if constexpr (PAIR) tcgen05_commit2_both(xempty0 + 8 * xst);
-                            else tcgen05_commit(xempty0 + 8 * xst);
+                        if constexpr (PAIR) {
+                            tcgen05_commit2_both(empty0 + 8 * s);
+                            if (xlast) tcgen05_commit2_both(xempty0 + 8 * xst);
+                        } else {
+                            tcgen05_commit(empty0 + 8 * s);
+                            if (xlast) tcgen05_commit(xempty0 + 8 * xst);
                         }
                     }
                     acc = 1u;
-                    if (xlast && ++xst == (1u << p.xst_sh)) xst = 0;
+                    if (xlast) xst = (xst + 1u) & xst_mask;
                     if (++s == (uint32_t)wbufs) { s = 0; ph ^= 1u; }
                 }
                 if (ok && lead) {
@@ -442,196 +455,228 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         }
     } else if (warp < 2 + NUM_DEQ_WARPS) {
         // ---- stage 2: dequantization of this CTA's channels --------------------------------------------
-        // lane = channel (a warp may only touch its quarter of the tensor-memory lanes); group grp takes every fourth
-        // k-block of the walk, so that it always works on the same weight buffers and sees each of their turns.  In a segment that is
-        // one k-block of every packed stage, always the same one.  The 128-byte swizzle of the packed boxes (16-byte
-        // piece XOR strip) puts the eight strips a warp reads on different banks.
+        // lane = channel (a warp may only touch its quarter of the tensor-memory lanes); group grp takes every fourth unit of
+        // the walk, four plane words of a channel per thread.  The 128-byte swizzle of the packed boxes (16-byte piece XOR
+        // strip) puts the eight strips a warp reads on different banks.
         const int quad = warp & 3, grp = (warp - 2) >> 2;
         const int strip = quad * 8 + (lane >> 2), c = lane & 3;
-        const int nblk = p.K / p.group, gshift = (p.group == 32) ? 5 : (p.group == 64) ? 6 : 7;
-        const uint32_t p_lane = smem_u32(p_tiles) + (uint32_t)strip * 128u + (uint32_t)c * 4u;
-        const uint32_t w_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + TMEM_W;
-        int pslot = 0;
-        uint32_t pph = 0u;
-        int s = grp;                                       // weight buffer of the group's next k-block and its parity
-        uint32_t ph = 0u;
-        uint32_t pos = 0, xc0 = 0;                         // k-blocks and activation stages of the segments before
-        while (ok && span.next(sg)) {
-            const int n = tile_ch0(sg.tile) + quad * 32 + lane;
-            const bool valid = n < p.N;
-            const __half *psc = p.scales + (size_t)(n >> 2) * nblk * 4 + c;
-            const uint16_t *pz = p.zeros + (size_t)(n >> 2) * nblk;
-            const int nkb = sg.kb1 - sg.kb0;
-            const int first = (int)((uint32_t)grp - pos) & (DEQ_GROUPS - 1);      // the group's k-block of a packed stage
-            pos += (uint32_t)nkb;
-            uint32_t piece[2];                             // byte offsets of its two plane words
+        const int nblk = p.K / p.group;
+        uint32_t p_src[4];                                 // the lane's plane words in the half of a packed stage its strip's swizzle puts first
 #pragma unroll
-            for (int w = 0; w < 2; ++w) piece[w] = (uint32_t)(((2 * first + w) ^ (strip & 7)) * 16);
-            // the block's scale and zero-point of each of the two words, fetched one k-block ahead
-            __half sv[2];
-            uint32_t zv[2];
-            auto fetch = [&](int i) {
+        for (int w = 0; w < 4; ++w) p_src[w] = (uint32_t)strip * 128u + (uint32_t)c * 4u + ((uint32_t)(w ^ (strip & 3)) * 16u);
+        const uint32_t half_swap = ((uint32_t)strip >> 2) & 1u;
+        const uint32_t w_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)p.wcol, xst_mask = (1u << p.xst_sh) - 1u;
+        // Weight buffer of the group's next unit and its parity.  All groups see every turn of what they wait for: a group's unit
+        // before this one is four back, its wait was for a commit six (four) units before that, and loads are issued in order;
+        // no ring is so short that an unseen turn could be two behind (six weight buffers only for tiles of four units and more).
+        uint32_t s = (uint32_t)grp, ph = 0u;
+        uint32_t pos = 0, xc0 = 0, pc0 = 0;                // units, activation stages and packed stages of the segments before
+        // BPU: quantization blocks of a unit
+        auto walk = [&](auto bpu_c) {
+            constexpr int BPU = decltype(bpu_c)::value;
+            while (ok && span.next(sg)) {
+                const int n = tile_ch0(sg.tile) + quad * 32 + lane;
+                // (LoadFull: the first group alone passes every unit's activations and weights on)
+                constexpr int STEP = V == kGemmLoadFull ? 1 : DEQ_GROUPS;
+                const int first = V == kGemmLoadFull ? (grp == 0 ? sg.u0 : sg.u1) : sg.u0 + ((int)((uint32_t)grp - pos) & (DEQ_GROUPS - 1));
+                const int units = sg.u1 - sg.u0;
+                pos += (uint32_t)units;
+                // scales and zero-points of a unit's blocks, fetched one turn ahead (channels past the last: of the last)
+                const int strip_n = min(n, p.N - 1) >> 2;
+                const __half *psc = p.scales + ((size_t)strip_n * nblk + (size_t)first * BPU) * 4 + c;
+                const uint16_t *pz = p.zeros + (size_t)strip_n * nblk + (size_t)first * BPU;
+                __half sv[BPU];
+                uint32_t zv[BPU];
+                auto fetch = [&]() {
 #pragma unroll
-                for (int w = 0; w < 2; ++w) {
-                    sv[w] = __float2half(0.f);
-                    zv[w] = 0u;
-                    if (valid && i < nkb && (w == 0 || gshift == 5)) {
-                        const int B = ((2 * (sg.kb0 + i) + w) * 32) >> gshift;
-                        sv[w] = __ldg(psc + (size_t)B * 4);
-                        zv[w] = __ldg(pz + B);
+                    for (int w = 0; w < BPU; ++w) {
+                        sv[w] = __ldg(psc + 4 * w);
+                        zv[w] = __ldg(pz + w);
                     }
-                }
-            };
-            fetch(first);
-            for (int i = first; i < nkb + first; i += DEQ_GROUPS) {       // one turn per packed stage; its last may have no k-block for this group
-                const bool has = i < nkb;
-                BlockConsts t0, t1;
-                __half s0 = sv[0], s1 = sv[0];
-                uint32_t z0 = (zv[0] >> (4 * c)) & 0xFu, z1 = z0;
-                if (gshift == 5) { s1 = sv[1]; z1 = (zv[1] >> (4 * c)) & 0xFu; }
-                t0.set(s0, z0);
-                t1.set(s1, z1);
-                if constexpr (V != kGemmLoadFull) {
-                    fetch(i + DEQ_GROUPS);
-                    if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(ploaded0 + 8 * pslot, pph))) { ok = false; break; }
-                }
-                uint32_t w[2][BITS];
-                if constexpr (V != kGemmLoadFull) {
-                    if (has) {
-                        const uint32_t src = p_lane + (uint32_t)pslot * P_STAGE_BYTES;
+                    psc += 4 * BPU * STEP;
+                    pz += BPU * STEP;
+                };
+                if (first < sg.u1) fetch();
+                for (int u = first; u < sg.u1; u += STEP) {
+                    const uint32_t i = (uint32_t)(u - sg.u0), xc = xc0 + (i >> p.xu_sh);
+                    const uint32_t xbar = xloaded0 + 8 * (xc & xst_mask), xpar = (xc >> p.xst_sh) & 1u;
+                    if constexpr (V != kGemmLoadFull) {
+                        BlockConsts t[BPU];
+                        __half s_cur[BPU];
+                        uint32_t z_cur[BPU];
 #pragma unroll
-                        for (int q = 0; q < 2; ++q)
+                        for (int w = 0; w < BPU; ++w) {
+                            s_cur[w] = sv[w];
+                            z_cur[w] = (zv[w] >> (4 * c)) & 0xFu;
+                            t[w].set(sv[w], z_cur[w]);
+                        }
+                        if (u + STEP < sg.u1) fetch();
+                        const uint32_t pc = pc0 + (i >> 1), ps = pc % P_STAGES;
+                        if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(ploaded0 + 8 * ps, (pc / P_STAGES) & 1u))) { ok = false; break; }
+                        uint32_t w4[4][BITS];
+                        const uint32_t stage = ps * P_STAGE_BYTES + (((i & 1u) ^ half_swap) << 6);
+#pragma unroll
+                        for (int w = 0; w < 4; ++w)
 #pragma unroll
                             for (int b = 0; b < BITS; ++b)
-                                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[q][b]) : "r"(src + piece[q] + b * P_PLANE_BYTES) : "memory");
-                    }
-                }
-                if (has) {
-                    // (the wait above it guarantees that the activation stage's turn before this one is over: see launch)
-                    const uint32_t xc = xc0 + ((uint32_t)i >> p.xkb_sh), xbar = xloaded0 + 8 * (xc & ((1u << p.xst_sh) - 1u)), xpar = (xc >> p.xst_sh) & 1u;
-                    if (!TMAN_STAMPED_WAIT(wait_b, mbar_wait(empty0 + 8 * s, ph ^ 1u))) { ok = false; break; }
-                    tcgen05_fence_after();
-                    if constexpr (V == kGemmSequential)
-                        if (!mbar_wait(xbar, xpar)) { ok = false; break; }
-                    if constexpr (V != kGemmLoadFull) {
-                        uint32_t out[16];
-                        if constexpr (V == kGemmConvertDq) dequant_word_convert<BITS>(w[0], s0, z0, out);
-                        else dequant_word<BITS>(w[0], t0, out);
-                        tcgen05_st_32x32b_x16(w_tmem + (uint32_t)(32 * s), out);
-                        if constexpr (V == kGemmConvertDq) dequant_word_convert<BITS>(w[1], s1, z1, out);
-                        else dequant_word<BITS>(w[1], t1, out);
-                        tcgen05_st_32x32b_x16(w_tmem + (uint32_t)(32 * s + 16), out);
+                                w4[w][b] = *reinterpret_cast<const uint32_t *>(smem + p_src[w] + stage + b * P_PLANE_BYTES);
+                        if (!TMAN_STAMPED_WAIT(wait_b, mbar_wait(empty0 + 8 * s, ph ^ 1u))) { ok = false; break; }
+                        tcgen05_fence_after();
+                        __syncwarp();
+                        if (lane == 0) {                                       // the packed words are in registers
+                            mbar_arrive(pempty0 + 8 * ps);
+                            if ((i & 1u) == 0u && u == sg.u1 - 1) mbar_arrive(pempty0 + 8 * ps);   // a last stage of one unit
+                        }
+                        if constexpr (V == kGemmSequential)
+                            if (!mbar_wait(xbar, xpar)) { ok = false; break; }
+                        const uint32_t dst = w_tmem + (uint32_t)W_COLS * s;
+#pragma unroll
+                        for (int w = 0; w < 4; ++w) {
+                            constexpr int WPB = 4 / BPU;
+                            uint32_t out[16];
+                            if constexpr (V == kGemmConvertDq) dequant_word_convert<BITS>(w4[w], s_cur[w / WPB], z_cur[w / WPB], out);
+                            else dequant_word<BITS>(w4[w], t[w / WPB], out);
+                            tcgen05_st_32x32b_x16(dst + (uint32_t)(16 * w), out);
+                        }
                         tcgen05_wait_st();
                     }
                     tcgen05_fence_before();
-                    // the MMA of this k-block also reads this CTA's activations
+                    // the MMA of this unit also reads this CTA's activations (their stage's turn before was over when the
+                    // weight buffer became free: their ring is no shorter than the weight buffers')
                     if (!TMAN_STAMPED_WAIT(wait_b, mbar_wait(xbar, xpar))) { ok = false; break; }
+                    __syncwarp();
+                    if (lane == 0) arrive_lead(full_lead + 8 * s);
+                    s += STEP;
+                    if (s >= (uint32_t)wbufs) { s -= (uint32_t)wbufs; ph ^= 1u; }
                 }
-                __syncwarp();
-                if (lane == 0) {
-                    if (has) arrive_lead(full_lead + 8 * s);
-                    if constexpr (V != kGemmLoadFull) mbar_arrive(pempty0 + 8 * pslot);
-                }
-                if (++pslot == PST) { pslot = 0; pph ^= 1u; }
-                if (has) {
-                    s += DEQ_GROUPS;                       // buffers: 8 or 4
-                    if (s >= wbufs) { s -= wbufs; ph ^= 1u; }
-                }
+                xc0 += (uint32_t)(units + (1 << p.xu_sh) - 1) >> p.xu_sh;
+                pc0 += (uint32_t)(units + 1) >> 1;
             }
-            xc0 += (uint32_t)(nkb + (1 << p.xkb_sh) - 1) >> p.xkb_sh;
-        }
+        };
+        if (p.group == 128) walk(IntC<1>());
+        else if (p.group == 64) walk(IntC<2>());
+        else walk(IntC<4>());
     } else {
         // ---- epilogue: this CTA's channels of a segment's accumulators ---------------------------------
-        // A warp reads chunks of 32 channels (one per lane) x 32 tokens.  Whole tiles and the finishing segment of a split
-        // tile: round to fp16; neighbouring lanes exchange every other token, so that a lane stores two adjacent channels
-        // of one token (4 bytes; a warp's store covers 64 bytes of two tokens).  Split tiles: the other segments write the
-        // fp32 accumulators to this CTA's partial tile ([token][channel]) and raise the warp's flag.  The finishing segment,
-        // always the last of its worker's walk, waits for the flags of the same warp in the workers before it and adds
-        // their sums in worker order.
+        // A warp has 32 channels (one per lane) x half of the tile's tokens.  Whole tiles: round to fp16; neighbouring lanes
+        // exchange every other token, so that a lane stores two adjacent channels of one token (4 bytes; a warp's store
+        // covers 64 bytes of two tokens).  Split tiles: a segment writes the fp32 accumulators that others sum to this CTA's
+        // partial tile and raises the warp's flag (of a span: all of them; of even pieces: all but its own share of the tokens,
+        // with a flag for each of the others).  Whoever sums waits for the flags of the same warp in the other workers, fetches
+        // their rows at once by bulk copies into the activation ring, which is idle by then (the finishing segment is the last
+        // of its worker's walk), and adds them to its own accumulators in worker order.  (Fetched by ordinary loads, a
+        // trip to L2 for every few of them, the sum made a call of 300 x 3584 x 4608 in two pieces take 25.8 us and one of 128 x 18944 x
+        // 3584 in five 31.6; this way 20.2 and 26.3.)
         const int quad = warp & 3;
-        const int ew = warp - 2 - NUM_DEQ_WARPS, epart = ew >> 2;
-        const int nchunks = (p.nt + 31) / 32;
-        auto partial_of = [&](int cta) { return p.partial + (size_t)cta * (kPartialBytesPerCta / 4) + quad * 32 + lane; };
-        auto warp_flag = [&](int cta) { return p.flags + (size_t)cta * NUM_EPI_WARPS + ew; };
+        const int ew = warp - 2 - NUM_DEQ_WARPS, half = p.nt >> 1, h0 = (ew >> 2) * half;
+        const uint32_t acc_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)h0;
         const bool odd = (lane & 1) != 0;
+        auto partial_of = [&](int cta) { return p.partial + (size_t)cta * (kPartialBytesPerCta / 4) + (size_t)(ew * half * 32); };
+        auto warp_flag = [&](int cta) { return p.flags + (size_t)cta * NUM_EPI_WARPS + ew; };
+        auto piece_flag = [&](int cta, int sender) { return p.piece_flags + ((size_t)cta * NUM_EPI_WARPS + ew) * kMaxSplit + sender; };
+        // (the loads before it stay inside the buffers whatever the header says; a header that does not match stops the stores)
+        const bool hdr_ok = header_matches(p.packed, p.K, p.N, p.bits, p.group);
+        if (!hdr_ok && lane == 0 && blockIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)TMAN_ERR_BAD_PACKED);
         uint32_t ti = 0;
         while (ok && span.next(sg)) {
-            const int row0 = tile_tm(sg.tile) * p.nt, n = tile_ch0(sg.tile) + quad * 32 + lane;
-            int first_w = worker;
-            if (sg.finishes && !sg.whole) first_w = span.owner(sg.tile, 0);
-            const int ncontrib = worker - first_w;
+            const int m0 = tile_tm(sg.tile) * p.nt + h0, n = tile_ch0(sg.tile) + quad * 32 + lane, left = min(half, p.M - m0);   // tokens to do (may be <= 0)
+            __half *y = p.y + (size_t)m0 * p.N + (n & ~1);
+            const bool put = n < p.N && hdr_ok;
+            // tokens t, t + 1 of this lane's channel -> two channels of one of the tokens
+            auto store2 = [&](int t, int end, float v0, float v1) {
+                const float keep = odd ? v1 : v0, send = odd ? v0 : v1;
+                const float got = __shfl_xor_sync(0xffffffffu, send, 1);
+                const __half2 h = odd ? __floats2half2_rn(got, keep) : __floats2half2_rn(keep, got);
+                const int tt = t + (odd ? 1 : 0);
+                if (tt < end && put) *reinterpret_cast<__half2 *>(y + (size_t)tt * p.N) = h;
+            };
             if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(accf, ti & 1u))) { ok = false; break; }
             tcgen05_fence_after();
-            if (ncontrib > 0) {
-                // their partial tiles were written at the start of their walks; bounded wait all the same
-                if (lane == 0) {
-                    for (int cw = first_w; cw < worker && ok; ++cw) {
-                        const uint32_t *f = warp_flag(cw * NCTA + (int)rank);
-                        uint64_t t0 = 0;
-                        for (uint32_t spin = 0;; ++spin) {
-                            uint32_t fv;
-                            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(fv) : "l"(f) : "memory");
-                            if (fv == 1u) break;
-                            if ((spin & 255u) == 255u) {
-                                const uint64_t now = global_timer_ns();
-                                if (t0 == 0) t0 = now;
-                                else if (now - t0 > 1000000000ull) { ok = false; break; }
-                            }
+            if (sg.whole) {
+#pragma unroll 1
+                for (int t = 0; t < left; t += 16) {
+                    uint32_t r[16];
+                    tcgen05_ld_32x32b_x16(acc_tmem + (uint32_t)t, r);
+                    tcgen05_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 16; e += 2) store2(t + e, left, __uint_as_float(r[e]), __uint_as_float(r[e + 1]));
+                }
+            } else {
+                const int S = p.split_s, me = S ? worker % S : 0;
+                // this worker's share of the sum
+                const int own0 = S ? min(half * me / S, left) : 0, own1 = S ? min(half * (me + 1) / S, left) : sg.finishes ? left : 0;
+                const int first_w = S ? worker - me : sg.finishes ? span.owner(sg.tile, 0) : worker;
+                const int senders = S ? S : worker - first_w;              // workers from first_w on, this one among even pieces
+                const bool other = lane < senders && first_w + lane != worker;
+                if (S || !sg.finishes) {
+                    float *mine = partial_of((int)blockIdx.x) + lane;
+#pragma unroll 1
+                    for (int t = 0; t < left; t += 8) {
+                        uint32_t r[8];
+                        tcgen05_ld_32x32b_x8(acc_tmem + (uint32_t)t, r);
+                        tcgen05_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if ((t + e < own0 || t + e >= own1) && t + e < left) __stcg(mine + (t + e) * 32, __uint_as_float(r[e]));
+                    }
+                    __threadfence();                       // every lane's stores, then the flags
+                    __syncwarp();
+                    uint32_t *to = S ? piece_flag((first_w + lane) * NCTA + (int)rank, me) : warp_flag((int)blockIdx.x);
+                    if (S ? other : lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(to), "r"(1u) : "memory");
+                }
+                if (senders > 0) {
+                    uint32_t *from = S ? piece_flag((int)blockIdx.x, lane) : warp_flag((first_w + lane) * NCTA + (int)rank);
+                    uint64_t t0 = 0;
+                    for (uint32_t spin = 0; other; ++spin) {
+                        uint32_t fv;
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(fv) : "l"(from) : "memory");
+                        if (fv == 1u) break;
+                        if ((spin & 255u) == 255u) {
+                            const uint64_t now = global_timer_ns();
+                            if (t0 == 0) t0 = now;
+                            else if (now - t0 > 1000000000ull) { ok = false; break; }
                         }
                     }
-                }
-                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-                if (!ok) break;
-            }
+                    ok = warp_all(ok);
+                    if (!ok) break;
+                    if (other) *from = kFlagEmpty;         // back to "empty" for the next launch
+                    asm volatile("fence.proxy.async;" ::: "memory");       // the others' stores, then the copies that read them
+                    const int slots = S ? S - 1 : senders, step = 128 / slots;            // 16 KB a warp: so many tokens of every sender at a time
+                    const float *src = partial_of((first_w + lane) * NCTA + (int)rank);
+                    const uint32_t bar = sums0 + 8 * ew, slot_off = (uint32_t)ew * 16384u;
+                    uint32_t par = 0;
 #pragma unroll 1
-            for (int q = epart; q < nchunks; q += 2) {
-                const int m0 = row0 + 32 * q, left = min(p.nt - 32 * q, p.M - m0);     // tokens of this chunk (may be <= 0)
-                uint32_t r[32];
-                tcgen05_ld_32x32b_x32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(32 * q), r);
-                tcgen05_wait_ld();
-                if (!sg.finishes) {
-                    float *dst = partial_of((int)blockIdx.x) + (size_t)(32 * q) * CH;
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (e < left) __stcg(dst + e * CH, __uint_as_float(r[e]));
-                    continue;
-                }
+                    for (int t0 = own0; t0 < own1; t0 += step) {
+                        const int cnt = min(step, own1 - t0);
+                        if (lane == 0) mbar_expect_tx(bar, (uint32_t)(slots * cnt) * 128u);
+                        __syncwarp();
+                        if (other)
+                            bulk_load(smem_u32(x_tiles) + slot_off + (uint32_t)((lane - (S && lane > me ? 1 : 0)) * cnt) * 128u, src + t0 * 32, (uint32_t)cnt * 128u, bar);
+                        ok = warp_all(mbar_wait(bar, par) || mbar_wait(bar, par));
+                        if (!ok) break;
+                        par ^= 1u;
 #pragma unroll 1
-                for (int cw = first_w; cw < worker; ++cw) {
-                    const float *src = partial_of(cw * NCTA + (int)rank) + (size_t)(32 * q) * CH;
+                        for (int t = 0; t < cnt; t += 8) {
+                            uint32_t r[8];
+                            tcgen05_ld_32x32b_x8(acc_tmem + (uint32_t)(t0 + t), r);
+                            tcgen05_wait_ld();
+                            const float *rows = reinterpret_cast<const float *>(x_tiles + slot_off) + t * 32 + lane;
+#pragma unroll 1
+                            for (int o = 0; o < slots; ++o, rows += cnt * 32)
 #pragma unroll
-                    for (int e0 = 0; e0 < 32; e0 += 16) {
-                        float a[16];
+                                for (int e = 0; e < 8; ++e)
+                                    if (t + e < cnt) r[e] = __float_as_uint(__uint_as_float(r[e]) + rows[e * 32]);
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) a[e] = (e0 + e < left) ? __ldcg(src + (e0 + e) * CH) : 0.f;
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) r[e0 + e] = __float_as_uint(__uint_as_float(r[e0 + e]) + a[e]);
+                            for (int e = 0; e < 8; e += 2) store2(t0 + t + e, t0 + cnt, __uint_as_float(r[e]), __uint_as_float(r[e + 1]));
+                        }
+                        __syncwarp();
                     }
-                }
-#pragma unroll
-                for (int e = 0; e < 32; e += 2) {
-                    const float keep = __uint_as_float(odd ? r[e + 1] : r[e]), send = __uint_as_float(odd ? r[e] : r[e + 1]);
-                    const float got = __shfl_xor_sync(0xffffffffu, send, 1);
-                    const __half2 h = odd ? __floats2half2_rn(got, keep) : __floats2half2_rn(keep, got);
-                    const int t = e + (odd ? 1 : 0);
-                    if (t < left && n < p.N) *reinterpret_cast<__half2 *>(p.y + (size_t)(m0 + t) * p.N + (n & ~1)) = h;
                 }
             }
             // the accumulators are read: the next segment's MMAs may start
             tcgen05_fence_before();
             __syncwarp();
             if (lane == 0) arrive_lead(acce_lead);
-            if (!sg.finishes) {
-                // partial tile complete: every lane's stores, then the flag
-                __threadfence();
-                __syncwarp();
-                if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(warp_flag((int)blockIdx.x)), "r"(1u) : "memory");
-            } else if (ncontrib > 0) {
-                // the partial tiles are consumed: their flags go back to "empty" for the next launch
-                __syncwarp();
-                if (lane == 0)
-                    for (int cw = first_w; cw < worker; ++cw) *warp_flag(cw * NCTA + (int)rank) = kFlagEmpty;
-            }
             ++ti;
         }
     }
@@ -660,12 +705,13 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
 
 // ---- host side ---------------------------------------------------------------------------
 // How a call's work is cut (host).  Pairs of CTAs beyond 16 tokens: a pair fetches an activation once per 256 channels and is
-// as fast or faster at every size measured (4-bit, group 128: 40 x 4096 x 14336 25.0 us against 26.4 with single CTAs, 128 x 3584
-// x 18944 25.1 / 26.2, 1024 x 4096 x 14336 96 / 108, 8192 x 18944 x 3584 775 / 873); up to 16 tokens a single CTA needs half
-// the columns.  The tokens go to as few tiles of at most 256 as hold them, or a few more where that deals out better; the time of
-// a k-block hardly falls below 96 tokens (the dequantization bounds it: 0.28 us at 40 tokens, 0.32 at 128) and follows the MMA
-// above (0.44 at 256).  Where whole tiles leave workers idle the k-blocks are split: in equal spans over the last tiles, or, for
-// few tiles, in even pieces; a split costs its tile's partial sums, written and read back, and another pipeline start.
+// as fast or faster at the sizes measured (4-bit, group 128: 40 x 4096 x 14336 18.7 us either way, 128 x 3584 x 18944 19.9
+// against 21.8 with single CTAs, 128 x 18944 x 3584 26.4 / 28.6; 2-bit, 128 x 3584 x 4608 16.0 / 15.8); up to 16 tokens a single CTA
+// needs half the columns.  The tokens go to as few tiles of at most 256 as hold them, or a few more where that deals out better;
+// a unit takes 0.41 us up to 128 tokens (the dequantization bounds it) and follows the MMA above (0.72 at 256).  Where whole
+// tiles leave workers idle the units are split: in equal spans over the last tiles, or, for few tiles, in even pieces; a
+// split costs 4 to 6 us for the partial sums, written, announced and read back (40 x 4096 x 14336: 56 whole tiles 18.7 us, spans
+// on 74 workers 21.5; 128 x 18944 x 3584 whole on 14 workers about 70, in five pieces 26.4).
 struct GemmPlan { int pair, nt, tiles_m, tiles_n, span_tiles, workers, col_fastest, split_s; };
 
 inline bool gemm_pair(int M) { return M > 16; }
@@ -677,18 +723,18 @@ GemmPlan plan_gemm(int M, int K, int N, int bits, int sms, int resident)
     GemmPlan g = {};
     const bool pair = gemm_pair(M);
     g.pair = pair ? 1 : 0;
-    const int ncta = pair ? 2 : 1, gran = pair ? 32 : 16, max_split = 32;
+    const int ncta = pair ? 2 : 1, gran = pair ? 32 : 16;
     const long long all = (sms < kMaxGemmCtas ? sms : kMaxGemmCtas) / ncta > 0 ? (sms < kMaxGemmCtas ? sms : kMaxGemmCtas) / ncta : 1;
     long long workers = all < resident ? all : resident;
     if (workers < 1) workers = 1;
-    const long long nu = K / (2 * BK);
+    const long long nu = K / UK;
     g.tiles_n = (N + CH * ncta - 1) / (CH * ncta);
     const bool may_split = nu * 2 * all * all < (1ll << 30);        // the spans' arithmetic is 32-bit
     // least time with tm tiles of tokens and w workers; fills in g
     auto cut = [&](int tm, long long w) {
         const int nt = ((M + tm - 1) / tm + gran - 1) / gran * gran, tiles_m = (M + nt - 1) / nt;
         const long long tiles = (long long)tiles_m * g.tiles_n;
-        const double lo = 0.26 + 0.0004 * nt, hi = 0.0017 * nt, unit = 2.0 * (lo > hi ? lo : hi), fix = 1.5;
+        const double lo = 0.40 + 0.0002 * nt, hi = 0.0028 * nt, unit = lo > hi ? lo : hi, fix = 1.2 + 0.007 * nt, sums = 3.5 + 0.012 * nt;
         double best = (double)((tiles + w - 1) / w) * (nu * unit + fix);
         g.nt = nt; g.tiles_m = tiles_m; g.span_tiles = 0; g.split_s = 0;
         auto take = [&](double cost, long long span, int split) {
@@ -699,10 +745,9 @@ GemmPlan plan_gemm(int M, int K, int N, int bits, int sms, int resident)
         // would be cut into many pieces per tile
         const long long rest = tiles % w, span = (rest != 0 && rest < w / 2 && tiles > w) ? rest + w : rest;
         if (span != 0 && 2 * tiles > w)                // (fewer tiles: even pieces, at most one tile a worker)
-            take((double)((tiles - span) / w) * (nu * unit + fix) + (double)((span * nu + w - 1) / w) * unit + fix + 2.8 +
-                     0.012 * nt * (double)w / (double)span, span, 0);
-        for (int S = 2; S <= max_split && tiles * S <= w && nu >= 2 * S; ++S)
-            take((double)((nu + S - 1) / S) * unit + fix + 2.5 + 0.012 * nt * (S - 1), tiles, S);
+            take((double)((tiles - span) / w) * (nu * unit + fix) + (double)((span * nu + w - 1) / w) * unit + fix + sums, span, 0);
+        for (int S = 2; S <= kMaxSplit && tiles * S <= w && nu >= 2 * S; ++S)
+            take((double)((nu + S - 1) / S) * unit + fix + sums + 0.8 * (S - 2), tiles, S);
         return best;
     };
     int tm_best = (M + MAX_TOKENS - 1) / MAX_TOKENS;
@@ -871,19 +916,14 @@ tman_status launch_mpgemm_variant(int variant, const void *packed, const void *x
     const int rows_cta = g.nt / (g.pair ? 2 : 1);
     const cuuint32_t estr[3] = {1, 1, 1};
 
-    // Activation stages: as many k-blocks as leave four stages or more in the ring, up to four (few rows: a load of one k-block
-    // would be small and the issuing thread the limit).  A weight buffer is written again when the MMA eight (four) k-blocks
-    // back has been committed; with XST stages of XKB k-blocks and 2 XST >= 8 (XKB = 1: buffers = XST = 4) the activation stage
-    // a k-block lies in has then been through its turn before, which a parity wait on it takes for granted.
-    const bool one_kb = variant == kGemmLoadFull || variant == kGemmSequential || rows_cta > 128;
-    const int xkb_sh = one_kb ? 0 : rows_cta > 64 ? 1 : 2;
-    const int xst_sh = one_kb ? 2 : (rows_cta << xkb_sh) * 128 * 8 <= X_RING_BYTES ? 3 : 2;
-    // activations as [k-block][token][64 k]: boxes of an activation stage x a CTA's token rows, 128-byte swizzle
+    const bool one_unit = variant == kGemmLoadFull || variant == kGemmSequential || rows_cta > 64;
+    const int p_xu_sh = one_unit ? 0 : 1;
+    // activations as [k-block][token][64 k]: boxes of one or two units x a CTA's token rows, 128-byte swizzle
     CUtensorMap tmap_x;
     {
         const cuuint64_t dims[3] = {(cuuint64_t)BK, (cuuint64_t)M, (cuuint64_t)(K / BK)};
         const cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)BK * 2};
-        const cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)rows_cta, (cuuint32_t)(1 << xkb_sh)};
+        const cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)rows_cta, (cuuint32_t)(UK / BK << p_xu_sh)};
         if (enc(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void *>(x), dims, strides, box, estr,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -892,13 +932,13 @@ tman_status launch_mpgemm_variant(int variant, const void *packed, const void *x
     Layout L = make_layout(K, N, bits, group);
     const uint8_t *pk = static_cast<const uint8_t *>(packed);
     // the bit-plane words as a 3-D array of 32-bit elements: (word and column inside a strip's plane
-    // row, plane, strip); one box = the eight words of four k-blocks for the strips of a CTA's channels, one plane
+    // row, plane, strip); one box = the eight words of two units for the strips of a CTA's channels, one plane
     CUtensorMap tmap_w;
     {
         const cuuint64_t wt = (cuuint64_t)(K / 32);
         const cuuint64_t wdims[3] = {wt * 4, (cuuint64_t)bits, (cuuint64_t)(N / 4)};
         const cuuint64_t wstrides[2] = {wt * 16, wt * 16 * (cuuint64_t)bits};
-        const cuuint32_t wbox[3] = {(cuuint32_t)(P_KB * BK / 8), 1, (cuuint32_t)(CH / 4)};
+        const cuuint32_t wbox[3] = {(cuuint32_t)(2 * UK / 8), 1, (cuuint32_t)(CH / 4)};
         if (enc(&tmap_w, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint8_t *>(pk + L.planes_off), wdims, wstrides,
                 wbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -913,18 +953,25 @@ tman_status launch_mpgemm_variant(int variant, const void *packed, const void *x
     p.y = static_cast<__half *>(y);
     p.status = reinterpret_cast<uint32_t *>(w8);
     p.flags = reinterpret_cast<uint32_t *>(w8 + kGemmFlagsOff);
+    p.piece_flags = reinterpret_cast<uint32_t *>(w8 + kGemmPieceFlagsOff);
     p.partial = reinterpret_cast<float *>(w8 + kGemmPartialOff);
     p.M = M; p.K = K; p.N = N; p.bits = bits; p.group = group;
     p.nt = g.nt;
-    p.wbufs = one_kb ? 4 : 8;
-    p.xkb_sh = xkb_sh;
-    p.xst_sh = xst_sh;
+    // Tensor memory: behind an accumulator of up to 128 columns there is room for six weight buffers, behind 256 for four.
+    // (LoadFull: two activation stages, with their weight tiles in the packed ring beside them.)
+    const bool six = g.nt <= 128 && K >= 4 * UK && variant == kGemmProduct;
+    p.wbufs = variant == kGemmLoadFull ? 2 : six ? 6 : 4;
+    p.wcol = g.nt <= 128 ? 128 : 256;
+    p.xu_sh = p_xu_sh;
+    p.xst_sh = variant == kGemmLoadFull ? 1 : 3;
+    while ((rows_cta * 256 << p.xu_sh << p.xst_sh) > X_RING_BYTES) --p.xst_sh;
     p.tiles_m = g.tiles_m;
     p.tiles_n = g.tiles_n;
     p.span_tiles = g.span_tiles;
+    p.split_s = g.split_s;
     p.col_fastest = g.col_fastest;
     p.stamps = reinterpret_cast<long long *>(w8 + kGemmPartialOff + (size_t)kMaxGemmCtas * kPartialBytesPerCta);
-    // the fp16 weights [N][K]: boxes of one k-block x a CTA's channels, 128-byte swizzle; unused maps are copies of the activation map
+    // the fp16 weights [N][K]: boxes of half a unit x a CTA's channels, 128-byte swizzle; unused maps are copies of the activation map
     CUtensorMap tmap_wf = tmap_x;
     if (variant == kGemmLoadFull) {
         const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)N};

@@ -108,6 +108,30 @@ def test_split_tile_cases(M, K, N, bits, G):
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[1], ys[2])   # fixed summation order: same bits
 
 
+# Even pieces that share the summing: 8 and 13 pieces, shares of no, one and some tokens, a warp without tokens (1 and 9 of a tile
+# of 16), a ragged last tile; spans of single CTAs and of pairs.
+SHARED = [(1, 16384, 128, 4, 128), (9, 32768, 264, 2, 64), (17, 16384, 256, 4, 32), (250, 32768, 136, 4, 128)]
+
+
+@pytest.mark.parametrize("M,K,N,bits,G", SHARED + [(2, 4096, 19200, 4, 64), (40, 8192, 10000, 3, 128)])
+def test_shared_sums(M, K, N, bits, G):
+    plan = B.tman_debug_gemm_plan(M, K, N, bits, G)
+    assert plan["pieces"] >= 8 or plan["span_tiles"] > 0, plan
+    # rounding as in test_edges_of_the_transposed_kernel
+    c = synth.small_case(M, K, N, bits, G, seed=7 * M + K + N + bits)
+    dev = H.device_case(c)
+    packed = H.pack_case(c, dev)
+    ws = H.alloc_workspace(B.OP_GEMM, c.M, c.K, c.N, c.bits, c.group)
+    ys = [H.alloc_y(c.M, c.N) for _ in range(3)]
+    for y in ys:
+        B.tman_mpgemm(packed, dev["x"], y, c.M, c.K, c.N, c.bits, c.group, ws)
+    assert B.tman_read_status(ws) == 0
+    assert torch.equal(ys[0], ys[1]) and torch.equal(ys[1], ys[2])
+    rows = np.random.default_rng(0).permutation(M)[:20]           # (the oracle is slow)
+    ref = orc.mpgemm(c.x[rows], c.codes, c.scales, c.zeros, c.group)
+    assert rel_err(H.to_f64(ys[0])[rows], ref) <= 1e-3
+
+
 @pytest.mark.parametrize("M,K,N,bits,G", SPANS)
 def test_span_cases(M, K, N, bits, G):
     plan = B.tman_debug_gemm_plan(M, K, N, bits, G)
