@@ -15,6 +15,7 @@
 // magnitude lies in [2^14, 2^15); sums are fp32 throughout.  Zero-point and scale are applied to a block's sum:
 // s * (sum - z * sum of the activations).
 #pragma once
+#include "sm100_ptx.cuh"
 #include "common.cuh"
 
 namespace tman {
@@ -45,7 +46,6 @@ struct MmaParams {
     int tk, tc, nkappa;                      // warps of a team (4, 8 or 16), teams of a CTA, K-slices
 };
 
-__device__ __forceinline__ uint32_t bsel(uint32_t m, uint32_t a, uint32_t b) { return (a & m) | (b & ~m); }
 __device__ __forceinline__ uint32_t rotl(uint32_t v, int n) { return __funnelshift_l(v, v, n); }
 __device__ __forceinline__ uint32_t rotr(uint32_t v, int n) { return __funnelshift_r(v, v, n); }
 __device__ __forceinline__ uint32_t comp(const uint4 &v, int c) { return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w; }

@@ -153,7 +153,6 @@ __device__ __forceinline__ void dequant_word(const uint32_t (&w)[BITS], const Bl
     // bit-block transpose of the plane words: first planes 0/1 and 2/3 are interleaved bit by bit,
     // then the two results two bits by two bits (each step is one shift and one bit-select).  Bits of a
     // nibble above the code are left over from its neighbours; the mask below drops them.
-    auto bsel = [](uint32_t m, uint32_t a, uint32_t b) { return (a & m) | (b & ~m); };
     uint32_t X[4];
     {
         const uint32_t a0 = bsel(0x55555555u, w[0], w[1] << 1), a1 = bsel(0x55555555u, w[0] >> 1, w[1]);
@@ -705,10 +704,10 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
 
 // ---- host side ---------------------------------------------------------------------------
 // How a call's work is cut (host).  Pairs of CTAs beyond 16 tokens: a pair fetches an activation once per 256 channels and is
-// as fast or faster at the sizes measured (4-bit, group 128: 40 x 4096 x 14336 18.7 us either way, 128 x 3584 x 18944 19.9
+// as fast or faster at the sizes measured (4-bit, group 128: 40 x 4096 x 14336 18.1 us either way, 128 x 3584 x 18944 19.9
 // against 21.8 with single CTAs, 128 x 18944 x 3584 26.4 / 28.6; 2-bit, 128 x 3584 x 4608 16.0 / 15.8); up to 16 tokens a single CTA
 // needs half the columns.  The tokens go to as few tiles of at most 256 as hold them, or a few more where that deals out better;
-// a unit takes 0.41 us up to 128 tokens (the dequantization bounds it) and follows the MMA above (0.72 at 256).  Where whole
+// a unit takes 0.39 us up to 128 tokens (the dequantization bounds it) and follows the MMA above (0.72 at 256).  Where whole
 // tiles leave workers idle the units are split: in equal spans over the last tiles, or, for few tiles, in even pieces; a
 // split costs 4 to 6 us for the partial sums, written, announced and read back (40 x 4096 x 14336: 56 whole tiles 18.7 us, spans
 // on 74 workers 21.5; 128 x 18944 x 3584 whole on 14 workers about 70, in five pieces 26.4).

@@ -809,10 +809,10 @@ static const GemvVariant kGemvVariants[kGemvVariantCount] = {
 
 // Whether a pass of `rows` rows goes to the tensor-core kernel (decode_mma.cuh) instead of the table lookups.  From five
 // rows always: an entry of eight fp16 rows costs four shared-memory wavefronts a lookup (4-bit 4096 x 28672, group 128:
-// 42.0 us by lookup, 23.1 us here; 2-bit, group 64: 29.8 / 22.4; 4-bit, group 32: 42.5 / 32.9).  With three and four rows
+// 42.0 us by lookup, 21.3 us here; 3-bit, group 64: 24.3).  With three and four rows
 // (two wavefronts) where a lookup per plane is many of them and the blocks are no shorter than two words: 4-bit, group 128
-// 23.8 / 20.5, 3-bit, group 64 20.2 / 20.0 (4096 x 4096: 7.4 / 6.8), but 2-bit, group 64 17.3 / 18.3 and 4-bit, group 32
-// 24.0 / 31.6.  One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.3 / 20.1).
+// 23.8 / 18.9, 3-bit, group 64 20.2 / 18.9 (4096 x 4096: 7.4 / 6.6), but 2-bit, group 64 17.2 / 18.1 and 4-bit, group 32
+// 24.0 / 31.2.  One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.2 / 18.4).
 static bool uses_mma(int bits, int group, int rows) { return rows >= 5 || (rows >= 3 && bits >= 3 && group >= 64); }
 
 static size_t variant_ws_bytes(const GemvVariant &v, int K, int N)
