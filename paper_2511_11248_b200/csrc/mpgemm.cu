@@ -13,6 +13,8 @@
 // pairs, at most one per SM or SM pair), whole as far as they go round; where whole tiles would leave SMs idle, the
 // units of the last tiles are laid end to end and dealt in equal spans, and a tile whose units fall into several
 // spans is summed through fp32 partial tiles in the workspace (see "split of the work").
+// The integer path (per-tensor ternary weights, INT8 activations; paper Sec. 6.2) is the same kernel with kind::i8: codes become
+// bytes by a table lookup, sums are exact 32-bit integers, the epilogue applies the token's and the tensor's scale.
 // Four kinds of agents run concurrently, guarded by mbarriers (the paper's DMA / vector-core / matrix-core stages):
 //   * warp 0, one lane : TMA loads of the activations (a ring of units, 128-byte swizzle) and, running ahead on a ring of its own, of the
 //                        packed bit-plane words (runs of 128 bytes per strip and plane);
@@ -49,7 +51,6 @@ constexpr int P_RING_BYTES = 64 * 1024;         // 8 stages for 2 bits, 4 for 3 
 constexpr int X_RING_BYTES = 128 * 1024;        // activation ring: stages of two units (8 of up to 32 rows, 4 of up to 64) or one (4 of up to 128)
 constexpr int W_TILE_BYTES = CH * BK * 2;       // half a unit of fp16 weights in shared memory (LoadFull variant only)
 constexpr int TMEM_COLS = 512;                  // accumulator from column 0, weight buffers of 64 columns behind it
-constexpr int W_COLS = UK / 2;
 constexpr int kMaxGemmCtas = 160;               // the workspace is sized for at most this many CTAs
 constexpr int GEMM_SMEM = P_RING_BYTES + X_RING_BYTES + 512;
 
@@ -92,6 +93,9 @@ struct GemmParams {
     int span_tiles;            // the last span_tiles tiles are dealt as equal spans of units (0: every tile whole)
     int split_s;               // even pieces of every tile (0: not split so)
     int col_fastest;           // tile number = row tile * tiles_n + column tile (else column tile * tiles_m + row tile)
+    int acc_sh, acc_col;       // log2 of the accumulators in tensor memory (two: the epilogue of a tile overlaps the next one), their distance in columns
+    const float *row_scale;    // integer path: scales of the tokens and of the tensor
+    float w_scale;
     long long *stamps;         // role time stamps (written only by a build with TMAN_ROLE_STAMPS)
 };
 
@@ -100,6 +104,7 @@ struct GemmParams {
 constexpr int kGemmProduct = 0;      // the product path, pipelined
 constexpr int kGemmConvertDq = 1;    // codes converted to floating point one by one, then subtract and multiply
 constexpr int kGemmLoadFull = 2;     // fp16 weights prepared in memory and loaded by TMA, no dequantization
+constexpr int kGemmInt8 = 4;         // integer path: ternary weights as 8-bit integers, 8-bit activations, exact 32-bit sums (2-bit codes, whole tiles)
 constexpr int kGemmSequential = 3;   // the product's dequantization; a unit is loaded when the one before it has been multiplied, and dequantized when it is loaded
 
 template <int I> struct IntC { static constexpr int value = I; };
@@ -187,6 +192,20 @@ __device__ __forceinline__ void dequant_word(const uint32_t (&w)[BITS], const Bl
         }
 }
 
+// 32 ternary weights of one channel (2-bit codes, zero-point 1) -> 32 INT8 in k order (level 1 as above; level 2 looks four codes
+// at a time up in a four-entry byte table with one byte permute).
+__device__ __forceinline__ void dequant_word_int8(const uint32_t (&w)[2], uint32_t *out)
+{
+    const uint32_t table = 0x000100FFu;          // -1, 0, +1; (3 does not occur) 0
+    const uint32_t a0 = bsel(0x55555555u, w[0], w[1] << 1), a1 = bsel(0x55555555u, w[0] >> 1, w[1]);
+    const uint32_t X[4] = {a0 & 0x33333333u, a1 & 0x33333333u, (a0 >> 2) & 0x33333333u, (a1 >> 2) & 0x33333333u};
+#pragma unroll
+    for (int ph = 0; ph < 4; ++ph) {
+        out[2 * ph] = __byte_perm(table, 0u, X[ph]);
+        out[2 * ph + 1] = __byte_perm(table, 0u, X[ph] >> 16);
+    }
+}
+
 // ---- split of the work ----------------------------------------------------------------------
 // T tiles (row tile fastest), W workers.  The first `whole` tiles (a multiple of W) are dealt whole,
 // round-robin.  The units of the remaining tiles (fewer than 2 W), laid end to end (a unit is as deep as the
@@ -259,6 +278,8 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
               const __grid_constant__ CUtensorMap tmap_wf, const GemmParams p)
 {
     constexpr int NCTA = PAIR ? 2 : 1;
+    constexpr bool INT8 = V == kGemmInt8;
+    constexpr int W_COLS = INT8 ? UK / 4 : UK / 2, X_UNIT_ROW = INT8 ? UK : 2 * UK;   // a unit: columns of weights, bytes of a token
     constexpr int P_STAGE_BYTES = BITS * P_PLANE_BYTES, P_STAGES = BITS == 2 ? 8 : 4;
     extern __shared__ __align__(1024) uint8_t smem[];
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;   // in a pair, CTA 0 issues the MMAs and owns the shared barriers
@@ -268,7 +289,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
     // buffer ready (the four warps of a group; in a pair both CTAs' in CTA 0) / free (MMA commit); accumulator full (commit) /
     // empty (epilogue warps; in a pair both CTAs' in CTA 0)
     const uint32_t ploaded0 = smem_u32(bars), pempty0 = smem_u32(bars + 8), xloaded0 = smem_u32(bars + 16), xempty0 = smem_u32(bars + 24),
-                   full0 = smem_u32(bars + 32), empty0 = smem_u32(bars + 40), accf = smem_u32(bars + 48), acce = smem_u32(bars + 49);
+                   full0 = smem_u32(bars + 32), empty0 = smem_u32(bars + 40), accf0 = smem_u32(bars + 48), acce0 = smem_u32(bars + 60);
     const uint32_t sums0 = smem_u32(bars + 52);            // partial sums of an epilogue warp loaded
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 50);
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (the shuffle tells the compiler that it is uniform)
@@ -286,8 +307,10 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
             mbar_init(empty0 + 8 * s, 1);
             mbar_init(sums0 + 8 * s, 1);
         }
-        mbar_init(accf, 1);
-        mbar_init(acce, NCTA * NUM_EPI_WARPS);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(accf0 + 8 * b, 1);
+            mbar_init(acce0 + 8 * b, NCTA * NUM_EPI_WARPS);
+        }
         *tmem_slot = 0xFFFFFFFFu;
         fence_barrier_init();
     } else if (threadIdx.x == 32 * 2) {
@@ -329,7 +352,8 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
     auto tile_tm = [&](int tile) { return p.col_fastest ? tile / p.tiles_n : tile % p.tiles_m; };
     auto tile_ct = [&](int tile) { return p.col_fastest ? tile % p.tiles_n : tile / p.tiles_m; };
     auto tile_ch0 = [&](int tile) { return tile_ct(tile) * (NCTA * CH) + (int)rank * CH; };      // this CTA's first channel
-    const uint32_t full_lead = PAIR ? mapa_u32(full0, 0) : full0, acce_lead = PAIR ? mapa_u32(acce, 0) : acce;
+    const uint32_t full_lead = PAIR ? mapa_u32(full0, 0) : full0, acce_lead = PAIR ? mapa_u32(acce0, 0) : acce0;
+    const uint32_t acc_mask = (1u << p.acc_sh) - 1u;   // tile ti of the walk: accumulator ti & acc_mask, its barriers' turn ti >> acc_sh
     auto arrive_lead = [&](uint32_t bar) {
         if constexpr (PAIR) mbar_arrive_cluster(bar);
         else mbar_arrive(bar);
@@ -343,7 +367,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         // stage a unit needs, further packed stages as far as their ring has room, the activations.  What a load needs
         // is worked out once a segment: a division per load made this thread the slowest agent (0.6 us per 64 k).
         const bool lead = elect_one();
-        const uint32_t x_stage_bytes = (uint32_t)rows_cta * 256u << p.xu_sh;
+        const uint32_t x_stage_bytes = (uint32_t)(rows_cta * X_UNIT_ROW) << p.xu_sh;
         const uint32_t p_base = smem_u32(p_tiles), x_base = smem_u32(x_tiles), xst_mask = (1u << p.xst_sh) - 1u;
         const int xu = 1 << p.xu_sh;
         Span ps = span;
@@ -388,7 +412,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                 if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(xempty0 + 8 * st, ((xc >> p.xst_sh) & 1u) ^ 1u)))) { ok = false; break; }
                 if (lead) {
                     mbar_expect_tx(bar, x_stage_bytes + (V == kGemmLoadFull ? 2 * W_TILE_BYTES : 0));
-                    tma_load_3d(x_base + st * x_stage_bytes, &tmap_x, 0, row0, 2 * u, bar);
+                    tma_load_3d(x_base + st * x_stage_bytes, &tmap_x, 0, row0, INT8 ? u : 2 * u, bar);
                     if constexpr (V == kGemmLoadFull) {
                         tma_load_2d(p_base + st * (2 * W_TILE_BYTES), &tmap_wf, u * UK, ch0, bar);
                         tma_load_2d(p_base + st * (2 * W_TILE_BYTES) + W_TILE_BYTES, &tmap_wf, u * UK + BK, ch0, bar);
@@ -401,35 +425,40 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         // (the warp walks as one, so that the operands of the MMAs sit in uniform registers; an elected lane issues)
         if (rank == 0) {
             const bool lead = elect_one();
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(p.nt >> 3) << 17) | ((uint32_t)((NCTA * CH) >> 4) << 24);
+            // (integer path: s32 sums of s8 x s8; else fp32 sums of fp16 x fp16)
+            const uint32_t idesc = (INT8 ? (2u << 4) | (1u << 7) | (1u << 10) : 1u << 4) | ((uint32_t)(p.nt >> 3) << 17) | ((uint32_t)((NCTA * CH) >> 4) << 24);
             // descriptors in 16-byte units: only the low word (start address) changes
             const uint64_t bdesc0 = make_kmajor_sw128_desc(smem_u32(x_tiles)), adesc0 = make_kmajor_sw128_desc(smem_u32(p_tiles));
             const uint32_t half_units = (uint32_t)rows_cta * 8u, xst_mask = (1u << p.xst_sh) - 1u;
             const int xu_mask = (1 << p.xu_sh) - 1;
             uint32_t ti = 0, ph = 0u, s = 0, xst = 0;
             while (ok && span.next(sg)) {
-                if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(acce, (ti & 1u) ^ 1u)))) { ok = false; break; }
+                if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(acce0 + 8 * (ti & acc_mask), ((ti >> p.acc_sh) & 1u) ^ 1u)))) { ok = false; break; }
                 tcgen05_fence_after();
+                const uint32_t acc_tmem = tmem_base + (uint32_t)p.acc_col * (ti & acc_mask), accf = accf0 + 8 * (ti & acc_mask);
                 uint32_t acc = 0u;
                 for (int u = sg.u0; u < sg.u1; ++u) {
                     if (!TMAN_STAMPED_WAIT(wait_b, warp_all(mbar_wait(full0 + 8 * s, ph)))) { ok = false; break; }
                     tcgen05_fence_after();
                     const int xi = (u - sg.u0) & xu_mask;                  // unit of the activation stage
                     const bool xlast = xi == xu_mask || u == sg.u1 - 1;
-                    const uint64_t bdesc = bdesc0 + 2u * ((xst << p.xu_sh) + (uint32_t)xi) * half_units;
+                    const uint64_t bdesc = bdesc0 + (INT8 ? 1u : 2u) * ((xst << p.xu_sh) + (uint32_t)xi) * half_units;
                     const uint64_t adesc = adesc0 + xst * (2 * W_TILE_BYTES / 16);
                     const uint32_t wt = tmem_base + (uint32_t)p.wcol + (uint32_t)W_COLS * s;
                     if (lead) {
 #pragma unroll
-                        for (int j = 0; j < UK / 16; ++j) {
+                        for (int j = 0; j < (INT8 ? UK / 32 : UK / 16); ++j) {
                             const uint64_t bd = bdesc + 2 * (j & 3) + (j >> 2) * half_units;
-                            if constexpr (V == kGemmLoadFull) {
+                            if constexpr (INT8) {
+                                if constexpr (PAIR) tcgen05_mma2_i8_ts(acc_tmem, wt + 8 * j, bd, idesc, acc);
+                                else tcgen05_mma_i8_ts(acc_tmem, wt + 8 * j, bd, idesc, acc);
+                            } else if constexpr (V == kGemmLoadFull) {
                                 const uint64_t ad = adesc + 2 * (j & 3) + (j >> 2) * (W_TILE_BYTES / 16);
-                                if constexpr (PAIR) tcgen05_mma2_f16(tmem_base, ad, bd, idesc, acc);
-                                else tcgen05_mma_f16(tmem_base, ad, bd, idesc, acc);
+                                if constexpr (PAIR) tcgen05_mma2_f16(acc_tmem, ad, bd, idesc, acc);
+                                else tcgen05_mma_f16(acc_tmem, ad, bd, idesc, acc);
                             } else {
-                                if constexpr (PAIR) tcgen05_mma2_f16_ts(tmem_base, wt + 8 * j, bd, idesc, acc);
-                                else tcgen05_mma_f16_ts(tmem_base, wt + 8 * j, bd, idesc, acc);
+                                if constexpr (PAIR) tcgen05_mma2_f16_ts(acc_tmem, wt + 8 * j, bd, idesc, acc);
+                                else tcgen05_mma_f16_ts(acc_tmem, wt + 8 * j, bd, idesc, acc);
                             }
                             acc = 1u;
                         }
@@ -495,7 +524,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                     psc += 4 * BPU * STEP;
                     pz += BPU * STEP;
                 };
-                if (first < sg.u1) fetch();
+                if (!INT8 && first < sg.u1) fetch();
                 for (int u = first; u < sg.u1; u += STEP) {
                     const uint32_t i = (uint32_t)(u - sg.u0), xc = xc0 + (i >> p.xu_sh);
                     const uint32_t xbar = xloaded0 + 8 * (xc & xst_mask), xpar = (xc >> p.xst_sh) & 1u;
@@ -505,11 +534,12 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                         uint32_t z_cur[BPU];
 #pragma unroll
                         for (int w = 0; w < BPU; ++w) {
+                            if constexpr (INT8) continue;
                             s_cur[w] = sv[w];
                             z_cur[w] = (zv[w] >> (4 * c)) & 0xFu;
                             t[w].set(sv[w], z_cur[w]);
                         }
-                        if (u + STEP < sg.u1) fetch();
+                        if (!INT8 && u + STEP < sg.u1) fetch();
                         const uint32_t pc = pc0 + (i >> 1), ps = pc % P_STAGES;
                         if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(ploaded0 + 8 * ps, (pc / P_STAGES) & 1u))) { ok = false; break; }
                         uint32_t w4[4][BITS];
@@ -529,6 +559,15 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                         if constexpr (V == kGemmSequential)
                             if (!mbar_wait(xbar, xpar)) { ok = false; break; }
                         const uint32_t dst = w_tmem + (uint32_t)W_COLS * s;
+                        if constexpr (INT8) {
+#pragma unroll
+                            for (int w = 0; w < 4; w += 2) {
+                                uint32_t out[16];
+                                dequant_word_int8(w4[w], out);
+                                dequant_word_int8(w4[w + 1], out + 8);
+                                tcgen05_st_32x32b_x16(dst + (uint32_t)(8 * w), out);
+                            }
+                        } else
 #pragma unroll
                         for (int w = 0; w < 4; ++w) {
                             constexpr int WPB = 4 / BPU;
@@ -552,7 +591,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                 pc0 += (uint32_t)(units + 1) >> 1;
             }
         };
-        if (p.group == 128) walk(IntC<1>());
+        if (INT8 || p.group == 128) walk(IntC<1>());
         else if (p.group == 64) walk(IntC<2>());
         else walk(IntC<4>());
     } else {
@@ -568,7 +607,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         // 3584 in five 31.6; this way 20.2 and 26.3.)
         const int quad = warp & 3;
         const int ew = warp - 2 - NUM_DEQ_WARPS, half = p.nt >> 1, h0 = (ew >> 2) * half;
-        const uint32_t acc_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)h0;
+        const uint32_t acc0_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)h0;
         const bool odd = (lane & 1) != 0;
         auto partial_of = [&](int cta) { return p.partial + (size_t)cta * (kPartialBytesPerCta / 4) + (size_t)(ew * half * 32); };
         auto warp_flag = [&](int cta) { return p.flags + (size_t)cta * NUM_EPI_WARPS + ew; };
@@ -581,26 +620,35 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
             const int m0 = tile_tm(sg.tile) * p.nt + h0, n = tile_ch0(sg.tile) + quad * 32 + lane, left = min(half, p.M - m0);   // tokens to do (may be <= 0)
             __half *y = p.y + (size_t)m0 * p.N + (n & ~1);
             const bool put = n < p.N && hdr_ok;
-            // tokens t, t + 1 of this lane's channel -> two channels of one of the tokens
-            auto store2 = [&](int t, int end, float v0, float v1) {
-                const float keep = odd ? v1 : v0, send = odd ? v0 : v1;
-                const float got = __shfl_xor_sync(0xffffffffu, send, 1);
-                const __half2 h = odd ? __floats2half2_rn(got, keep) : __floats2half2_rn(keep, got);
+            // sums of tokens t, t + 1 of this lane's channel -> two channels of one of the tokens
+            auto store2 = [&](int t, int end, uint32_t v0, uint32_t v1, float sc = 0.f) {
+                const uint32_t keep = odd ? v1 : v0, got = __shfl_xor_sync(0xffffffffu, odd ? v0 : v1, 1);
+                const uint32_t c0 = odd ? got : keep, c1 = odd ? keep : got;
+                __half2 h;
+                if constexpr (INT8) h = __floats2half2_rn((float)(int)c0 * sc, (float)(int)c1 * sc);
+                else h = __floats2half2_rn(__uint_as_float(c0), __uint_as_float(c1));
                 const int tt = t + (odd ? 1 : 0);
                 if (tt < end && put) *reinterpret_cast<__half2 *>(y + (size_t)tt * p.N) = h;
             };
-            if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(accf, ti & 1u))) { ok = false; break; }
+            const uint32_t acc_b = ti & acc_mask;
+            if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(accf0 + 8 * acc_b, (ti >> p.acc_sh) & 1u))) { ok = false; break; }
             tcgen05_fence_after();
+            const uint32_t acc_tmem = acc0_tmem + (uint32_t)p.acc_col * acc_b;
             if (sg.whole) {
 #pragma unroll 1
                 for (int t = 0; t < left; t += 16) {
                     uint32_t r[16];
                     tcgen05_ld_32x32b_x16(acc_tmem + (uint32_t)t, r);
+                    float sc[8];
+                    if constexpr (INT8) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) sc[e] = __ldg(p.row_scale + min(m0 + t + 2 * e + (odd ? 1 : 0), p.M - 1)) * p.w_scale;
+                    }
                     tcgen05_wait_ld();
 #pragma unroll
-                    for (int e = 0; e < 16; e += 2) store2(t + e, left, __uint_as_float(r[e]), __uint_as_float(r[e + 1]));
+                    for (int e = 0; e < 8; ++e) store2(t + 2 * e, left, r[2 * e], r[2 * e + 1], INT8 ? sc[e] : 0.f);
                 }
-            } else {
+            } else if constexpr (!INT8) {
                 const int S = p.split_s, me = S ? worker % S : 0;
                 // this worker's share of the sum
                 const int own0 = S ? min(half * me / S, left) : 0, own1 = S ? min(half * (me + 1) / S, left) : sg.finishes ? left : 0;
@@ -666,7 +714,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                                 for (int e = 0; e < 8; ++e)
                                     if (t + e < cnt) r[e] = __float_as_uint(__uint_as_float(r[e]) + rows[e * 32]);
 #pragma unroll
-                            for (int e = 0; e < 8; e += 2) store2(t0 + t + e, t0 + cnt, __uint_as_float(r[e]), __uint_as_float(r[e + 1]));
+                            for (int e = 0; e < 8; e += 2) store2(t0 + t + e, t0 + cnt, r[e], r[e + 1]);
                         }
                         __syncwarp();
                     }
@@ -675,7 +723,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
             // the accumulators are read: the next segment's MMAs may start
             tcgen05_fence_before();
             __syncwarp();
-            if (lane == 0) arrive_lead(acce_lead);
+            if (lane == 0) arrive_lead(acce_lead + 8 * acc_b);
             ++ti;
         }
     }
@@ -771,6 +819,20 @@ GemmPlan plan_gemm(int M, int K, int N, int bits, int sms, int resident)
         g.col_fastest = (rows_c * a_tile + cols_c * b_tile < rows_r * a_tile + cols_r * b_tile) ? 1 : 0;
     }
     return g;
+}
+
+// the bit-plane words as a 3-D array of 32-bit elements: (word and column inside a strip's plane row, plane, strip); one
+// box = the eight words of two units for the strips of a CTA's channels, one plane
+bool planes_map(EncodeTiledFn enc, CUtensorMap *map, const uint8_t *packed, int K, int N, int bits, int group)
+{
+    const cuuint64_t wt = (cuuint64_t)(K / 32);
+    const cuuint64_t dims[3] = {wt * 4, (cuuint64_t)bits, (cuuint64_t)(N / 4)};
+    const cuuint64_t strides[2] = {wt * 16, wt * 16 * (cuuint64_t)bits};
+    const cuuint32_t box[3] = {(cuuint32_t)(2 * UK / 8), 1, (cuuint32_t)(CH / 4)};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint8_t *>(packed + make_layout(K, N, bits, group).planes_off), dims, strides, box,
+               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int BITS, bool PAIR, int V>
@@ -930,19 +992,8 @@ tman_status launch_mpgemm_variant(int variant, const void *packed, const void *x
     }
     Layout L = make_layout(K, N, bits, group);
     const uint8_t *pk = static_cast<const uint8_t *>(packed);
-    // the bit-plane words as a 3-D array of 32-bit elements: (word and column inside a strip's plane
-    // row, plane, strip); one box = the eight words of two units for the strips of a CTA's channels, one plane
     CUtensorMap tmap_w;
-    {
-        const cuuint64_t wt = (cuuint64_t)(K / 32);
-        const cuuint64_t wdims[3] = {wt * 4, (cuuint64_t)bits, (cuuint64_t)(N / 4)};
-        const cuuint64_t wstrides[2] = {wt * 16, wt * 16 * (cuuint64_t)bits};
-        const cuuint32_t wbox[3] = {(cuuint32_t)(2 * UK / 8), 1, (cuuint32_t)(CH / 4)};
-        if (enc(&tmap_w, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint8_t *>(pk + L.planes_off), wdims, wstrides,
-                wbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return TMAN_ERR_CUDA;
-    }
+    if (!planes_map(enc, &tmap_w, pk, K, N, bits, group)) return TMAN_ERR_CUDA;
 
     uint8_t *w8 = static_cast<uint8_t *>(ws);
     GemmParams p;
@@ -968,6 +1019,8 @@ tman_status launch_mpgemm_variant(int variant, const void *packed, const void *x
     p.tiles_n = g.tiles_n;
     p.span_tiles = g.span_tiles;
     p.split_s = g.split_s;
+    p.acc_sh = 0; p.acc_col = 0;
+    p.row_scale = nullptr; p.w_scale = 0.f;
     p.col_fastest = g.col_fastest;
     p.stamps = reinterpret_cast<long long *>(w8 + kGemmPartialOff + (size_t)kMaxGemmCtas * kPartialBytesPerCta);
     // the fp16 weights [N][K]: boxes of half a unit x a CTA's channels, 128-byte swizzle; unused maps are copies of the activation map
@@ -987,6 +1040,67 @@ tman_status launch_mpgemm_variant(int variant, const void *packed, const void *x
     if (variant == kGemmLoadFull) return launch_bits<4, kGemmLoadFull>(tmap_x, tmap_w, tmap_wf, p, g, s);
     if (variant == kGemmSequential) return launch_bits<4, kGemmSequential>(tmap_x, tmap_w, tmap_wf, p, g, s);
     return launch_bits<4, kGemmProduct>(tmap_x, tmap_w, tmap_wf, p, g, s);
+}
+
+// Integer path: ternary weights times 8-bit integer activations, y = fp16( row_scale[m] * w_scale * sum ).  Whole tiles only (the
+// call has no workspace for partial sums).  Tiles of up to 192 tokens leave room for two accumulators, so that a tile's
+// epilogue hides behind the next tile; 256 for one, whose epilogue does not.  A unit takes at least 0.2 us, whatever its
+// tokens, in issuing its MMAs and commits (the multiplications themselves: 0.2 us at 192), which bounds most sizes.  Measured at
+// 128 / 160 / 192 / 256 tokens a tile: 2048 x 2560 x 6912 41.0 / 36.2 / 35.4 / 39.5 us, 4096 x 6912 x 2560 74.3 / 62.1 / 50.9 / 65.3.
+// (Weights through shared memory in tiles of 128 tokens x 256 channels of one CTA, one row of dequantization warps: 44.3 and 97.1.)
+tman_status launch_mpgemm_ternary_i8(const void *packed, const int8_t *a8, const float *row_scale, float w_scale, void *y,
+                                     int M, int K, int N, int group, void *ws, cudaStream_t s)
+{
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return TMAN_ERR_CUDA;
+    const int sms = sm_count();
+    if (sms <= 0) return TMAN_ERR_CUDA;
+    GemmPlan g = {};
+    g.pair = gemm_pair(M) ? 1 : 0;
+    const int ncta = g.pair ? 2 : 1, gran = g.pair ? 32 : 16, workers = sms / ncta > 0 ? sms / ncta : 1;
+    g.tiles_n = (N + CH * ncta - 1) / (CH * ncta);
+    // least modelled time: rounds of tiles x (units of 128 k, and the epilogue where it does not hide behind them)
+    double best = 1e300;
+    for (int nt = gran; nt <= MAX_TOKENS; nt += gran) {
+        const long long tiles = (long long)((M + nt - 1) / nt) * g.tiles_n, rounds = (tiles + workers - 1) / workers;
+        const double unit_us = nt > 192 ? 0.00105 * nt : 0.2, tile_us = unit_us * (K / UK), epi_us = 0.4 + 0.008 * nt;
+        const double us = nt > 192 ? rounds * (tile_us + epi_us) : rounds * (tile_us > epi_us ? tile_us : epi_us) + epi_us;
+        if (us < best) { best = us; g.nt = nt; }
+    }
+    g.tiles_m = (M + g.nt - 1) / g.nt;
+    const long long tiles = (long long)g.tiles_m * g.tiles_n;
+    if (tiles >= (1ll << 31)) return TMAN_ERR_SHAPE;
+    g.workers = (int)(tiles < workers ? tiles : workers);
+    GemmParams p = {};
+    p.M = M; p.K = K; p.N = N; p.bits = 2; p.group = group;
+    p.nt = g.nt; p.tiles_m = g.tiles_m; p.tiles_n = g.tiles_n;
+    p.packed = static_cast<const uint8_t *>(packed);
+    p.y = static_cast<__half *>(y);
+    p.status = static_cast<uint32_t *>(ws);
+    p.row_scale = row_scale;
+    p.w_scale = w_scale;
+    const int rows_cta = g.nt / ncta;
+    p.acc_sh = g.nt <= 192 ? 1 : 0;
+    p.wcol = g.nt <= 128 ? 256 : g.nt <= 192 ? 384 : 256;
+    p.wbufs = K >= 8 * UK && (g.nt <= 128 || g.nt > 192) ? 8 : 4;
+    p.acc_col = g.nt <= 128 ? 128 : 192;
+    p.xu_sh = 1;
+    p.xst_sh = 3;
+    while ((rows_cta * UK << p.xu_sh << p.xst_sh) > X_RING_BYTES) --p.xst_sh;
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUtensorMap tmap_x;
+    {
+        const cuuint64_t dims[3] = {(cuuint64_t)UK, (cuuint64_t)M, (cuuint64_t)(K / UK)};
+        const cuuint64_t strides[2] = {(cuuint64_t)K, (cuuint64_t)UK};
+        const cuuint32_t box[3] = {(cuuint32_t)UK, (cuuint32_t)rows_cta, (cuuint32_t)(1 << p.xu_sh)};
+        if (enc(&tmap_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<int8_t *>(a8), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return TMAN_ERR_CUDA;
+    }
+    CUtensorMap tmap_w;
+    if (!planes_map(enc, &tmap_w, p.packed, K, N, 2, group)) return TMAN_ERR_CUDA;
+    return launch_bits<2, kGemmInt8>(tmap_x, tmap_w, tmap_x, p, g, s);
 }
 
 }  // namespace tman

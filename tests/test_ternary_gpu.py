@@ -201,6 +201,15 @@ def test_int8_prefill_matches_the_integer_oracle(M, K, N, group):
     assert B.tman_read_status(ws) == 5 and bool((y == 3.0).all())
 
 
+# a single CTA's last size and a pair's first, tiles of 32 to 192 tokens with a ragged last one, one packed stage and half of a
+# second (K = 128, 384, 1152), four and eight weight buffers (K below and from 1024), channels that end inside a CTA and a pair,
+# several tiles per worker (both accumulators)
+@pytest.mark.parametrize("M,K,N,group", [(16, 128, 72, 32), (17, 384, 392, 64), (33, 1152, 264, 128), (193, 896, 520, 128),
+                                         (385, 1024, 20000, 64), (1537, 128, 4104, 32)])
+def test_int8_prefill_edges(M, K, N, group):
+    test_int8_prefill_matches_the_integer_oracle(M, K, N, group)
+
+
 @pytest.mark.parametrize("M,K,N,group", [(2, 1024, 40, 64), (3, 2560, 264, 128), (4, 6912, 2560, 128), (5, 1152, 72, 32),
                                          (8, 2560, 6912, 64), (7, 16384, 16, 128)])
 def test_ternary_decode_with_several_rows(M, K, N, group):
