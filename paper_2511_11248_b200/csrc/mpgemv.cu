@@ -743,6 +743,9 @@ static tman_status launch_one(GemvParams p, int sms, cudaStream_t s)
         p.units += (p.Ng[g] / 4 + S * SUBS - 1) / (S * SUBS);
     }
     for (int g = p.count; g < kGemvMaxGroup; ++g) p.unit0[g] = p.units;
+    // Units of one strip: about half of a CTA's warps get one.  With all of them at work (fewer CTAs) and with one each (as many
+    // CTAs as units) 4-bit 4096 x 1024 takes 3.84 and 3.64 us instead of 3.59, two rows 4.70 and 5.33 instead of 5.23.
+    if (S == 1 && !INT && p.P * kGemvWarps > 2 * p.units) p.P = (2 * p.units + kGemvWarps - 1) / kGemvWarps;
     if (p.P > p.units) p.P = p.units;
     // every CTA must be resident while it polls for the others' partial sums
     if ((long long)p.nkappa * p.P > (long long)sms) return TMAN_ERR_UNSUPPORTED;
@@ -791,6 +794,12 @@ static tman_status launch_mt(GemvParams p, int sms, cudaStream_t s)
     constexpr int S = (HR && MT == 2) ? 2 : ((BITS == 2) ? 4 : 2);
     constexpr int HALF = HR ? 0 : 1;
     if (p.count > 1) return launch_one<BITS, MT, S, PRE, HALF, 1, ROLL, HR>(p, sms, s);
+    // One matrix of so few columns that a strip per sub-warp is enough: units of one strip, and fewer CTAs (launch_one).
+    // In a graph, 4-bit 4096 x 1024: 3.86 -> 3.59 us (one row), 5.42 -> 5.23 (two), 2-bit 4096 x 512: 3.85 -> 3.12, 5.34 -> 4.16; near the
+    // line (4096 x 2048) 4.19 -> 4.09 and 5.77 -> 5.74, above it the larger units are as fast or faster.
+    constexpr int W = HALF ? 16 : 32 / MT;
+    const int ctas = sms / ((p.K / 32 + W - 1) / W);
+    if (p.N / 4 <= ctas * kGemvWarps * (32 / W)) return launch_one<BITS, MT, 1, PRE, HALF, 0, ROLL, HR>(p, sms, s);
     return launch_one<BITS, MT, S, PRE, HALF, 0, ROLL, HR>(p, sms, s);
 }
 

@@ -110,6 +110,24 @@ def test_rows_in_fp16_tables_stay_near_the_predicted_error(M, factor):
     assert rel_err(got, ref) <= 2e-3
 
 
+@pytest.mark.parametrize("M,bits,G", [(1, 2, 64), (1, 3, 128), (1, 4, 32), (2, 4, 128), (3, 2, 32), (4, 2, 64)])
+@pytest.mark.parametrize("K,N", [(128, 8), (1152, 40), (4096, 2304), (4096, 2312), (4096, 2368), (4096, 2376)])
+def test_lookup_units_of_one_strip_and_the_line_above_them(M, bits, G, K, N):
+    # 148 SMs: K = 4096 in slices of 512 or 1024 k leaves 576 or 592 strips of four columns to units of one strip.  One row: fp32
+    # sums, the result rounded to fp16; more rows: fp16 tables, the bound of test_rows_in_fp16_tables_stay_near_the_predicted_error.
+    c = synth.small_case(M, K, N, bits, G, seed=900 + M + K + N)
+    dev = H.device_case(c)
+    packed = H.pack_case(c, dev)
+    ws = H.alloc_workspace(B.OP_GEMV, M, K, N, bits, G)
+    ref = orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)
+    for _ in range(2):                                       # the second call finds the workspace as the first left it
+        y = H.alloc_y(M, N)
+        B.tman_mpgemv(packed, dev["x"], y, M, K, N, bits, G, ws)
+        assert B.tman_read_status(ws) == 0
+        H.check_guards()
+        assert rel_err(H.to_f64(y), ref) <= (5.1e-4 if M == 1 else 2e-3)
+
+
 @pytest.mark.parametrize("M,bits,G", [(3, 3, 64), (4, 4, 128), (5, 2, 32), (5, 3, 64), (6, 2, 64), (7, 4, 32), (8, 2, 128), (8, 3, 128), (8, 4, 64)])
 @pytest.mark.parametrize("K,Ns", [(128, (8,)), (640, (32, 40)), (2176, (264,)), (4096, (2056, 8, 40))])
 def test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, Ns):
