@@ -4,7 +4,8 @@
 // Work split.  A warp owns one 128-deep chunk of k for the whole call: its activations (the eight columns of the MMA's
 // B operand) stay in 16 registers.  It walks over groups of 32 output columns: a lane's 16-byte load is one plane word
 // (32 k) of the four columns of a strip, 8 strips x 4 words a warp.  TK warps with consecutive chunks form a team that
-// walks the same groups; a CTA has TC teams (TK x TC <= 16).  After a group the team's sums are added through shared
+// walks the same groups; a CTA has TC teams (TK x TC <= 16).  CPW = 2: a warp owns two neighbouring chunks, so that K = 4096 needs
+// no second CTA and no partial sums through memory; their activations are in shared memory.  After a group the team's sums are added through shared
 // memory (one team barrier a group, two buffers); the K-slices of 128 x TK k that different CTAs own are combined through
 // fp32 partial sums in the workspace whose "no sum pending" pattern says when they are there (see mpgemv.cu).
 //
@@ -155,12 +156,13 @@ __device__ __forceinline__ bool wait_for_sums(const float4 *src, size_t stride4,
 }
 
 constexpr int kMmaThreads = 512;
-template <int BITS, int R> struct MmaCfg {
+template <int BITS, int R, int NE, int CPW> struct MmaCfg {
     static constexpr int RED_WARP = 8 * 128;                                     // a warp's sums of a group: 8 columns of B x 32 columns
     static constexpr int RED_BYTES = 2 * 16 * RED_WARP;
     static constexpr int SCALE_BYTES = 16 * 8 * 4;                               // the power-of-two scale of every (column of B, warp)
+    static constexpr int FRAG_CHUNK = 2048 + R * NE * 128;                       // a warp's activations of a chunk: B fragments, block sums
     static constexpr int PATCH_WARP = R > 1 ? BITS * 512 : 0;                    // R > 1: a group's plane words, redistributed among lanes
-    static constexpr int SMEM = RED_BYTES + SCALE_BYTES + 16 * PATCH_WARP;
+    static constexpr int SMEM = RED_BYTES + SCALE_BYTES + 16 * (PATCH_WARP + (CPW > 1 ? CPW * FRAG_CHUNK : 0));
     static constexpr int DEPTH = BITS == 2 ? 4 : 2;                              // groups whose loads are in flight per warp
 };
 
@@ -168,10 +170,10 @@ template <int BITS, int R> struct MmaCfg {
 //   R = 1: column = block of the chunk x T + row, T = 8 / NB rows (NE = 2), NB = 128 / group blocks; a lane whose word lies in
 //          another block than its column holds zeros.  NE = 1: only the even columns (T = 4 / NB rows), one value per accumulator pair.
 //   R = 2, 4: column = row; the chunk's blocks of 64 / 32 k are multiplied one after the other, a lane's word in halves / quarters.
-template <int BITS, int R, int NB, int NE>
+template <int BITS, int R, int NB, int NE, int CPW>
 __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaParams p)
 {
-    using C = MmaCfg<BITS, R>;
+    using C = MmaCfg<BITS, R, NE, CPW>;
     constexpr int DEPTH = C::DEPTH;
     constexpr int T = (NE == 2 ? 8 : 4) / NB;                                    // rows the columns hold
     static_assert(R == 1 || (NB == 1 && NE == 2), "sub-word passes use all eight columns for rows");
@@ -180,8 +182,9 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
     const int TK = p.tk, team = warp / TK, wk = warp - team * TK;                // this warp's team and place in it
     const int kappa = blockIdx.y, P = gridDim.x;
     const int words = p.K >> 5;
-    const int chunk = kappa * TK + wk;
-    const bool active = chunk < p.chunks;
+    constexpr int csh = CPW - 1;
+    const int chunk = (kappa * TK + wk) * CPW;                                   // this warp's first chunk
+    const bool active = chunk < p.chunks, both = CPW > 1 && chunk + 1 < p.chunks;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
@@ -200,19 +203,19 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
         for (int t = 1; t < kGemvMaxGroup; ++t) mtx += (t < p.count && g >= p.grp0[t]) ? 1 : 0;
         return mtx;
     };
-    auto load = [&](int g, uint4 (&w)[BITS], uint2 &sc, uint32_t &z) {
-        if (!active) return;
+    auto load = [&](int g, int c, uint4 (&w)[BITS], uint2 &sc, uint32_t &z) {
+        if (!(c ? both : active)) return;
         const int gc = min(g, p.groups - 1), mtx = matrix_of(gc);               // past the last group: the last again, never used
         const int nb = min((gc - p.grp0[mtx]) * 8 + gid, (p.Ng[mtx] >> 2) - 1);
-        const uint8_t *q = p.planes[mtx] + (size_t)nb * strip_bytes + lane_off;
+        const uint8_t *q = p.planes[mtx] + (size_t)nb * strip_bytes + lane_off + 64 * c;
 #pragma unroll
         for (int i = 0; i < BITS; ++i) w[i] = __ldcs(reinterpret_cast<const uint4 *>(q + (size_t)i * row_bytes));
-        const size_t blk = (size_t)nb * p.nblk + blk_off;
+        const size_t blk = (size_t)nb * p.nblk + blk_off + (uint32_t)(c << (7 - p.group_shift));
         sc = __ldg(p.scales[mtx] + blk);
         z = __ldg(p.zeros[mtx] + blk);
     };
 #pragma unroll
-    for (int d = 0; d < DEPTH; ++d) load(g_first + d * g_stride, wbuf[d], sbuf[d], zbuf[d]);
+    for (int d = 0; d < DEPTH; ++d) load(g_first + (d >> csh) * g_stride, d & csh, wbuf[d], sbuf[d], zbuf[d]);
 
     bool hdr_ok = true;
 #pragma unroll
@@ -227,65 +230,87 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // ---- this warp's activations: B fragments, block sums and scales ---------------------------------------
-    uint32_t xb[16];
-    float S[R][NE];                                  // activation sums of the accumulator columns this lane holds, in the sums' units
+    // (of two chunks in shared memory, written and read by the same lane; of one in registers)
+    uint4 xb1[4];
+    float S1[R][NE];
+    uint8_t *const frags = smem + C::RED_BYTES + C::SCALE_BYTES + 16 * C::PATCH_WARP + warp * (CPW * C::FRAG_CHUNK);
     float *const row_back = reinterpret_cast<float *>(smem + C::RED_BYTES);      // [B column][warp]: what undoes the scaling
     LaneMasks<R> lm;
     lm.template set<BITS>(R == 2 ? tig >> 1 : tig);
     {
         const int col = NE == 2 ? gid : gid >> 1;                                // B column of this lane
         const int b_row = col % T, b_blk = col / T;
-        const bool live = active && b_row < p.M && (NE == 2 || !(gid & 1)) && (R > 1 || NB == 1 || (tig * NB) / 4 == b_blk);
-        uint4 raw[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int word = R == 1 ? tig : R == 2 ? 2 * (i >> 1) + (tig & 1) : i;
-            const int ph = R == 1 ? i : R == 2 ? (tig >> 1) + 2 * (i & 1) : tig;
-            raw[i] = make_uint4(0u, 0u, 0u, 0u);
-            if (live) raw[i] = __ldg(reinterpret_cast<const uint4 *>(p.x + (size_t)b_row * p.K + (size_t)chunk * 128 + word * 32 + ph * 8));
-        }
-        float amax = 0.f, sum[R];
-#pragma unroll
-        for (int b = 0; b < R; ++b) sum[b] = 0.f;
+        const bool live = b_row < p.M && (NE == 2 || !(gid & 1)) && (R > 1 || NB == 1 || (tig * NB) / 4 == b_blk);
+        uint4 raw[CPW][4];
+        float amax;
         __half2 mx = __floats2half2_rn(0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int c = 0; c < CPW; ++c)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const uint32_t u = comp(raw[i], e);
-                const __half2 h = *reinterpret_cast<const __half2 *>(&u);
-                mx = __hmax2(mx, __habs2(h));
-                const float2 f = __half22float2(h);
-                sum[R == 1 ? 0 : R == 2 ? i >> 1 : i] += f.x + f.y;
+            for (int i = 0; i < 4; ++i) {
+                const int word = R == 1 ? tig : R == 2 ? 2 * (i >> 1) + (tig & 1) : i;
+                const int ph = R == 1 ? i : R == 2 ? (tig >> 1) + 2 * (i & 1) : tig;
+                raw[c][i] = make_uint4(0u, 0u, 0u, 0u);
+                if (live && (c ? both : active))
+                    raw[c][i] = __ldg(reinterpret_cast<const uint4 *>(p.x + (size_t)b_row * p.K + (size_t)(chunk + c) * 128 + word * 32 + ph * 8));
             }
+#pragma unroll
+        for (int c = 0; c < CPW; ++c)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t u = comp(raw[c][i], e);
+                    mx = __hmax2(mx, __habs2(*reinterpret_cast<const __half2 *>(&u)));
+                }
         amax = fmaxf(__low2float(mx), __high2float(mx));
 #pragma unroll
-        for (int mask = 1; mask < 4; mask <<= 1) {
-            amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, mask));
-#pragma unroll
-            for (int b = 0; b < R; ++b) sum[b] += __shfl_xor_sync(0xffffffffu, sum[b], mask);
-        }
+        for (int mask = 1; mask < 4; mask <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, mask));
         const uint32_t be = min(__float_as_uint(amax) >> 23, 240u);              // amax = 1.f * 2^(be - 127)
         const float fac = __uint_as_float((be ? 268u - be : 127u) << 23);
         const float back = __uint_as_float((be ? be + 10u : 151u) << 23);         // 2^24 / fac
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int c = 0; c < CPW; ++c) {
+            float sum[R];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t u0 = comp(raw[i], j >> 1), u1 = comp(raw[i], 2 + (j >> 1));
-                const __half2 h0 = *reinterpret_cast<const __half2 *>(&u0), h1 = *reinterpret_cast<const __half2 *>(&u1);
-                const float f = fac * field_factor(R == 1 ? i : R == 2 ? (tig >> 1) + 2 * (i & 1) : tig, j);
-                const __half2 h = __floats2half2_rn((j & 1 ? __high2float(h0) : __low2float(h0)) * f,
-                                                    (j & 1 ? __high2float(h1) : __low2float(h1)) * f);
-                xb[4 * i + j] = *reinterpret_cast<const uint32_t *>(&h);
+            for (int b = 0; b < R; ++b) sum[b] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t u = comp(raw[c][i], e);
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&u));
+                    sum[R == 1 ? 0 : R == 2 ? i >> 1 : i] += f.x + f.y;
+                }
+#pragma unroll
+            for (int mask = 1; mask < 4; mask <<= 1)
+#pragma unroll
+                for (int b = 0; b < R; ++b) sum[b] += __shfl_xor_sync(0xffffffffu, sum[b], mask);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint32_t xb[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t u0 = comp(raw[c][i], j >> 1), u1 = comp(raw[c][i], 2 + (j >> 1));
+                    const __half2 h0 = *reinterpret_cast<const __half2 *>(&u0), h1 = *reinterpret_cast<const __half2 *>(&u1);
+                    const float f = fac * field_factor(R == 1 ? i : R == 2 ? (tig >> 1) + 2 * (i & 1) : tig, j);
+                    const __half2 h = __floats2half2_rn((j & 1 ? __high2float(h0) : __low2float(h0)) * f,
+                                                        (j & 1 ? __high2float(h1) : __low2float(h1)) * f);
+                    xb[j] = *reinterpret_cast<const uint32_t *>(&h);
+                }
+                if constexpr (CPW == 1) xb1[i] = make_uint4(xb[0], xb[1], xb[2], xb[3]);
+                else *reinterpret_cast<uint4 *>(frags + c * C::FRAG_CHUNK + i * 512 + lane * 16) = make_uint4(xb[0], xb[1], xb[2], xb[3]);
             }
+            // activation sums of the accumulator columns this lane holds, in the sums' units (against zero-points held as z x 2^-24)
+#pragma unroll
+            for (int b = 0; b < R; ++b)
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+                    const float v = __shfl_sync(0xffffffffu, sum[b] * fac, 4 * (2 * tig + e));   // a lane of that B column
+                    if constexpr (CPW == 1) S1[b][e] = v;
+                    else *reinterpret_cast<float *>(frags + c * C::FRAG_CHUNK + 2048 + (b * NE + e) * 128 + lane * 4) = v;
+                }
         }
-#pragma unroll
-        for (int b = 0; b < R; ++b) sum[b] *= fac;                               // (against zero-points held as z x 2^-24)
-#pragma unroll
-        for (int e = 0; e < NE; ++e)
-#pragma unroll
-            for (int b = 0; b < R; ++b) S[b][e] = __shfl_sync(0xffffffffu, sum[b], 4 * (2 * tig + e));   // a lane of that B column
         if (tig == 0 && (NE == 2 || !(gid & 1))) row_back[col * 16 + warp] = back;
     }
 
@@ -297,7 +322,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
     // ---- one group: 32 columns x this warp's 128 k ----------------------------------------------------------
     uint8_t *red = smem;
     uint8_t *patch = smem + C::RED_BYTES + C::SCALE_BYTES + warp * C::PATCH_WARP;
-    auto group_sums = [&](const uint4 (&wr)[BITS], uint2 sc_l, uint32_t z_l, float4 (&out)[NE]) {
+    auto group_sums = [&](const uint8_t *frag, const uint4 (&wr)[BITS], uint2 sc_l, uint32_t z_l, float4 (&out)[NE]) {
         float tot[2][2][NE];
 #pragma unroll
         for (int gg = 0; gg < R; ++gg) {
@@ -321,7 +346,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
             }
             auto quarter = [&](auto qc) {
                 constexpr int Q = decltype(qc)::value;
-                const uint32_t *b = xb + 4 * ((4 / R) * gg + Q);
+                const uint4 bq = CPW == 1 ? xb1[(4 / R) * gg + Q] : *reinterpret_cast<const uint4 *>(frag + ((4 / R) * gg + Q) * 512 + lane * 16);
+                const uint32_t b[4] = {bq.x, bq.y, bq.z, bq.w};
                 uint32_t o[4][4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) quarter_pairs<BITS, R, Q>(pw[c], lm, o[c]);
@@ -352,7 +378,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
                 const float z0 = s ? zef.y : zef.x, z1 = s ? zof.y : zof.x;
 #pragma unroll
                 for (int e = 0; e < NE; ++e) {
-                    const float t0 = fmaf(-z0, S[gg][e], acc[s][e]), t1 = fmaf(-z1, S[gg][e] * 0.0625f, acc[s][2 + e]);
+                    const float S = CPW == 1 ? S1[gg][e] : *reinterpret_cast<const float *>(frag + 2048 + (gg * NE + e) * 128 + lane * 4);
+                    const float t0 = fmaf(-z0, S, acc[s][e]), t1 = fmaf(-z1, S * 0.0625f, acc[s][2 + e]);
                     tot[s][0][e] = gg == 0 ? sf.x * t0 : fmaf(sf.x, t0, tot[s][0][e]);
                     tot[s][1][e] = gg == 0 ? sf.y * t1 : fmaf(sf.y, t1, tot[s][1][e]);
                 }
@@ -399,22 +426,31 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
 #pragma unroll
     for (int e = 0; e < NE; ++e) my_red[e] = red_at(0, warp, NE == 2 ? 2 * tig + e : tig, gid);
     int turn = 0, flip = 0;
+    float4 out[NE];
 #pragma unroll 1
-    for (int g0 = g_first; g0 < p.groups; g0 += DEPTH * g_stride) {
+    for (int g0 = g_first; g0 < p.groups; g0 += (DEPTH >> csh) * g_stride) {
 #pragma unroll
         for (int d = 0; d < DEPTH; ++d) {
-            const int g = g0 + d * g_stride;
+            const int g = g0 + (d >> csh) * g_stride, c = d & csh;
             if (g >= p.groups) break;                // uniform over the team
-            if (active) {
+            if (c ? both : active) {
                 if constexpr (R > 1) {
                     __syncwarp();
 #pragma unroll
                     for (int i = 0; i < BITS; ++i) *reinterpret_cast<uint4 *>(patch + i * 512 + lane * 16) = wbuf[d][i];
                     __syncwarp();
                 }
-                float4 out[NE];
-                group_sums(wbuf[d], sbuf[d], zbuf[d], out);
-                load(g + DEPTH * g_stride, wbuf[d], sbuf[d], zbuf[d]);
+                float4 cur[NE];
+                group_sums(frags + c * C::FRAG_CHUNK, wbuf[d], sbuf[d], zbuf[d], cur);
+                load(g + (DEPTH >> csh) * g_stride, c, wbuf[d], sbuf[d], zbuf[d]);
+#pragma unroll
+                for (int e = 0; e < NE; ++e) {
+                    if (CPW > 1 && c) { cur[e].x += out[e].x; cur[e].y += out[e].y; cur[e].z += out[e].z; cur[e].w += out[e].w; }
+                    out[e] = cur[e];
+                }
+            }
+            if (c != csh) continue;                  // the group's second chunk follows
+            if (active) {
 #pragma unroll
                 for (int e = 0; e < NE; ++e)
                     if ((NE == 2 ? 2 * tig + e : tig) % T < p.M)

@@ -818,9 +818,9 @@ static const GemvVariant kGemvVariants[kGemvVariantCount] = {
 
 // Whether a pass of `rows` rows goes to the tensor-core kernel (decode_mma.cuh) instead of the table lookups.  From five
 // rows always: an entry of eight fp16 rows costs four shared-memory wavefronts a lookup (4-bit 4096 x 28672, group 128:
-// 42.0 us by lookup, 21.3 us here; 3-bit, group 64: 24.3).  With three and four rows
+// 42.0 us by lookup, 20.6 us here; 3-bit, group 64: 21.6; 2-bit: 19.3).  With three and four rows
 // (two wavefronts) where a lookup per plane is many of them and the blocks are no shorter than two words: 4-bit, group 128
-// 23.8 / 18.9, 3-bit, group 64 20.2 / 18.9 (4096 x 4096: 7.4 / 6.6), but 2-bit, group 64 17.2 / 18.1 and 4-bit, group 32
+// 23.8 / 18.9, 3-bit, group 64 20.2 / 18.9 (4096 x 4096: 7.4 / 5.6), but 2-bit, group 64 17.2 / 18.1 and 4-bit, group 32
 // 24.0 / 31.2.  One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.2 / 18.4).
 static bool uses_mma(int bits, int group, int rows) { return rows >= 5 || (rows >= 3 && bits >= 3 && group >= 64); }
 
@@ -843,23 +843,28 @@ static bool variant_feasible(const GemvVariant &v, int K, int N, int sms, size_t
 
 // How the tensor-core kernel cuts a pass: warps of a team (each one 128-deep chunk of k), teams per CTA, K-slices, CTAs per
 // K-slice.  16 warps of a team give the fewest partial sums; 8 and 4 are for short K or few columns, where more CTAs get work.
-struct MmaSplit { int tk, tc, nkappa, ctas; };
+struct MmaSplit { int tk, tc, nkappa, ctas, cpw; };
 static MmaSplit split_mma(int M, int K, int N, int groups, int sms, size_t ws_limit)
 {
     const int chunks = K / 128;
-    MmaSplit best = {0, 0, 0, 0};
+    MmaSplit best = {0, 0, 0, 0, 0};
     double best_us = 1e300;
-    for (int tk = 16; tk >= 4; tk >>= 1) {
-        const int parts = (chunks + tk - 1) / tk;
+    for (int way = 0; way < 4; ++way) {                     // 16 warps with two chunks each, then 16, 8, 4 with one
+        const int cpw = way == 0 ? 2 : 1, tk = way == 0 ? 16 : 32 >> way;
+        const int parts = (chunks + tk * cpw - 1) / (tk * cpw);
         if (parts > sms) continue;                          // every CTA must be resident while it polls
         if (parts > 1 && kWsStatusBytes + (size_t)parts * M * N * sizeof(float) > ws_limit) continue;
         int tc = 16 / tk, ctas = sms / parts;
         while (tc > 1 && (groups + tc - 1) / tc < ctas) tc >>= 1;
         if (ctas > (groups + tc - 1) / tc) ctas = (groups + tc - 1) / tc;
-        const int steps = (groups + ctas * tc - 1) / (ctas * tc);
-        // a step costs half its time in latency however many warps take part; the partial sums are written and read back
-        const double us = steps * 0.5 * (tk * tc / 16.0 + 1) + (parts > 1 ? 1.0 : 0.0) + (double)parts * M * N * 8e-6 / 3.0;
-        if (us < best_us) { best_us = us; best = {tk, tc, parts, ctas}; }
+        const int steps = (groups + ctas * tc - 1) / (ctas * tc) * cpw;
+        // a step costs half its time in latency however many warps take part, a tenth more with two chunks a warp (activations
+        // from shared memory, a longer start); the partial sums are written, waited for and read back.  Two chunks against one,
+        // in a graph, 4-bit group 128: 4096 x 4096 5.6 / 6.5 us (four rows), 6.5 / 6.9 (eight), 4096 x 28672 19.5 / 18.9 and 20.6 / 21.3;
+        // 3-bit group 64, eight rows 21.6 / 24.3; 14336 x 4096, four rows 14.5 / 11.9.
+        const double us = steps * 0.5 * (tk * tc / 16.0 + 1) * (cpw == 2 ? 1.1 : 1.0) + (cpw == 2 ? 0.25 : 0.0) + (parts > 1 ? 1.6 : 0.0) +
+                          (double)parts * M * N * 8e-6 / 3.0 * (parts > 1);
+        if (us < best_us) { best_us = us; best = {tk, tc, parts, ctas, cpw}; }
     }
     return best;
 }
@@ -908,10 +913,10 @@ GemvPlan plan_gemv(int M, int K, int N, int bits, int group, int sms, size_t ws_
         ps.mma = uses_mma(bits, group, take);
         if (ps.mma) {
             const MmaSplit sp = split_mma(take, K, N, (N + 31) / 32, sms, need);
-            ps.words = 4 * sp.tk;
+            ps.words = 4 * sp.tk * sp.cpw;
             ps.nkappa = sp.nkappa;
             ps.ctas_per_slice = sp.ctas;
-            ps.smem_bytes = MmaCfg<4, 4>::SMEM;             // at most
+            ps.smem_bytes = MmaCfg<4, 4, 2, 2>::SMEM;             // at most
         }
         if (need > g.ws_bytes) g.ws_bytes = need;
         left -= take;
@@ -919,15 +924,13 @@ GemvPlan plan_gemv(int M, int K, int N, int bits, int group, int sms, size_t ws_
     return g;
 }
 
-template <int BITS, int R, int NB, int NE>
-static tman_status launch_mma(MmaParams p, int sms, size_t ws_limit, cudaStream_t s)
+template <int BITS, int R, int NB, int NE, int CPW>
+static tman_status launch_mma_split(MmaParams p, const MmaSplit &sp, cudaStream_t s)
 {
-    const MmaSplit sp = split_mma(p.M, p.K, p.N, p.groups, sms, ws_limit);
-    if (!sp.ctas) return TMAN_ERR_UNSUPPORTED;
     p.chunks = p.K / 128;
     p.tk = sp.tk; p.tc = sp.tc; p.nkappa = sp.nkappa;
-    constexpr int smem = MmaCfg<BITS, R>::SMEM;
-    auto kern = decode_mma_kernel<BITS, R, NB, NE>;
+    constexpr int smem = MmaCfg<BITS, R, NE, CPW>::SMEM;
+    auto kern = decode_mma_kernel<BITS, R, NB, NE, CPW>;
     static std::atomic<bool> raised[kMaxDevices];
     int dev = 0;
     if (!device_info(&dev)) return TMAN_ERR_CUDA;
@@ -942,6 +945,14 @@ static tman_status launch_mma(MmaParams p, int sms, size_t ws_limit, cudaStream_
     cfg.attrs = attr;
     cfg.numAttrs = packed_write_pending(s, /*clear=*/true) ? 0 : 1;      // as in launch_one
     return launch_with_smem(kern, smem, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, p); });
+}
+
+template <int BITS, int R, int NB, int NE>
+static tman_status launch_mma(const MmaParams &p, int sms, size_t ws_limit, cudaStream_t s)
+{
+    const MmaSplit sp = split_mma(p.M, p.K, p.N, p.groups, sms, ws_limit);
+    if (!sp.ctas) return TMAN_ERR_UNSUPPORTED;
+    return sp.cpw == 2 ? launch_mma_split<BITS, R, NB, NE, 2>(p, sp, s) : launch_mma_split<BITS, R, NB, NE, 1>(p, sp, s);
 }
 
 template <int BITS>

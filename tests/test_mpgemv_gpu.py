@@ -150,6 +150,16 @@ def test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, Ns):
             assert rel_err(H.to_f64(y), ref) <= 5.1e-4
 
 
+@pytest.mark.parametrize("M,bits,G,K,N", [(M, b, G, K, 4104) for K in (2176, 4096) for M, b, G in
+                                          [(3, 3, 64), (4, 4, 128), (5, 2, 32), (6, 2, 64), (8, 2, 128), (8, 3, 128), (8, 4, 32)]] + [(8, 3, 64, 16384, 4736)])
+def test_tensor_core_rows_with_two_chunks_a_warp(M, bits, G, K, N):
+    # an odd number of chunks (the last warp at work has one), one K-slice and four; the bound of the test above, whose chunks here
+    # share a scale two by two (activations below 2^-29 of a pair's largest would lose bits: none)
+    plan = B.tman_debug_gemv_plan(M, K, N, bits, G)
+    assert plan["passes"][0]["words"] == 128, plan           # 16 warps x 2 chunks x 4 plane words
+    test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, (N,))
+
+
 def test_repeat_calls_share_workspace_and_agree():
     c = synth.small_case(2, 2048, 264, 4, 64, seed=21)
     dev = H.device_case(c)
