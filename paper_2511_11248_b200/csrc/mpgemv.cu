@@ -1,7 +1,7 @@
 // Decode path: bit-serial table-lookup mpGEMV (paper Sec. 2.2 "Bit-serial table lookup", Fig. 2;
 // Sec. 4.3 "Mapping of LUT-based Decoding").
 //
-// One to four activation rows by table lookup, described here; more rows (and four where that is faster, uses_mma below) on
+// One and two activation rows (and three and four where that is faster, uses_mma below) by table lookup, described here; more rows on
 // the tensor cores (decode_mma.cuh).
 //
 // Work split.  The reduction dimension is cut into K-slices of 16 or 32 plane words (16 for one
@@ -819,10 +819,14 @@ static const GemvVariant kGemvVariants[kGemvVariantCount] = {
 // Whether a pass of `rows` rows goes to the tensor-core kernel (decode_mma.cuh) instead of the table lookups.  From five
 // rows always: an entry of eight fp16 rows costs four shared-memory wavefronts a lookup (4-bit 4096 x 28672, group 128:
 // 42.0 us by lookup, 20.6 us here; 3-bit, group 64: 21.6; 2-bit: 19.3).  With three and four rows
-// (two wavefronts) where a lookup per plane is many of them and the blocks are no shorter than two words: 4-bit, group 128
-// 23.8 / 18.9, 3-bit, group 64 20.2 / 18.9 (4096 x 4096: 7.4 / 5.6), but 2-bit, group 64 17.2 / 18.1 and 4-bit, group 32
-// 24.0 / 31.2.  One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.2 / 18.4).
-static bool uses_mma(int bits, int group, int rows) { return rows >= 5 || (rows >= 3 && bits >= 3 && group >= 64); }
+// (two wavefronts) where the blocks are no shorter than two words: 4-bit, group 128
+// 23.8 / 18.9, 3-bit, group 64 20.2 / 18.9 (4096 x 4096: 7.4 / 5.6), 2-bit, group 128 17.3 / 16.9 (6.8 / 5.5); but 4-bit, group 32
+// 24.0 / 31.2.  2-bit, group 64 (few planes to look up, halves of a chunk to multiply) as far as a call is short: 4096 x 6144 8.4 / 7.0,
+// 14336 x 4096 11.3 / 11.5, 4096 x 28672 17.3 / 18.2.  One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.2 / 18.4).
+static bool uses_mma(int bits, int group, int rows, long long weights)
+{
+    return rows >= 5 || (rows >= 3 && group >= 64 && (bits >= 3 || group == 128 || weights <= 48000000ll));
+}
 
 static size_t variant_ws_bytes(const GemvVariant &v, int K, int N)
 {
@@ -910,7 +914,7 @@ GemvPlan plan_gemv(int M, int K, int N, int bits, int group, int sms, size_t ws_
         ps.ctas_per_slice = sms / ps.nkappa;
         ps.smem_bytes = v.half_slices ? kGemvTableBytes / 2 : kGemvTableBytes + 64;
         const size_t need = variant_ws_bytes(v, K, N);
-        ps.mma = uses_mma(bits, group, take);
+        ps.mma = uses_mma(bits, group, take, (long long)K * N);
         if (ps.mma) {
             const MmaSplit sp = split_mma(take, K, N, (N + 31) / 32, sms, need);
             ps.words = 4 * sp.tk * sp.cpw;
@@ -976,9 +980,7 @@ static tman_status launch_mma_rows(const GemvParams &g, int rows, int sms, size_
     p.M = rows; p.K = g.K; p.N = g.N;
     p.bits = g.bits; p.group = g.group; p.group_shift = g.group_shift; p.nblk = g.nblk;
     // the columns of B hold the blocks of a chunk as long as there are enough of them for the rows
-    if constexpr (BITS > 2) {
-        if (p.group >= 64 && rows <= 4) return p.group == 128 ? launch_mma<BITS, 1, 1, 1>(p, sms, ws, s) : launch_mma<BITS, 1, 2, 2>(p, sms, ws, s);
-    }
+    if (p.group >= 64 && rows <= 4) return p.group == 128 ? launch_mma<BITS, 1, 1, 1>(p, sms, ws, s) : launch_mma<BITS, 1, 2, 2>(p, sms, ws, s);
     if (p.group == 128) return launch_mma<BITS, 1, 1, 2>(p, sms, ws, s);
     return p.group == 64 ? launch_mma<BITS, 2, 1, 2>(p, sms, ws, s) : launch_mma<BITS, 4, 1, 2>(p, sms, ws, s);
 }
