@@ -513,7 +513,7 @@ def bench_gemm(torch, B, H, synth, peaks):
         tot_flops += flops
         tot_sec += sec
     tf = tot_flops / tot_sec / 1e12
-    out.update({"bound": "tensor", "kernel": "mpgemm_kernel<4,2,true> (4-bit, CTA pairs, two row blocks per CTA)",
+    out.update({"bound": "tensor", "kernel": "mpgemm_kernel<4,true,0> (4-bit, CTA pairs)",
                 "workload": "config4: prefill mpGEMM M=1024, K=4096, N in {4096, 14336}, 4-bit, group 128 "
                             "(sum of flops / sum of time; 4 rotating copies of inputs and outputs, 40 calls each)",
                 "achieved": tf, "peak": peaks["tf_burst"], "unit": "TFLOP/s", "frac": tf / peaks["tf_burst"],
