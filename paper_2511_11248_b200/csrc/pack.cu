@@ -1,5 +1,6 @@
 // Offline repack into the bit-plane layout, its inverse, and the test-only extractors.
 // Pure integer work; every result has exactly one correct value.
+#include "sm100_ptx.cuh"
 #include "common.cuh"
 #include <algorithm>
 #include <mutex>
@@ -10,21 +11,21 @@ namespace tman {
 // The whole repack is one launch, bound by HBM: codes read once, packed words written once.
 //   Plane blocks (the first `plane_blocks`): a tile of 32 strips (128 columns) x 8 words (256 k), one warp per word.
 //     A lane owns one strip: it reads the four codes of a row as one 32-bit load (a warp reads 128 bytes of a row, 32
-//     rows in flight per thread) and gathers, for every plane, the row's four bits into the byte of the word they
-//     belong to; a 4 x 4 byte transpose then gives the words of the four columns (paper Sec. 2.2: W = sum_i 2^i W_i).
+//     rows in flight per thread: five blocks an SM leave the registers for that, eight do not) and turns four rows' codes
+//     at a time into bytes of the planes' words (bit transpose); a 4 x 4 byte transpose then gives the words of the four columns (paper Sec. 2.2: W = sum_i 2^i W_i).
 //     The words go through shared memory so that eight adjacent words of a strip and plane leave as one 128-byte run:
 //     written straight from the lanes they would be 16-byte pieces (half a sector) K/2 bytes apart.
 //   Scale blocks (the rest): one thread per strip and four quantization blocks, 32 bytes of scales in one piece.
 //   The first block also writes the header and zeroes the padding between sections, so that the whole buffer is a
 //     function of the inputs.
 // Byte loads, 16-byte pieces and four launches took 65.7 us for 4096 x 14336 4-bit codes (88 MB: 13.6 us at the copy
-// rate); this takes 22.5 us.
+// rate).  With a shift and a mask per code bit and eight blocks an SM 20.6 us (2-bit 18.9); so 18.1 (17.5).
 // VEC: codes and zeros are 4-byte aligned and scales 8-byte aligned (N % 8 == 0 keeps every row so); otherwise the same
 // elements are read one by one.
 constexpr int kPackThreads = 256, kPackStrips = 32, kPackWords = 8;
 
 template <int BITS, bool VEC>
-__global__ void __launch_bounds__(kPackThreads) pack_kernel(const uint8_t *__restrict__ codes, const __half *__restrict__ scales,
+__global__ void __launch_bounds__(kPackThreads, 5) pack_kernel(const uint8_t *__restrict__ codes, const __half *__restrict__ scales,
                                                             const uint8_t *__restrict__ zeros, uint8_t *__restrict__ packed,
                                                             int K, int N, int group, int strip_tiles, int plane_blocks)
 {
@@ -43,23 +44,25 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const uint8_t *__res
                 if constexpr (VEC) u[r] = __ldcs(reinterpret_cast<const uint32_t *>(src));
                 else u[r] = (uint32_t)src[0] | ((uint32_t)src[1] << 8) | ((uint32_t)src[2] << 16) | ((uint32_t)src[3] << 24);
             }
+            // Word bit 8 b + 4 h + ph is row 8 ph + 2 b + h: byte b of a plane is, per column, a 4 x 4 bit transpose of four
+            // rows' codes, for h = 0 in the low nibbles and h = 1 in the high ones.
+            uint32_t by[4][4];                             // [plane][b]: byte c = byte b of column c's word
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                uint32_t r[4];
+#pragma unroll
+                for (int ph = 0; ph < 4; ++ph) r[ph] = bsel(0x0F0F0F0Fu, u[8 * ph + 2 * b], u[8 * ph + 2 * b + 1] << 4);
+                const uint32_t t0 = bsel(0x55555555u, r[0], r[1] << 1), t1 = bsel(0x55555555u, r[0] >> 1, r[1]);
+                const uint32_t t2 = bsel(0x55555555u, r[2], r[3] << 1), t3 = bsel(0x55555555u, r[2] >> 1, r[3]);
+                by[0][b] = bsel(0x33333333u, t0, t2 << 2);
+                by[1][b] = bsel(0x33333333u, t1, t3 << 2);
+                by[2][b] = bsel(0x33333333u, t0 >> 2, t2);
+                by[3][b] = bsel(0x33333333u, t1 >> 2, t3);
+            }
 #pragma unroll
             for (int i = 0; i < BITS; ++i) {
-                uint32_t by[4];                            // by[b]: byte c = byte b of column c's word
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    uint32_t a = 0u;
-#pragma unroll
-                    for (int r = 0; r < 32; ++r)
-                        if ((plane_bit(r) >> 3) == b) {
-                            const int to = plane_bit(r) & 7;
-                            const uint32_t t = to >= i ? u[r] << (to - i) : u[r] >> (i - to);
-                            a |= t & (0x01010101u << to);
-                        }
-                    by[b] = a;
-                }
-                const uint32_t lo01 = __byte_perm(by[0], by[1], 0x5140), hi01 = __byte_perm(by[0], by[1], 0x7362);
-                const uint32_t lo23 = __byte_perm(by[2], by[3], 0x5140), hi23 = __byte_perm(by[2], by[3], 0x7362);
+                const uint32_t lo01 = __byte_perm(by[i][0], by[i][1], 0x5140), hi01 = __byte_perm(by[i][0], by[i][1], 0x7362);
+                const uint32_t lo23 = __byte_perm(by[i][2], by[i][3], 0x5140), hi23 = __byte_perm(by[i][2], by[i][3], 0x7362);
                 const uint4 w = make_uint4(__byte_perm(lo01, lo23, 0x5410), __byte_perm(lo01, lo23, 0x7632),
                                            __byte_perm(hi01, hi23, 0x5410), __byte_perm(hi01, hi23, 0x7632));
                 // (word index XOR strip: the lanes of a store spread over all banks)
