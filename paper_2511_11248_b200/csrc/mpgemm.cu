@@ -48,6 +48,7 @@ constexpr int NUM_EPI_WARPS = 8;                // two per quarter of the tensor
 constexpr int GEMM_THREADS = 32 * (2 + NUM_DEQ_WARPS + NUM_EPI_WARPS);
 constexpr int P_PLANE_BYTES = (CH / 4) * 128;   // one plane of a packed stage (two units): a 128-byte run per strip
 constexpr int P_RING_BYTES = 64 * 1024;         // 8 stages for 2 bits, 4 for 3 and 4
+constexpr int P_LOAD_BARS = 8;                  // "loaded" barriers of the packed stages, whatever the number of their slots (see the dequantization)
 constexpr int X_RING_BYTES = 128 * 1024;        // activation ring: stages of two units (8 of up to 32 rows, 4 of up to 64) or one (4 of up to 128)
 constexpr int W_TILE_BYTES = CH * BK * 2;       // half a unit of fp16 weights in shared memory (LoadFull variant only)
 constexpr int TMEM_COLS = 512;                  // accumulator from column 0, weight buffers of 64 columns behind it
@@ -380,7 +381,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
             if (pmore) { pu = pg.u0; pend = pg.u1; pstrip = tile_ch0(pg.tile) / 4; }
         };
         auto packed_issue = [&]() {
-            const uint32_t st = pc % P_STAGES, bar = ploaded0 + 8 * st, dst = p_base + st * P_STAGE_BYTES;
+            const uint32_t bar = ploaded0 + 8 * (pc % P_LOAD_BARS), dst = p_base + pc % P_STAGES * P_STAGE_BYTES;
             if (lead) {
                 mbar_expect_tx(bar, P_STAGE_BYTES);
 #pragma unroll
@@ -494,9 +495,13 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         for (int w = 0; w < 4; ++w) p_src[w] = (uint32_t)strip * 128u + (uint32_t)c * 4u + ((uint32_t)(w ^ (strip & 3)) * 16u);
         const uint32_t half_swap = ((uint32_t)strip >> 2) & 1u;
         const uint32_t w_tmem = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)p.wcol, xst_mask = (1u << p.xst_sh) - 1u;
-        // Weight buffer of the group's next unit and its parity.  All groups see every turn of what they wait for: a group's unit
-        // before this one is four back, its wait was for a commit six (four) units before that, and loads are issued in order;
-        // no ring is so short that an unseen turn could be two behind (six weight buffers only for tiles of four units and more).
+        // Weight buffer of the group's next unit and its parity.  A wait names a turn of its barrier by the parity alone and would also
+        // pass while the turn before it is incomplete; a group does not wait for the loads of the units between its own, and these
+        // may arrive in any order.  What it knows from the unit before, four back: the weight buffer of that one was free, so the
+        // unit six (four) before it has been multiplied and every load up to there is complete.  The packed stages' "loaded" barriers
+        // take turns over eight stages, also where the ring has four slots: seven stages of one or two units lie between two turns
+        // of a barrier, at least seven units or, with six buffers (tiles of four units and more), eleven, so that the turn before is
+        // among those loads.  (Four slots with a barrier each: stages of one unit at the end of odd tiles leave turns unseen.)
         uint32_t s = (uint32_t)grp, ph = 0u;
         uint32_t pos = 0, xc0 = 0, pc0 = 0;                // units, activation stages and packed stages of the segments before
         // BPU: quantization blocks of a unit
@@ -541,7 +546,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                         }
                         if (!INT8 && u + STEP < sg.u1) fetch();
                         const uint32_t pc = pc0 + (i >> 1), ps = pc % P_STAGES;
-                        if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(ploaded0 + 8 * ps, (pc / P_STAGES) & 1u))) { ok = false; break; }
+                        if (!TMAN_STAMPED_WAIT(wait_a, mbar_wait(ploaded0 + 8 * (pc % P_LOAD_BARS), (pc / P_LOAD_BARS) & 1u))) { ok = false; break; }
                         uint32_t w4[4][BITS];
                         const uint32_t stage = ps * P_STAGE_BYTES + (((i & 1u) ^ half_swap) << 6);
 #pragma unroll

@@ -80,6 +80,22 @@ def test_edges_of_the_transposed_kernel(M, K, N, bits, G):
     assert rel_err(got, orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)) <= 1e-3
 
 
+# Several tiles a worker whose K / 128 is odd, whole and in spans, with six and with four weight buffers: the last packed stage of a
+# tile holds one unit, so that a group of dequantization warps does not see every turn of the ring of 3- and 4-bit weights.
+ODD_UNITS = [(60, 1152, 40008, 4, 128), (1000, 640, 9992, 3, 64), (700, 1408, 12296, 4, 32), (260, 1152, 20488, 3, 128)]
+
+
+@pytest.mark.parametrize("M,K,N,bits,G", ODD_UNITS)
+def test_several_tiles_of_odd_units(M, K, N, bits, G):
+    plan = B.tman_debug_gemm_plan(M, K, N, bits, G)
+    assert plan["tiles_m"] * plan["tiles_n"] > plan["workers"] and not plan["pieces"], plan
+    c = synth.small_case(M, K, N, bits, G, seed=13 * M + K + N + bits)
+    y = run_gemm(c)
+    rows = block_rows(M, c.seed)
+    # rounding as in test_edges_of_the_transposed_kernel
+    check_every_output(c, y, rows, orc.mpgemm_rows(c.x, c.codes, c.scales, c.zeros, c.group, rows), tol=1e-3)
+
+
 # Long K and few tiles: every tile's k-blocks go to several workers, which exchange fp32 chunks through
 # the workspace and share the summing.  Pairs of CTAs with two and one row block, a single CTA, ragged
 # M and N, every bit width; compared element by element.
