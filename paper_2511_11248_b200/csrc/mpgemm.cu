@@ -48,7 +48,7 @@ constexpr int NUM_EPI_WARPS = 8;                // two per quarter of the tensor
 constexpr int GEMM_THREADS = 32 * (2 + NUM_DEQ_WARPS + NUM_EPI_WARPS);
 constexpr int P_PLANE_BYTES = (CH / 4) * 128;   // one plane of a packed stage (two units): a 128-byte run per strip
 constexpr int P_RING_BYTES = 64 * 1024;         // 8 stages for 2 bits, 4 for 3 and 4
-constexpr int P_LOAD_BARS = 8;                  // "loaded" barriers of the packed stages, whatever the number of their slots (see the dequantization)
+constexpr int P_LOAD_BARS = 8, X_LOAD_BARS = 8; // "loaded" barriers of the packed stages and, integer path, of the activations', whatever the number of slots (see the dequantization)
 constexpr int X_RING_BYTES = 128 * 1024;        // activation ring: stages of two units (8 of up to 32 rows, 4 of up to 64) or one (4 of up to 128)
 constexpr int W_TILE_BYTES = CH * BK * 2;       // half a unit of fp16 weights in shared memory (LoadFull variant only)
 constexpr int TMEM_COLS = 512;                  // accumulator from column 0, weight buffers of 64 columns behind it
@@ -407,7 +407,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                     --ahead;
                     while (pmore && warp_all(mbar_test(packed_bar(), packed_par()))) packed_issue();
                 }
-                const uint32_t st = xc & xst_mask, bar = xloaded0 + 8 * st;
+                const uint32_t st = xc & xst_mask, bar = xloaded0 + 8 * (INT8 ? xc % X_LOAD_BARS : st);
                 if constexpr (V == kGemmSequential)
                     if (xc > 0 && !warp_all(mbar_wait(xempty0 + 8 * ((xc - 1) & xst_mask), ((xc - 1) >> p.xst_sh) & 1u))) { ok = false; break; }
                 if (!TMAN_STAMPED_WAIT(wait_a, warp_all(mbar_wait(xempty0 + 8 * st, ((xc >> p.xst_sh) & 1u) ^ 1u)))) { ok = false; break; }
@@ -498,10 +498,12 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         // Weight buffer of the group's next unit and its parity.  A wait names a turn of its barrier by the parity alone and would also
         // pass while the turn before it is incomplete; a group does not wait for the loads of the units between its own, and these
         // may arrive in any order.  What it knows from the unit before, four back: the weight buffer of that one was free, so the
-        // unit six (four) before it has been multiplied and every load up to there is complete.  The packed stages' "loaded" barriers
-        // take turns over eight stages, also where the ring has four slots: seven stages of one or two units lie between two turns
-        // of a barrier, at least seven units or, with six buffers (tiles of four units and more), eleven, so that the turn before is
-        // among those loads.  (Four slots with a barrier each: stages of one unit at the end of odd tiles leave turns unseen.)
+        // unit `wbufs` before it has been multiplied and every load up to there is complete.  The packed stages' "loaded" barriers
+        // take turns over eight stages, also where the ring has four slots: seven stages lie between two turns of a barrier, at least
+        // seven units, or, with six or eight buffers (tiles of four or eight units and more), eleven or thirteen, so that the turn
+        // before is among those loads.  (Four slots with a barrier each: the stages of one unit that end odd tiles leave turns
+        // unseen.)  So do the activations' on the integer path.  On the fp16 path a barrier per slot is enough: this unit's weight
+        // buffer is waited for first, so every load up to the unit six (four) back is complete, and the slot's turn before is no later.
         uint32_t s = (uint32_t)grp, ph = 0u;
         uint32_t pos = 0, xc0 = 0, pc0 = 0;                // units, activation stages and packed stages of the segments before
         // BPU: quantization blocks of a unit
@@ -532,7 +534,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                 if (!INT8 && first < sg.u1) fetch();
                 for (int u = first; u < sg.u1; u += STEP) {
                     const uint32_t i = (uint32_t)(u - sg.u0), xc = xc0 + (i >> p.xu_sh);
-                    const uint32_t xbar = xloaded0 + 8 * (xc & xst_mask), xpar = (xc >> p.xst_sh) & 1u;
+                    const uint32_t xbar = xloaded0 + 8 * (INT8 ? xc % X_LOAD_BARS : xc & xst_mask), xpar = (INT8 ? xc / X_LOAD_BARS : xc >> p.xst_sh) & 1u;
                     if constexpr (V != kGemmLoadFull) {
                         BlockConsts t[BPU];
                         __half s_cur[BPU];
@@ -584,8 +586,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                         tcgen05_wait_st();
                     }
                     tcgen05_fence_before();
-                    // the MMA of this unit also reads this CTA's activations (their stage's turn before was over when the
-                    // weight buffer became free: their ring is no shorter than the weight buffers')
+                    // the MMA of this unit also reads this CTA's activations
                     if (!TMAN_STAMPED_WAIT(wait_b, mbar_wait(xbar, xpar))) { ok = false; break; }
                     __syncwarp();
                     if (lane == 0) arrive_lead(full_lead + 8 * s);

@@ -14,16 +14,19 @@ ORDER = ("packed", "buffer", "x")                             # a group's waits 
 SRC = open(os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_11248_b200", "csrc", "mpgemm.cu")).read()
 
 
-def barriers_of_packed_stages(p_stages):
-    """Over how many stages the kernel's "loaded" barriers of the packed words take turns."""
-    own = re.search(r"constexpr int P_LOAD_BARS = (\d+);", SRC)
-    if own is None:
-        return p_stages                                       # a barrier for every slot of the ring
-    assert SRC.count("ploaded0 + 8 * (pc % P_LOAD_BARS)") == 2 and "(pc / P_LOAD_BARS) & 1u" in SRC
+def load_barriers(ring, stages, int8):
+    """Over how many stages the kernel's "loaded" barriers of a ring take turns (P packed words, X activations)."""
+    own = re.search(r"constexpr int [^;]*\b%s_LOAD_BARS = (\d+)" % ring, SRC)
+    if own is None or (ring == "X" and not int8):
+        return stages                                         # a barrier for every slot of the ring
+    if ring == "P":
+        assert SRC.count("ploaded0 + 8 * (pc % P_LOAD_BARS)") == 2 and "(pc / P_LOAD_BARS) & 1u" in SRC
+    else:
+        assert SRC.count("xloaded0 + 8 * (INT8 ? xc % X_LOAD_BARS :") == 2 and "(INT8 ? xc / X_LOAD_BARS :" in SRC
     return int(own.group(1))
 
 
-def wrong_turn(segments, p_stages, p_bars, wbufs, xu, x_stages, withheld):
+def wrong_turn(segments, p_stages, wbufs, xu, x_stages, withheld, int8):
     """segments: units of each.  withheld: ("packed" | "x", stage) that never arrives, ("mma", unit) that is never issued
     or ("group", unit) that is never begun.
     Returns the wait (kind, unit) that passes on the wrong turn, or None."""
@@ -42,6 +45,7 @@ def wrong_turn(segments, p_stages, p_bars, wbufs, xu, x_stages, withheld):
     units = len(p_of)
     read, ready, done = [False] * units, [False] * units, 0   # words in registers; weights and activations handed on; MMAs committed
     loads = {"packed": [0, len(parts)], "x": [0, len(x_last)]}
+    bars = {"packed": load_barriers("P", p_stages, int8), "x": load_barriers("X", x_stages, int8)}
     at = [[g, 0] for g in range(GROUPS)]                      # a group's unit, the wait it stands at
 
     def loaded(kind, stage):
@@ -68,7 +72,7 @@ def wrong_turn(segments, p_stages, p_bars, wbufs, xu, x_stages, withheld):
                     passes = u < wbufs or u - wbufs < done
                     wrong = u >= 2 * wbufs and u - 2 * wbufs >= done
                 else:
-                    stage, turns = (p_of[u], p_bars) if kind == "packed" else (x_of[u], x_stages)
+                    stage, turns = (p_of if kind == "packed" else x_of)[u], bars[kind]
                     passes = loaded(kind, stage)
                     wrong = stage >= turns and not loaded(kind, stage - turns)
                 if wrong:
@@ -97,20 +101,28 @@ def walks(nu):
                     yield [first, last]
 
 
-def check(segments, p_stages, p_bars, wbufs, xu, x_stages):
+def check(segments, p_stages, wbufs, xu, x_stages, int8=False):
     for kind in ("packed", "x", "mma", "group"):
         for i in range(sum(segments)):
-            got = wrong_turn(segments, p_stages, p_bars, wbufs, xu, x_stages, (kind, i))
-            assert got is None, (segments, p_stages, p_bars, wbufs, xu, x_stages, (kind, i), got)
+            got = wrong_turn(segments, p_stages, wbufs, xu, x_stages, (kind, i), int8)
+            assert got is None, (segments, p_stages, wbufs, xu, x_stages, (kind, i), got)
 
 
-# (weight buffers, units and stages of activations, admitted unit counts of a tile): what launch_mpgemm_variant chooses
+# (weight buffers, units and stages of activations, admitted unit counts of a tile): what launch_mpgemm_variant chooses,
+# and launch_mpgemm_ternary_i8 (whole tiles only, 2-bit weights)
 RINGS = {
     "fp16, up to 64 tokens": (6, 2, 8, lambda nu: nu >= 4),
     "fp16, up to 128 tokens": (6, 2, 4, lambda nu: nu >= 4),
     "fp16, up to 64 tokens, short K": (4, 2, 8, lambda nu: nu < 4),
     "fp16, up to 128 tokens, short K": (4, 2, 4, lambda nu: nu < 4),
     "fp16, up to 256 tokens": (4, 1, 4, lambda nu: True),
+}
+RINGS_INT8 = {
+    "up to 128 tokens": (8, 2, 8, lambda nu: nu >= 8),
+    "up to 128 tokens, short K": (4, 2, 8, lambda nu: nu < 8),
+    "up to 192 tokens": (4, 2, 4, lambda nu: True),
+    "up to 256 tokens": (8, 2, 4, lambda nu: nu >= 8),
+    "up to 256 tokens, short K": (4, 2, 4, lambda nu: nu < 8),
 }
 
 
@@ -120,4 +132,11 @@ def test_no_wait_for_packed_words_passes_on_the_turn_before(name):
     for p_stages in (8, 4):                                   # 2-bit weights; 3 and 4
         for nu in (n for n in (1, 2, 3, 4, 5, 6, 7, 9, 12) if admits(n)):
             for segments in walks(nu):
-                check(segments, p_stages, barriers_of_packed_stages(p_stages), wbufs, xu, x_stages)
+                check(segments, p_stages, wbufs, xu, x_stages)
+
+
+@pytest.mark.parametrize("name", list(RINGS_INT8))
+def test_no_wait_for_activations_of_the_integer_path_passes_on_the_turn_before(name):
+    wbufs, xu, x_stages, admits = RINGS_INT8[name]
+    for nu in (n for n in (1, 2, 3, 4, 5, 7, 8, 9, 11, 13, 20) if admits(n)):
+        check([nu] * (3 + 24 // nu), 8, wbufs, xu, x_stages, int8=True)

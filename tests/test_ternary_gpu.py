@@ -210,6 +210,11 @@ def test_int8_prefill_edges(M, K, N, group):
     test_int8_prefill_matches_the_integer_oracle(M, K, N, group)
 
 
+def test_int8_prefill_of_large_tiles_of_odd_units():
+    # tiles of 224 tokens (eight weight buffers, four activation stages of two units), 27 units each, two tiles for most workers
+    test_int8_prefill_matches_the_integer_oracle(1024, 3456, 6912, 128)
+
+
 @pytest.mark.parametrize("M,K,N,group", [(2, 1024, 40, 64), (3, 2560, 264, 128), (4, 6912, 2560, 128), (5, 1152, 72, 32),
                                          (8, 2560, 6912, 64), (7, 16384, 16, 128)])
 def test_ternary_decode_with_several_rows(M, K, N, group):
