@@ -115,7 +115,9 @@ tman_status tman_unpack_weights(const void *packed, size_t packed_bytes,
  * stream order), by a memory copy, or by any kernel that does not signal early completion.  What
  * is not: a kernel of the caller's own that calls cudaTriggerProgrammaticLaunchCompletion (PTX
  * griddepcontrol.launch_dependents) and then writes the packed buffer, directly followed by a decode
- * call on the same stream -- put an event or another kernel between them.  Activations and the
+ * call on the same stream -- put an event or another kernel (not a decode) between them; tman_mpgemm,
+ * tman_mpgemm_ternary_i8 and the row quantizations, which may begin early as well, will do: they let
+ * their successor begin only when their own predecessor has completed.  Activations and the
  * workspace have no such rule: they are read only after the predecessor has completed. */
 
 /* Decode (paper Sec. 2.2 "Bit-serial table lookup", Fig. 2; Sec. 4.3): activation tables are

@@ -295,9 +295,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 50);
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (the shuffle tells the compiler that it is uniform)
 
-    // The next kernel of the stream may set itself up while this one runs, as this one does now; nothing below the wait
-    // starts before the previous kernel has ended.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // (down to the wait: beside the previous kernel of the stream, without a look at memory)
     if (threadIdx.x == 0) {
         for (int s = 0; s < 8; ++s) {
             mbar_init(ploaded0 + 8 * s, 1);
@@ -336,6 +334,9 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
     if constexpr (PAIR)
         if (tmem_base == 0xFFFFFFFFu) tmem_base = ld_shared_cluster_u32(mapa_u32(smem_u32(tmem_slot), rank ^ 1u));
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The next kernel of the stream may start now, not before: a decode reads its weights at once, and who wrote them may be
+    // the kernel this one has waited for.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     bool ok = tmem_base != 0xFFFFFFFFu;
     const bool run = (smem_u32(smem) & 1023u) == 0u;       // the swizzled tiles need 1 KB alignment (same in every CTA)

@@ -1099,10 +1099,10 @@ tman_status launch_mpgemv_grouped(int count, const void *const *packed, const vo
 // processor", IBM J. Res. Dev. 34, 1990, division by a correctly rounded reciprocal: q' = q + (x - q s) y, the remainder
 // exact by fused multiply-add; the first step brings q, off by at most 1.5 units in the last place, to a neighbour of the
 // quotient, the second rounds it).  No intermediate leaves the normal range: 2^-24 <= |x| < 2^16 and 2^-40 < s < 2^10.
-// Launched so that it may start while its predecessor drains, and lets its successor do the same.
+// Launched so that it may start while its predecessor drains; its successor may start when the predecessor has ended.
 // Against two passes with a full division per value in one CTA of 512 threads a row: 2048 rows of 2560 and the INT8
 // product with 6912 channels after them 61.3 -> 50.2 us; one row and its decode, mean of 2560 x 6912 and 6912 x 2560,
-// 7.6 -> 6.1 us.
+// 7.4 -> 5.7 us (6.0 with the successor let go before the wait, which suited two to four rows better: 7.7 against 8.0).
 template <typename OUT>
 __device__ __forceinline__ void store_eight(OUT *out, const int (&q)[8])
 {
@@ -1122,8 +1122,8 @@ __global__ void __launch_bounds__(1024) quantize_rows_regs_kernel(const __half *
                                                                   OUT *__restrict__ a, float *__restrict__ s_a)
 {
     __shared__ float red[32];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (after the wait: a decode that follows reads its weights at once)
     const uint4 *row = reinterpret_cast<const uint4 *>(x) + (size_t)blockIdx.x * nvec;
     OUT *out = a + (size_t)blockIdx.x * nvec * 8;
     uint4 v[VPT];
