@@ -316,29 +316,32 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
         prefetch_tensormap(&tmap_x);
         prefetch_tensormap(V == kGemmLoadFull ? &tmap_wf : &tmap_w);
     }
-    __syncthreads();
-    if (warp == 1) {
-        if constexpr (PAIR) {
-            tcgen05_alloc2(smem_u32(tmem_slot), TMEM_COLS);
-            tcgen05_relinquish2();
-        } else {
-            tcgen05_alloc(smem_u32(tmem_slot), TMEM_COLS);
-            tcgen05_relinquish();
-        }
-    }
-    tcgen05_fence_before();
-    __syncthreads();
-    if constexpr (PAIR) cluster_sync_all();            // both CTAs' barriers and tensor memory are set up
-    tcgen05_fence_after();
-    uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_slot);
-    if constexpr (PAIR)
-        if (tmem_base == 0xFFFFFFFFu) tmem_base = ld_shared_cluster_u32(mapa_u32(smem_u32(tmem_slot), rank ^ 1u));
+    if constexpr (PAIR) cluster_sync_all();            // both CTAs' barriers are set up
+    else __syncthreads();
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    // The next kernel of the stream may start now, not before: a decode reads its weights at once, and who wrote them may be
-    // the kernel this one has waited for.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-    bool ok = tmem_base != 0xFFFFFFFFu;
+    // Tensor memory only now: the previous kernel may be one that signals early and allocates its own on this SM afterwards; it
+    // would wait for this one's columns, and this one for its end.  (Warp 0 needs none and starts its loads meanwhile, which hides the
+    // allocation: with all warps behind it every call took 0.8 us longer.)  The next kernel may start only then, for the same reason,
+    // and because a decode reads its weights at once, which may have been written by the kernel this one has waited for.
+    uint32_t tmem_base = 0xFFFFFFFFu;
+    bool ok = true;
+    if (warp != 0) {
+        if (warp == 1) {
+            if constexpr (PAIR) {
+                tcgen05_alloc2(smem_u32(tmem_slot), TMEM_COLS);
+                tcgen05_relinquish2();
+            } else {
+                tcgen05_alloc(smem_u32(tmem_slot), TMEM_COLS);
+                tcgen05_relinquish();
+            }
+        }
+        tcgen05_fence_before();
+        asm volatile("bar.sync 1, %0;" ::"n"(GEMM_THREADS - 32) : "memory");
+        tcgen05_fence_after();
+        tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_slot);
+        ok = tmem_base != 0xFFFFFFFFu;
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
     const bool run = (smem_u32(smem) & 1023u) == 0u;       // the swizzled tiles need 1 KB alignment (same in every CTA)
     if (!run && threadIdx.x == 0 && blockIdx.x == 0) atomicCAS(p.status, 0u, (uint32_t)TMAN_ERR_LAYOUT);
     long long wait_a = 0, wait_b = 0;                  // clocks in this thread's waits (time-stamp builds only)

@@ -95,18 +95,12 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// Arrive on a barrier of another CTA of the cluster.  Only the signal crosses CTAs: the data a
-// CTA's tensor core reads is in that CTA's own shared memory, made visible by the writer's
-// fence.proxy.async, so no cluster-scope release (a slow memory barrier) is needed here.
+// Arrive on a barrier of another CTA of the cluster.  Only the signal crosses CTAs: the weights a CTA's half of a paired MMA reads are
+// in that CTA's own tensor memory, whose writer has waited for its stores (tcgen05.wait::st) and ordered them before this arrive
+// (tcgen05.fence::before_thread_sync), so no cluster-scope release (a slow memory barrier) is needed here.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ uint32_t ld_shared_cluster_u32(uint32_t cluster_addr)
-{
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
-    return v;
 }
 __device__ __forceinline__ void tcgen05_alloc2(uint32_t dst_smem, uint32_t ncols)
 {

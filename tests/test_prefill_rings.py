@@ -140,3 +140,13 @@ def test_no_wait_for_activations_of_the_integer_path_passes_on_the_turn_before(n
     wbufs, xu, x_stages, admits = RINGS_INT8[name]
     for nu in (n for n in (1, 2, 3, 4, 5, 7, 8, 9, 11, 13, 20) if admits(n)):
         check([nu] * (3 + 24 // nu), 8, wbufs, xu, x_stages, int8=True)
+
+
+def test_tensor_memory_is_taken_after_the_wait_and_before_the_signal():
+    # A predecessor that signals early and allocates tensor memory on the same SM afterwards would wait for this kernel's columns,
+    # and this kernel for its end; the same between this kernel and a successor of that kind.
+    kernel = SRC[SRC.index("mpgemm_kernel(const __grid_constant__"):SRC.index("// ---- stage 1")]
+    wait, signal = (kernel.index("griddepcontrol." + w) for w in ("wait;", "launch_dependents;"))
+    allocs = [m.start() for m in re.finditer(r"tcgen05_alloc2?\(", kernel)]
+    assert len(allocs) == 2 and wait < min(allocs) and max(allocs) < signal
+    assert kernel.count("griddepcontrol.") == 2
