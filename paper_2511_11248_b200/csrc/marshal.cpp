@@ -96,11 +96,15 @@ PyObject *py_grouped(PyObject *, PyObject *const *args, Py_ssize_t n)
     Py_ssize_t count = 0;
     bool ok = true;
     for (int i = 0; i < 3 && ok; ++i) {
+        if (i == 0) {                           // packed_list needs a length, as it does for len()
+            count = PyObject_Size(args[at[0]]);
+            ok = count >= 0;
+            if (!ok) break;
+        }
         seq[i] = PySequence_Fast(args[at[i]], "expected a sequence");
         ok = seq[i] != nullptr;
-        if (ok && i == 0) count = PySequence_Fast_GET_SIZE(seq[0]);
-        if (ok && PySequence_Fast_GET_SIZE(seq[i]) < count) {
-            PyErr_SetString(PyExc_IndexError, "y_list and N_list need an entry for every matrix");
+        if (ok && PySequence_Fast_GET_SIZE(seq[i]) != count) {
+            PyErr_SetString(PyExc_IndexError, "packed_list, y_list and N_list need an entry for every matrix and no more");
             ok = false;
         }
     }

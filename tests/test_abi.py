@@ -225,3 +225,29 @@ def test_marshalled_calls_report_status_and_bad_arguments(lib):
         fast.mpgemv(t, 3, t, 1, 128, 8, 4, 64, t, 0)
     with pytest.raises(IndexError):
         fast.mpgemv_grouped([t, t], t, [t], 1, 128, [8, 8], 4, 64, t, 0)
+
+
+def host_tensor():
+    """Host memory on a 256-byte boundary for calls that are refused before anything reads it, and a stream for the binding."""
+    torch = pytest.importorskip("torch")
+    whole = torch.zeros((1 << 16) + 256, dtype=torch.uint8)
+
+    class Stream:
+        cuda_stream = 0
+    return torch, whole[(-whole.data_ptr()) % 256:][:1 << 16], Stream()
+
+
+def test_grouped_call_refuses_lists_of_other_lengths(lib):
+    # (nine rows: a call that gets as far as the library is refused there with TMAN_ERR_SHAPE)
+    from paper_2511_11248_b200 import binding as B
+    _, t, s = host_tensor()
+    with pytest.raises(IndexError):
+        B.tman_mpgemv_grouped([t, t], t, [t, t, t], 9, 128, [8, 8], 4, 64, t, s)
+    with pytest.raises(IndexError):
+        B.tman_mpgemv_grouped([t, t], t, [t, t], 9, 128, [8, 8, 8], 4, 64, t, s)
+    with pytest.raises(TypeError):
+        B.tman_mpgemv_grouped((p for p in (t, t)), t, [t, t], 9, 128, [8, 8], 4, 64, t, s)
+    for ys, ns in (([t, t], [8, 8]), (iter([t, t]), (n for n in (8, 8)))):
+        with pytest.raises(B.TmanError) as e:
+            B.tman_mpgemv_grouped([t, t], t, ys, 9, 128, ns, 4, 64, t, s)
+        assert e.value.status == 2
