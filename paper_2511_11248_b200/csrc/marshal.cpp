@@ -17,33 +17,64 @@ namespace {
 
 enum { F_GEMV, F_GROUPED, F_GEMM, F_QUANT, F_QUANT_I8, F_TERNARY, F_TERNARY_I8, F_PACK, F_COUNT };
 void *g_fn[F_COUNT];
-PyObject *g_data_ptr, *g_nbytes;               // interned attribute names
+PyObject *g_data_ptr, *g_nbytes, *g_numel, *g_element_size;                // interned attribute names
 
 // Address of a tensor (None: 0).  False with a Python error set when the object has none.
 bool address(PyObject *t, void **out)
 {
     if (t == Py_None) { *out = nullptr; return true; }
     PyObject *r = PyObject_CallMethodNoArgs(t, g_data_ptr);
+    if (r && !PyLong_Check(r)) {                // another integer type, say of NumPy
+        PyObject *n = PyNumber_Long(r);
+        Py_DECREF(r);
+        r = n;
+    }
     if (!r) return false;
     *out = PyLong_AsVoidPtr(r);
     Py_DECREF(r);
     return !PyErr_Occurred();
 }
+// Size of a tensor, or of any object with the numel() and element_size() of one.
 bool bytes_of(PyObject *t, size_t *out)
 {
     PyObject *r = PyObject_GetAttr(t, g_nbytes);
-    if (!r) return false;
+    if (!r) {
+        if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return false;
+        PyErr_Clear();
+        PyObject *n = PyObject_CallMethodNoArgs(t, g_numel), *e = n ? PyObject_CallMethodNoArgs(t, g_element_size) : nullptr;
+        r = e ? PyNumber_Multiply(n, e) : nullptr;
+        Py_XDECREF(n);
+        Py_XDECREF(e);
+        if (!r) return false;
+    }
     *out = PyLong_AsSize_t(r);
     Py_DECREF(r);
     return !PyErr_Occurred();
 }
 bool integer(PyObject *o, int *out)
 {
-    int overflow = 0;
-    const long v = PyLong_AsLongAndOverflow(o, &overflow);
-    if (v == -1 && PyErr_Occurred()) return false;
-    *out = (int)v;                              // like ctypes' c_int: the low 32 bits
+    const unsigned long v = PyLong_AsUnsignedLongMask(o);
+    if (v == (unsigned long)-1 && PyErr_Occurred()) return false;
+    *out = (int)(unsigned)v;                    // like ctypes' c_int: the low 32 bits
     return true;
+}
+// The same of whatever int() takes (an entry of N_list: a float, an element of an array or a tensor)
+bool integer_of(PyObject *o, int *out)
+{
+    if (PyLong_Check(o)) return integer(o, out);
+    PyObject *n = PyNumber_Long(o);
+    const bool ok = n && integer(n, out);
+    Py_XDECREF(n);
+    return ok;
+}
+// Whatever float() takes
+bool real_of(PyObject *o, double *out)
+{
+    PyObject *f = PyNumber_Float(o);
+    if (!f) return false;
+    *out = PyFloat_AsDouble(f);
+    Py_DECREF(f);
+    return !PyErr_Occurred();
 }
 
 // Reads arguments left to right; the first failure sticks.
@@ -54,7 +85,7 @@ struct Reader {
     void *ptr() { void *p = nullptr; ok = ok && address(*a++, &p); return p; }
     void *buf(size_t *n) { void *p = nullptr; ok = ok && address(*a, &p) && bytes_of(*a, n); ++a; return p; }
     int num() { int v = 0; ok = ok && integer(*a++, &v); return v; }
-    float real() { float v = 0.f; if (ok) { const double d = PyFloat_AsDouble(*a++); ok = !PyErr_Occurred(); v = (float)d; } return v; }
+    float real() { double v = 0.0; ok = ok && real_of(*a++, &v); return (float)v; }
     tman_stream_t stream() { void *p = nullptr; if (ok) { p = PyLong_AsVoidPtr(*a++); ok = !PyErr_Occurred(); } return (tman_stream_t)p; }
 };
 
@@ -115,7 +146,7 @@ PyObject *py_grouped(PyObject *, PyObject *const *args, Py_ssize_t n)
     for (Py_ssize_t i = 0; ok && i < count && i < MAX; ++i) {
         void *p = nullptr;
         ok = address(PySequence_Fast_GET_ITEM(seq[0], i), &p) && bytes_of(PySequence_Fast_GET_ITEM(seq[0], i), &pb[i]) &&
-             address(PySequence_Fast_GET_ITEM(seq[1], i), &y[i]) && integer(PySequence_Fast_GET_ITEM(seq[2], i), &Ns[i]);
+             address(PySequence_Fast_GET_ITEM(seq[1], i), &y[i]) && integer_of(PySequence_Fast_GET_ITEM(seq[2], i), &Ns[i]);
         pk[i] = p;
     }
     for (int i = 0; i < 3; ++i) Py_XDECREF(seq[i]);
@@ -227,6 +258,8 @@ PyMODINIT_FUNC PyInit__marshal(void)
 {
     g_data_ptr = PyUnicode_InternFromString("data_ptr");
     g_nbytes = PyUnicode_InternFromString("nbytes");
-    if (!g_data_ptr || !g_nbytes) return nullptr;
+    g_numel = PyUnicode_InternFromString("numel");
+    g_element_size = PyUnicode_InternFromString("element_size");
+    if (!g_data_ptr || !g_nbytes || !g_numel || !g_element_size) return nullptr;
     return PyModule_Create(&module);
 }

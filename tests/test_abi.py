@@ -251,3 +251,39 @@ def test_grouped_call_refuses_lists_of_other_lengths(lib):
         with pytest.raises(B.TmanError) as e:
             B.tman_mpgemv_grouped([t, t], t, ys, 9, 128, ns, 4, 64, t, s)
         assert e.value.status == 2
+
+
+def test_marshalled_calls_take_what_int_and_float_take(lib):
+    """Buffers that have a tensor's data_ptr(), numel() and element_size() only, output widths as any kind of number, a weight scale
+    as a text, integers beyond 32 bits cut to their low bits: every call reaches the library (nine rows: TMAN_ERR_SHAPE)."""
+    np = pytest.importorskip("numpy")
+    torch, t, s = host_tensor()
+    from paper_2511_11248_b200 import binding as B
+
+    class Buffer:
+        def data_ptr(self):
+            return np.int64(t.data_ptr())
+
+        def numel(self):
+            return t.numel() // 4
+
+        def element_size(self):
+            return 4
+
+    b = Buffer()
+    calls = [lambda: B.tman_mpgemv(b, b, b, 9, 128, 8, 4, 64, b, s),
+             lambda: B.tman_mpgemv(t, t, t, 2 ** 70 + 9, 128, 8, 4, 64, t, s),
+             lambda: B.tman_mpgemv_grouped([b, b], b, [b, b], 9, 128, [8, 8], 4, 64, b, s),
+             lambda: B.tman_mpgemv_ternary(t, t, t, "0.5", t, None, 9, 128, 8, 64, t, s),
+             lambda: B.tman_mpgemv_ternary(t, t, t, torch.tensor(0.5), t, None, 9, 128, 8, 64, t, s)]
+    for ns in ([8.0, "8"], np.array([8.0, 8.0]), np.array([8, 8]), torch.tensor([8.0, 8.0])):
+        calls.append(lambda ns=ns: B.tman_mpgemv_grouped([t, t], t, [t, t], 9, 128, ns, 4, 64, t, s))
+    for call in calls:
+        with pytest.raises(B.TmanError) as e:
+            call()
+        assert e.value.status == 2
+    with pytest.raises(B.TmanError) as e:                     # the size is read: too small for the packed weights
+        B.tman_mpgemv(type("Small", (Buffer,), {"numel": lambda self: 75})(), t, t, 1, 128, 8, 4, 64, t, s)
+    assert e.value.status == 4
+    with pytest.raises(AttributeError):
+        B.tman_mpgemv(None, t, t, 1, 128, 8, 4, 64, t, s)
