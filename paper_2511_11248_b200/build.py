@@ -30,8 +30,8 @@ def _stale(lib: str = LIB) -> bool:
 
 def build_marshal(force: bool = False) -> str:
     """The CPython extension that binding.py calls the hot entry points through."""
-    src = os.path.join(CSRC, "marshal.cpp")
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= os.path.getmtime(src):
+    src, header = os.path.join(CSRC, "marshal.cpp"), os.path.join(ROOT, "include", "tman.h")      # (the header: the prototypes it calls by)
+    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL) >= max(os.path.getmtime(src), os.path.getmtime(header)):
         return MARSHAL
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"],
            "-I", os.path.join(ROOT, "include"), src, "-o", MARSHAL]

@@ -287,3 +287,19 @@ def test_marshalled_calls_take_what_int_and_float_take(lib):
     assert e.value.status == 4
     with pytest.raises(AttributeError):
         B.tman_mpgemv(None, t, t, 1, 128, 8, 4, 64, t, s)
+
+
+def test_marshalling_is_rebuilt_when_the_header_changes(lib, monkeypatch, tmp_path):
+    # it calls the library by the header's prototypes; a compiler that does nothing tells whether it would have been built
+    from paper_2511_11248_b200 import build
+    header = tmp_path / "include" / "tman.h"
+    header.parent.mkdir()
+    header.write_text("")
+    monkeypatch.setattr(build, "ROOT", str(tmp_path))
+    monkeypatch.setenv("CXX", "false")                        # (an error, if it is called)
+    built = os.path.getmtime(build.MARSHAL)
+    os.utime(header, (built - 10, built - 10))
+    assert build.build_marshal() == build.MARSHAL
+    os.utime(header, (built + 10, built + 10))
+    with pytest.raises(RuntimeError):
+        build.build_marshal()
