@@ -1174,16 +1174,26 @@ __global__ void __launch_bounds__(1024) quantize_rows_regs_kernel(const __half *
     }
 }
 
-// Any K and rows longer than the registers of a CTA hold: two passes over the row, element by element.
-template <typename OUT>
+// Any K and rows longer than the registers of a CTA hold: two passes over the row (the second from L1/L2), eight values at a time
+// where the rows allow 16-byte accesses (VEC: K % 8 == 0), else one by one.  2048 rows of 32776: 76.7 us, one by one 177.6; one row
+// of 65536: 9.9 and 21.6.
+template <typename OUT, bool VEC>
 __global__ void __launch_bounds__(1024) quantize_rows_kernel(const __half *__restrict__ x, int K, int qmax,
                                                              OUT *__restrict__ a, float *__restrict__ s_a)
 {
     __shared__ float red[32];
     const __half *row = x + (size_t)blockIdx.x * K;
     OUT *out = a + (size_t)blockIdx.x * K;
+    const int nvec = VEC ? K >> 3 : 0;
+    const uint4 *row8 = reinterpret_cast<const uint4 *>(row);
     float amax = 0.f;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) amax = fmaxf(amax, fabsf(__half2float(row[k])));
+    for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+        const uint4 q = __ldg(row8 + i);
+        const __half2 *h = reinterpret_cast<const __half2 *>(&q);
+        const __half2 m = __hmax2(__hmax2(__habs2(h[0]), __habs2(h[1])), __hmax2(__habs2(h[2]), __habs2(h[3])));
+        amax = fmaxf(amax, fmaxf(__low2float(m), __high2float(m)));
+    }
+    for (int k = 8 * nvec + threadIdx.x; k < K; k += blockDim.x) amax = fmaxf(amax, fabsf(__half2float(row[k])));
     for (int mask = 16; mask > 0; mask >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, mask));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = amax;
     __syncthreads();
@@ -1196,10 +1206,19 @@ __global__ void __launch_bounds__(1024) quantize_rows_kernel(const __half *__res
     amax = red[0];
     const float scale = amax > 0.f ? __fdiv_rn(amax, (float)qmax) : 1.f;
     if (threadIdx.x == 0) s_a[blockIdx.x] = scale;
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        const int r = __float2int_rn(__fdiv_rn(__half2float(row[k]), scale));
-        out[k] = (OUT)max(-qmax, min(qmax, r));
+    auto quant = [&](__half v) {
+        const int r = __float2int_rn(__fdiv_rn(__half2float(v), scale));
+        return (int)max(-qmax, min(qmax, r));
+    };
+    for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+        const uint4 q = __ldg(row8 + i);
+        const __half *h = reinterpret_cast<const __half *>(&q);
+        int o[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) o[e] = quant(h[e]);
+        store_eight<OUT>(out + (size_t)i * 8, o);
     }
+    for (int k = 8 * nvec + threadIdx.x; k < K; k += blockDim.x) out[k] = (OUT)quant(row[k]);
 }
 
 template <typename OUT>
@@ -1209,12 +1228,13 @@ static tman_status launch_quantize(const void *x, int M, int K, int qmax, OUT *a
     const int nvec = K / 8;
     // Few rows: the latency of one row counts, every vector its own thread.  Many rows: four vectors a thread, so that a
     // row's reduction is spread over fewer threads (2048 rows of 2560: 96 threads; the limit of 1024 threads holds 8 x 4
-    // values each, longer rows go element by element).
+    // values each, longer rows are read twice).
     const bool few = M <= 2 * kGemvPlanSms && nvec <= 1024;
     const int vpt = few ? 1 : 4;
     if (K % 8 != 0 || nvec > 1024 * 4) {
         const int threads = K >= 8192 ? 1024 : (K >= 2048 ? 512 : 256);
-        quantize_rows_kernel<OUT><<<(unsigned)M, threads, 0, s>>>(xh, K, qmax, a, s_a);
+        if (K % 8 == 0) quantize_rows_kernel<OUT, true><<<(unsigned)M, threads, 0, s>>>(xh, K, qmax, a, s_a);
+        else quantize_rows_kernel<OUT, false><<<(unsigned)M, threads, 0, s>>>(xh, K, qmax, a, s_a);
         return launch_status();
     }
     cudaLaunchConfig_t cfg = {};
