@@ -123,9 +123,11 @@ tman_status tman_unpack_weights(const void *packed, size_t packed_bytes,
 /* Decode (paper Sec. 2.2 "Bit-serial table lookup", Fig. 2; Sec. 4.3): activation tables are
  * built in shared memory, packed bit-plane bytes index them, partial sums are
  * shift-accumulated per quantization block, scaled, and summed across blocks in fp32.
- * M in [1, 8], normally in one pass over the weights.  Five rows and more (three and more for 3- and 4-bit weights in groups of
- * 64 or 128) are multiplied on the tensor cores instead: codes and activations exact in fp16, sums in fp32.  Precision: one row --
- * fp32 table entries and sums; on the tensor cores as for one row.  Two to four rows by lookup -- each row of a K-slice is scaled by a power of two into [1, 2) (exactly
+ * M in [1, 8], normally in one pass over the weights.  Five rows and more are multiplied on the tensor cores instead, and three and
+ * four in groups of 64 or 128 except long calls of 2-bit weights in groups of 64 (K x N above 48 million): codes exact in fp16, activations
+ * in fp16 scaled by a power of two (exact down to 2^-21 of the largest of a row's 128 or 256 neighbours, else off by less than 2^-32 of
+ * it), sums in fp32.  Precision: one row -- fp32 table entries and sums; on the tensor cores as for one row.  Two to four rows by
+ * lookup -- each row of a K-slice is scaled by a power of two into [1, 2) (exactly
  * undone at the end), table entries are rounded to fp16 and the bits x 4 lookups of a 32-activation word
  * are added in fp16, everything after in fp32 (the paper's 16-bit table entries and low-precision
  * aggregation inside a block, Sec. 4.3, Sec. 5): error at most about 1.5e-3 of the largest output,

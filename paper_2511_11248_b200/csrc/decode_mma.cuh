@@ -12,8 +12,10 @@
 // Operands.  The plane words of a column are merged (two levels of rotate and bit-select) so that a mask yields two
 // codes in the low bits of the two halves of a register: as fp16 these are code x 2^(d - 24), d the field's bit position
 // (a half float below 2^-13 is its low eleven bits x 2^-24), exact matrix operands as they stand.  The 2^d is taken out
-// of the activations the other operand holds, which are scaled by a power of two per (row, chunk) so that their largest
-// magnitude lies in [2^14, 2^15); sums are fp32 throughout.  Zero-point and scale are applied to a block's sum:
+// of the activations the other operand holds, which are scaled by a power of two per row and chunk (CPW = 2: two chunks) so that
+// their largest magnitude lies in [2^14, 2^15); sums are fp32 throughout.  d is at most 7: an activation down to 2^-21 of that largest
+// one is exact, a smaller one is rounded to a multiple of 2^-24, an error below 2^-32 of the largest.  Zero-point and scale are applied to
+// a block's sum:
 // s * (sum - z * sum of the activations).
 #pragma once
 #include "sm100_ptx.cuh"

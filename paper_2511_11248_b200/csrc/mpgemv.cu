@@ -189,9 +189,9 @@ struct UnitRegs {
 // eight 16-bit values is below 2^24), a word's lookups and the pair sum stay exact in fp32, and from there
 // on the sums are 32-bit integers: the slice's lanes, the K-slices and the result are added as integers;
 // only the final product with the row's and the tensor's scale is floating point (Sec. 4.3).
-// ROLL: one set of unit registers; every strip's registers are refilled with the next unit's strip as
-// soon as its lookups are done (larger units, fewer per-unit fixed costs, same bytes in flight).
-template <int BITS, int MT, int S, int PRE, int HALF, int GROUPED, int ROLL, int HR, int INT>
+// One set of unit registers: every strip's registers are refilled with the next unit's strip as soon as its lookups are
+// done (larger units, fewer per-unit fixed costs, same bytes in flight).
+template <int BITS, int MT, int S, int PRE, int HALF, int GROUPED, int HR, int INT>
 __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParams p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
     // host, so these reads are in bounds whatever the header says, and no kernel that may still be
     // running writes the packed buffer (see the top of the file).  Their latency overlaps the table build.
     const int wu0 = j + p.P * warp, wstride = p.P * kGemvWarps;
-    UnitRegs<BITS, S> regs[ROLL ? 1 : 2];
-    load_unit(regs[0], wu0);
+    UnitRegs<BITS, S> regs;
+    load_unit(regs, wu0);
 
     // Everything below may depend on the previous kernel in the stream (activations, workspace).
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -319,7 +319,6 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
                 if (gv < nwords)
                     raw[ph] = __ldg(reinterpret_cast<const __half2 *>(p.x + (size_t)(word0 + gv) * 32 + 8 * ph + 2 * gc));
             }
-            if constexpr (!ROLL) load_unit(regs[1], wu0 + wstride);
 #pragma unroll
             for (int ph = 0; ph < 4; ++ph) {
                 const float2 f = __half22float2(raw[ph]);
@@ -355,7 +354,6 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
                 for (int c = 0; c < 4; ++c) xraw[r][c] = __ldg(px + c);
             }
         }
-        if constexpr (!ROLL) load_unit(regs[1], wu0 + wstride);
 
         // largest magnitude of each row over the K-slice -> power-of-two scale (every warp computes the same)
         float inv[2];
@@ -430,7 +428,6 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
 #pragma unroll
             for (int c = 0; c < 4; ++c) xraw[c] = __ldg(px + c);
         }
-        if constexpr (!ROLL) load_unit(regs[1], wu0 + wstride);
 
         // ---- phase A: activation tables (paper Sec. 2.2; one table per 8 activations, 256 entries,
         // entry = 16-entry table of the low four + sum of the selected high four) -----------------
@@ -525,8 +522,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
 #pragma unroll
         for (int s = 0; s < S; ++s) { sc_s[s] = r.sc[s]; z_s[s] = r.z[s]; }
         const int g_u = r.g, col_u = r.col;
-        UnitAddr nxt;
-        if constexpr (ROLL) nxt = unit_addr(r, next_wu);
+        const UnitAddr nxt = unit_addr(r, next_wu);
 #pragma unroll
         for (int s = 0; s < S; ++s) {
 #pragma unroll
@@ -574,7 +570,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
                     for (int m = 0; m < MT; ++m) vals[(s * 4 + c4) * MT + m] = a[m];
                 }
             }
-            if constexpr (ROLL) load_strip(r, s, nxt);
+            load_strip(r, s, nxt);
         }
 
         // lanes v and v^1 hold the two words of one block: add them first, keeping half the columns
@@ -648,17 +644,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
         }
     };
 
-    if constexpr (ROLL) {
-        for (int wu = wu0; wu < p.units; wu += wstride) compute_unit(regs[0], wu, wu + wstride);
-    } else {
-        for (int wu = wu0; wu < p.units; wu += 2 * wstride) {
-            compute_unit(regs[0], wu, 0);
-            load_unit(regs[0], wu + 2 * wstride);
-            if (wu + wstride >= p.units) break;        // uniform over the warp
-            compute_unit(regs[1], wu + wstride, 0);
-            load_unit(regs[1], wu + 3 * wstride);
-        }
-    }
+    for (int wu = wu0; wu < p.units; wu += wstride) compute_unit(regs, wu, wu + wstride);
 
     // ---- combine K-slices: every CTA polls the partial sums of its share of the columns ----------
     if (p.nkappa > 1) {
@@ -726,7 +712,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1) mpgemv_kernel(const GemvParam
     }
 }
 
-template <int BITS, int MT, int S, int PRE, int HALF, int GROUPED, int ROLL, int HR, int INT = 0>
+template <int BITS, int MT, int S, int PRE, int HALF, int GROUPED, int HR, int INT = 0>
 static tman_status launch_one(GemvParams p, int sms, cudaStream_t s)
 {
     constexpr int W = HALF ? 16 : 32 / MT;
@@ -753,7 +739,7 @@ static tman_status launch_one(GemvParams p, int sms, cudaStream_t s)
     const DeviceInfo *info = device_info(&dev);
     if (!info) return TMAN_ERR_CUDA;
     if ((uint32_t)info->reserved_smem.load(std::memory_order_relaxed) != kGemvSmemBase) return TMAN_ERR_UNSUPPORTED;
-    auto kern = mpgemv_kernel<BITS, MT, S, PRE, HALF, GROUPED, ROLL, HR, INT>;
+    auto kern = mpgemv_kernel<BITS, MT, S, PRE, HALF, GROUPED, HR, INT>;
     static std::atomic<bool> raised[kMaxDevices];
     // the grid has at most one CTA per SM; the occupancy query says whether an SM can hold one at all
     // (asked once per device and variant)
@@ -789,25 +775,26 @@ template <int BITS, int MT, int PRE, int HR>
 static tman_status launch_mt(GemvParams p, int sms, cudaStream_t s)
 {
     // one row: fp32 tables over half-warp slices, large units; more rows: fp16 row pairs, smaller units
-    // (measured: 2 strips per unit).  All on one rolling set of registers.
-    constexpr int ROLL = 1;
+    // (measured: 2 strips per unit)
     constexpr int S = (HR && MT == 2) ? 2 : ((BITS == 2) ? 4 : 2);
     constexpr int HALF = HR ? 0 : 1;
-    if (p.count > 1) return launch_one<BITS, MT, S, PRE, HALF, 1, ROLL, HR>(p, sms, s);
+    if (p.count > 1) return launch_one<BITS, MT, S, PRE, HALF, 1, HR>(p, sms, s);
     // One matrix of so few columns that a strip per sub-warp is enough: units of one strip, and fewer CTAs (launch_one).
     // In a graph, 4-bit 4096 x 1024: 3.86 -> 3.59 us (one row), 5.42 -> 5.23 (two), 2-bit 4096 x 512: 3.85 -> 3.12, 5.34 -> 4.16; near the
     // line (4096 x 2048) 4.19 -> 4.09 and 5.77 -> 5.74, above it the larger units are as fast or faster.
     constexpr int W = HALF ? 16 : 32 / MT;
     const int ctas = sms / ((p.K / 32 + W - 1) / W);
-    if (p.N / 4 <= ctas * kGemvWarps * (32 / W)) return launch_one<BITS, MT, 1, PRE, HALF, 0, ROLL, HR>(p, sms, s);
-    return launch_one<BITS, MT, S, PRE, HALF, 0, ROLL, HR>(p, sms, s);
+    if (p.N / 4 <= ctas * kGemvWarps * (32 / W)) return launch_one<BITS, MT, 1, PRE, HALF, 0, HR>(p, sms, s);
+    return launch_one<BITS, MT, S, PRE, HALF, 0, HR>(p, sms, s);
 }
 
 // ---- the plan: which kernel variants serve a call (host arithmetic only) -------------------------
 // A variant carries up to `rows` activation rows per pass over the weights in K-slices of `words` plane
 // words; its table entries have `slots` 32-bit slots (one fp32 row, or two fp16 rows each; 0: no tables, the tensor-core
 // kernel).  The time of a pass is modelled as fixed + per_mb x megabytes of bit planes; the constants were fitted to calls
-// timed in a CUDA graph on a B200 (4-bit, group 128, 4096 x 4096 and 4096 x 28672; one row also 2-bit 4096 x 14336).
+// timed in a CUDA graph on a B200 (4-bit, group 128, 4096 x 4096 and 4096 x 28672; one row also 2-bit 4096 x 14336; the last
+// two lines before the tensor-core kernel took two chunks of k per warp: 4096 x 28672 is modelled 20.5 and 23.1 us and takes 18.9
+// and 20.6.  They only weigh one pass of more rows against several of fewer, which this does not change).
 struct GemvVariant { int rows, words, slots, half_slices; double fixed_us, us_per_mb; };
 static const GemvVariant kGemvVariants[kGemvVariantCount] = {
     {1, 16, 1, 1, 4.10, 0.190},
@@ -822,7 +809,10 @@ static const GemvVariant kGemvVariants[kGemvVariantCount] = {
 // (two wavefronts) where the blocks are no shorter than two words: 4-bit, group 128
 // 23.8 / 18.9, 3-bit, group 64 20.2 / 18.9 (4096 x 4096: 7.4 / 5.6), 2-bit, group 128 17.3 / 16.9 (6.8 / 5.5); but 4-bit, group 32
 // 24.0 / 31.2.  2-bit, group 64 (few planes to look up, halves of a chunk to multiply) as far as a call is short: 4096 x 6144 8.4 / 7.0,
-// 14336 x 4096 11.3 / 11.5, 4096 x 28672 17.3 / 18.2.  One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.2 / 18.4).
+// 14336 x 4096 11.3 / 11.5, 4096 x 28672 17.3 / 18.2.  Where K fills the teams of warps badly the lookups would be faster here and
+// there (three rows, 18944 x 3584: 2-bit, group 128 12.0 / 13.3, 3-bit, group 64 14.1 / 15.0; 2-bit, group 64, 11008 x 4096 9.6 / 10.5); such
+// calls stay on the tensor cores, whose sums are fp32 throughout: the lookups' fp16 ones are three times further from the exact product.
+// One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.2 / 18.4).
 static bool uses_mma(int bits, int group, int rows, long long weights)
 {
     return rows >= 5 || (rows >= 3 && group >= 64 && (bits >= 3 || group == 128 || weights <= 48000000ll));
@@ -1071,7 +1061,7 @@ tman_status launch_mpgemv_grouped(int count, const void *const *packed, const vo
     p.M = 0; p.nkappa = 0; p.P = 0; p.units = 0;
     p.group_shift = (group == 32) ? 5 : (group == 64) ? 6 : 7;
     p.nblk = K / group;
-    // a table entry carries up to eight rows (four fp16 pairs): normally one pass over the weights
+    // a table entry carries up to four rows (two fp16 pairs), the tensor cores eight: normally one pass over the weights
     int m0 = 0;
     for (int ps = 0; ps < plan.npass; ++ps) {
         const int rows = plan.pass[ps].rows;
@@ -1317,9 +1307,9 @@ tman_status launch_mpgemv_ternary(const void *packed, const int16_t *a, const fl
         p.acc_out = acc_out ? acc_out + (size_t)m0 * N : nullptr;
         for (int g = 0; g < kGemvMaxGroup; ++g) p.y[g] = static_cast<__half *>(y) + (size_t)m0 * N;
         tman_status st;
-        if (mt == 1) st = pre ? launch_one<2, 1, 4, 1, 1, 0, 1, 0, 1>(p, sms, s) : launch_one<2, 1, 4, 0, 1, 0, 1, 0, 1>(p, sms, s);
-        else if (mt == 2) st = pre ? launch_one<2, 2, 2, 1, 0, 0, 1, 0, 1>(p, sms, s) : launch_one<2, 2, 2, 0, 0, 0, 1, 0, 1>(p, sms, s);
-        else st = pre ? launch_one<2, 4, 1, 1, 0, 0, 1, 0, 1>(p, sms, s) : launch_one<2, 4, 1, 0, 0, 0, 1, 0, 1>(p, sms, s);
+        if (mt == 1) st = pre ? launch_one<2, 1, 4, 1, 1, 0, 0, 1>(p, sms, s) : launch_one<2, 1, 4, 0, 1, 0, 0, 1>(p, sms, s);
+        else if (mt == 2) st = pre ? launch_one<2, 2, 2, 1, 0, 0, 0, 1>(p, sms, s) : launch_one<2, 2, 2, 0, 0, 0, 0, 1>(p, sms, s);
+        else st = pre ? launch_one<2, 4, 1, 1, 0, 0, 0, 1>(p, sms, s) : launch_one<2, 4, 1, 0, 0, 0, 0, 1>(p, sms, s);
         if (st != TMAN_OK) return st;
     }
     return TMAN_OK;
