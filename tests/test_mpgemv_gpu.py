@@ -155,10 +155,25 @@ def test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, Ns):
                                                        (8, 4, 32)]] + [(8, 3, 64, 16384, 4736)])
 def test_tensor_core_rows_with_two_chunks_a_warp(M, bits, G, K, N):
     # an odd number of chunks (the last warp at work has one), one K-slice and four; the bound of the test above, whose chunks here
-    # share a scale two by two (activations below 2^-29 of a pair's largest would lose bits: none)
+    # share a scale two by two (an activation below 2^-21 of a pair's largest is off by up to 2^-32 of that: below the fp32 sums' rounding)
     plan = B.tman_debug_gemv_plan(M, K, N, bits, G)
     assert plan["passes"][0]["words"] == 128, plan           # 16 warps x 2 chunks x 4 plane words
     test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, (N,))
+
+
+@pytest.mark.parametrize("M,bits,G,K", [(4, 4, 128, 4096), (8, 3, 64, 4096), (8, 2, 32, 1152), (3, 2, 128, 640)])
+def test_tensor_core_rows_with_a_large_spread_of_activations(M, bits, G, K):
+    # Activations from 2^-24 to 2^4 side by side (sums of larger ones would leave fp16's range): below 2^-21 of the largest neighbour
+    # they lose bits as operands, at most 2^-32 of it each, far below the bound of the tests above
+    c = synth.small_case(M, K, 40, bits, G, seed=700 + M + K)
+    rng = np.random.default_rng(M + K)
+    x = rng.standard_normal((M, K)) * 2.0 ** rng.integers(-24, 0, size=(M, K))
+    big = np.arange(0, K, 37)
+    x[:, big] = 2.0 ** 4 * rng.choice([-1.0, 1.0], size=(M, big.size))
+    c.x[:] = x.astype(np.float16)
+    got, *_ = run_gemv(c)
+    ref = orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)
+    assert rel_err(got, ref) <= 5.1e-4
 
 
 def test_repeat_calls_share_workspace_and_agree():
