@@ -126,7 +126,9 @@ tman_status tman_unpack_weights(const void *packed, size_t packed_bytes,
  * M in [1, 8], normally in one pass over the weights.  Five rows and more are multiplied on the tensor cores instead, and three and
  * four in groups of 64 or 128 except long calls of 2-bit weights in groups of 64 (K x N above 48 million): codes exact in fp16, activations
  * in fp16 scaled by a power of two (exact down to 2^-21 of the largest of a row's 128 or 256 neighbours, else off by less than 2^-32 of
- * it), sums in fp32.  Precision: one row -- fp32 table entries and sums; on the tensor cores as for one row.  Two to four rows by
+ * it), sums in fp32.  One and two rows of short reductions (K <= 5120; by columns, bits and group) are multiplied on the integer tensor
+ * cores: activations as 32-bit integers (rounded by at most 2^-24 of the largest of 128 neighbours), a block's sum exact, the rest fp32.
+ * Precision: one row, and everything on tensor cores -- fp32 table entries or better, fp32 sums.  Two to four rows by
  * lookup -- each row of a K-slice is scaled by a power of two into [1, 2) (exactly
  * undone at the end), table entries are rounded to fp16 and the bits x 4 lookups of a 32-activation word
  * are added in fp16, everything after in fp32 (the paper's 16-bit table entries and low-precision
@@ -164,7 +166,7 @@ tman_status tman_quantize_rows(const void *x_f16, int M, int K, int qmax, int16_
                                tman_stream_t stream);
 
 /* Decode of M rows (1 <= M <= 8, in passes of up to four rows; K <= 16384): the bit-serial table lookup of
- * tman_mpgemv on integers.  Tables hold exact integer sums of activations, lookups are shift-accumulated,
+ * tman_mpgemv on integers (two rows and more with K <= 5120: the integer tensor cores).  Tables hold exact integer sums of activations, lookups are shift-accumulated,
  * the activation sum is subtracted once (zero-point 1), K-slices are added as 32-bit integers;
  *   y[m][n] = fp16( row_scale[m] * w_scale * sum_k a[m][k] * (q[k][n] - 1) ).
  * acc_i32 (device, int32 [M][N], 16-byte aligned, may be NULL) receives the exact integer sums.

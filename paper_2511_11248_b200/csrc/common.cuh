@@ -94,6 +94,16 @@ inline int sm_count()
     return d ? d->sms.load(std::memory_order_acquire) : 0;
 }
 
+// Asks for the decode kernels' common split of an SM's 256 KB between shared memory (132 KB) and L1: an SM changes its split only when it
+// is idle, so that kernels of different splits do not follow one another without a gap (a layer of alternating kernels 76 -> 86 us).
+// 132 KB hold two CTAs of decode_digits_kernel and leave the lookups the L1 that their loads in flight pass through (with 228 KB of shared
+// memory 14336 x 4096, 4-bit, takes 12.3 us instead of 9.8).  A hint: failure changes nothing.
+constexpr int kSharedPercent = 58;        // of 228 KB
+template <typename Kernel> inline void prefer_common_split(Kernel kern)
+{
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, kSharedPercent) != cudaSuccess) (void)cudaGetLastError();
+}
+
 // Launches `launch()` (cudaSuccess or an error) of a kernel that needs `bytes` of dynamic shared memory.  The kernel's
 // limit is raised once per device, `raised[device]` remembers it; a launch that fails all the same (the context may have
 // been reset in between) raises the limit again and tries once more.
@@ -148,7 +158,7 @@ constexpr int kGemvMaxRows = 8;
 constexpr int kGemvVariantCount = 4;
 constexpr int kGemvSmemLimit = 227 * 1024;
 constexpr int kGemvPlanSms = 148;
-struct GemvPass { int variant, rows, variant_rows, words, nkappa, ctas_per_slice, smem_bytes; bool mma; };
+struct GemvPass { int variant, rows, variant_rows, words, nkappa, ctas_per_slice, smem_bytes; bool mma, digits; };
 struct GemvPlan { int npass; GemvPass pass[kGemvMaxRows]; size_t ws_bytes; double cost_us; };
 tman_status launch_quantize_rows(const void *x, int M, int K, int qmax, int16_t *a, float *s_a, cudaStream_t s);
 tman_status launch_mpgemv_ternary(const void *packed, const int16_t *a, const float *s_a, float s_w, void *y,

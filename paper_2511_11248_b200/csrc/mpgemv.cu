@@ -1,8 +1,8 @@
 // Decode path: bit-serial table-lookup mpGEMV (paper Sec. 2.2 "Bit-serial table lookup", Fig. 2;
 // Sec. 4.3 "Mapping of LUT-based Decoding").
 //
-// One and two activation rows (and three and four where that is faster, uses_mma below) by table lookup, described here; more rows on
-// the tensor cores (decode_mma.cuh).
+// One and two activation rows (and three and four where that is faster, uses_mma below) by table lookup, described here, short reductions
+// of them on the integer tensor cores (decode_digits.cuh, uses_digits below); more rows on the tensor cores (decode_mma.cuh).
 //
 // Work split.  The reduction dimension is cut into K-slices of 16 or 32 plane words (16 for one
 // activation row; 32, 16 for 2, 3-4 rows, whose table entries carry the rows as fp16 pairs).  One
@@ -35,6 +35,7 @@
 // in plain stream order instead (packed_write_pending below), and the header states the rule for
 // kernels of the caller's own.
 #include "decode_mma.cuh"
+#include "decode_digits.cuh"
 
 namespace tman {
 
@@ -751,6 +752,7 @@ static tman_status launch_one(GemvParams p, int sms, cudaStream_t s)
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGemvThreads, kSmem) != cudaSuccess)
                 return TMAN_ERR_CUDA;
+            prefer_common_split(kern);
             f = per_sm >= 1 ? 1 : -1;
             fits[dev].store(f, std::memory_order_relaxed);
         }
@@ -863,6 +865,73 @@ static MmaSplit split_mma(int M, int K, int N, int groups, int sms, size_t ws_li
     return best;
 }
 
+// ---- decode on the integer tensor cores (decode_digits.cuh) ----------------------------------------------------------
+// How a launch is laid out: CTAs, warps of a team, units of the warps' rings, turns between reductions (0: it does not fit).
+struct DigitSplit { int ctas, tk_shift, depth, flush, smem, scale_row, zero_row; };
+static DigitSplit split_digits(int rows, int K, int strips, int bits, int group, int nb, bool ints, int sms)
+{
+    DigitSplit d = {};
+    const int pairs = (K / 128 + 1) / 2, nblk = K / group;
+    const int slot = rows * (512 + nb * 16), turn = kDigitWarps * rows * 128;    // a chunk's activations; the warps' sums of a turn
+    const int fixed = kDigitGroups * (int)sizeof(DigitGroup) + (nb > 1 ? rows * 512 : 0), ring = kDigitWarps * 2 * bits * 512;
+    d.scale_row = ints ? 0 : (nblk * 8 + 127) / 128 * 128 + (nb == 4 ? 32 : 16);
+    d.zero_row = ints ? 0 : (nblk * 2 + 4 + 127) / 128 * 128 + 4;
+    // One CTA an SM, in half its shared memory so that the next call's can start beside it, or two of this call where there are five
+    // groups each (4-bit 4096 x 28672: 14.8 us with one, 13.5 with two); else one with all of it.
+    const bool two = strips >= 40 * sms;
+    const int at_most = two ? 2 * sms : sms;
+    d.ctas = strips < at_most ? strips : at_most;
+    const int share = (strips + d.ctas - 1) / d.ctas, groups = (share + 7) / 8;
+    const int rest = fixed + 2 * pairs * slot + share * (d.scale_row + d.zero_row) + 16;
+    int room = kDigitSmemHalf;
+    d.depth = rest + 2 * ring + turn <= room ? 2 : 1;
+    if (rest + ring + turn > room) {
+        room = kDigitSmem;
+        d.depth = rest + 2 * ring + turn <= room ? 2 : 1;
+    }
+    const int base = rest + d.depth * ring;
+    if (groups > kDigitGroups - kGemvMaxGroup || base + turn > room || (two && room > kDigitSmemHalf)) return d;
+    d.tk_shift = kDigitWarpsShift;
+    int best = 1 << 30;
+    for (int shift = kDigitWarpsShift; shift >= 0; --shift) {
+        const int tc = kDigitWarps >> shift, steps = (groups + tc - 1) / tc * ((pairs + (1 << shift) - 1) >> shift);
+        if (steps < best) { best = steps; d.tk_shift = shift; }
+    }
+    const int tc = kDigitWarps >> d.tk_shift, turns = (groups + kGemvMaxGroup + tc - 1) / tc;
+    d.flush = (room - base) / turn;
+    if (d.flush > turns) d.flush = turns;
+    d.smem = base + d.flush * turn;
+    return d;
+}
+
+// Whether a pass of `rows` rows goes to the integer tensor cores instead of the table lookups (columns: of all matrices).  In a graph,
+// lookup / here, us: one row, 2-bit group 64 2048 x 8192 4.35 / 3.24, 4096 x 4096 4.30 / 3.34, 4096 x 28672 11.7 / 10.3; 4-bit group 128 4096 x
+// 4096 5.13 / 4.25, 4096 x 28672 15.9 / 13.5; two rows 6.63 / 5.36 (4096 x 4096), 6.55 / 4.28 (2048 x 8192).  The lines:
+// K: every CTA prepares all activations (8192 x 2048 5.14 / 5.66, 14336 x 4096 9.9 / 11.0).  Few columns: the same work for little
+// (4096 x 512 3.25 / 4.82; 4096 x 1024, one row 3.51 / 3.63).  20480 columns are too many for one CTA an SM and fill two badly (4096 x
+// 20480 12.2 / 14.1, 2-bit 8.9 / 9.0; 2048 x 20480 8.0 / 7.6).  Where rows and blocks need more columns of B than the MMA has (more tiles), the
+// work grows with the columns: two rows of group 64 4096 x 4096 6.34 / 5.60, 4096 x 6144 7.68 / 8.16, 2048 x 8192 6.33 / 4.38; group 32 2048
+// x 8192 4.63 / 3.97 and 6.29 / 5.22, 4096 x 6144 5.47 / 6.12.  3 and 4 bits of group 64, one row: 4096 x 4096 4.61 / 4.03, x 20480 10.4 / 11.7.
+static bool uses_digits(int bits, int group, int rows, int K, long long columns, int sms)
+{
+    if (rows > 2 || K > 5120 || columns * rows < K / 2) return false;
+    const int blocks = 128 / group;
+    const bool one_tile = group == 128 || (group == 64 && rows == 1);
+    long long most = one_tile && (group == 128 || bits == 2) ? 10ll * K : 8192;
+    if (K > 2048 && group == 64 && (rows == 2 || bits == 3)) most = 5120;
+    if (columns > most || (group == 32 && K > 2048)) return false;
+    if (K > 2048 && columns >= 96ll * sms && columns < 160ll * sms) return false;
+    return split_digits(rows, K, (int)(columns / 4), bits, group, blocks, false, sms).flush > 0;
+}
+
+// The same for the integer path, whose product follows a row quantization: products 2560 x 6912 and back in turn, each with its
+// quantization, two rows 13.8 / 13.6 us, six 28.9 / 23.1, eight (which the lookups take in two passes) 32.0 / 27.0; 4096 x 4096 two rows
+// 13.3 / 12.7, three 16.1 / 13.7.  One row stays with the lookups (ternary_decode of one row 47.1 / 48.4).
+static bool uses_digits_ternary(int rows, int K, int N, int group, int sms)
+{
+    return rows >= 2 && K <= 5120 && (long long)N * rows >= K / 2 && split_digits(rows, K, N / 4, 2, group, 1, true, sms).flush > 0;
+}
+
 GemvPlan plan_gemv(int M, int K, int N, int bits, int group, int sms, size_t ws_limit)
 {
     // best[m]: least modelled time for m rows; a pass with variant v takes min(rows_v, m) of them
@@ -904,7 +973,15 @@ GemvPlan plan_gemv(int M, int K, int N, int bits, int group, int sms, size_t ws_
         ps.ctas_per_slice = sms / ps.nkappa;
         ps.smem_bytes = v.half_slices ? kGemvTableBytes / 2 : kGemvTableBytes + 64;
         const size_t need = variant_ws_bytes(v, K, N);
-        ps.mma = uses_mma(bits, group, take, (long long)K * N);
+        ps.digits = uses_digits(bits, group, take, K, N, sms);
+        ps.mma = !ps.digits && uses_mma(bits, group, take, (long long)K * N);
+        if (ps.digits) {
+            const DigitSplit sp = split_digits(take, K, N / 4, bits, group, 128 / group, false, sms);
+            ps.words = K / 32;
+            ps.nkappa = 1;
+            ps.ctas_per_slice = sp.ctas;
+            ps.smem_bytes = sp.smem;
+        }
         if (ps.mma) {
             const MmaSplit sp = split_mma(take, K, N, (N + 31) / 32, sms, need);
             ps.words = 4 * sp.tk * sp.cpw;
@@ -938,6 +1015,7 @@ static tman_status launch_mma_split(MmaParams p, const MmaSplit &sp, cudaStream_
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = packed_write_pending(s, /*clear=*/true) ? 0 : 1;      // as in launch_one
+    if (!raised[dev].load(std::memory_order_relaxed)) prefer_common_split(kern);
     return launch_with_smem(kern, smem, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, p); });
 }
 
@@ -975,10 +1053,75 @@ static tman_status launch_mma_rows(const GemvParams &g, int rows, int sms, size_
     return p.group == 64 ? launch_mma<BITS, 2, 1, 2>(p, sms, ws, s) : launch_mma<BITS, 4, 1, 2>(p, sms, ws, s);
 }
 
+template <int BITS, int NB, int NT, int DEPTH, bool INT>
+static tman_status launch_digits_split(DigitParams p, const DigitSplit &d, cudaStream_t s)
+{
+    p.chunks = p.K / 128;
+    p.strips_q = p.strip0[kGemvMaxGroup] / d.ctas; p.strips_r = p.strip0[kGemvMaxGroup] % d.ctas;
+    p.pairs = (p.chunks + 1) / 2;
+    p.pairs_q = p.pairs >> d.tk_shift; p.pairs_r = p.pairs & ((1 << d.tk_shift) - 1);
+    p.scale_row = d.scale_row; p.zero_row = d.zero_row;
+    p.tk_shift = d.tk_shift; p.tc = kDigitWarps >> d.tk_shift; p.flush = d.flush;
+    p.by_rows = (0x80000000u + (uint32_t)p.M - 1u) / (uint32_t)p.M;
+    auto kern = decode_digits_kernel<BITS, NB, NT, DEPTH, INT>;
+    static std::atomic<bool> raised[kMaxDevices];
+    int dev = 0;
+    if (!device_info(&dev)) return TMAN_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)d.ctas);
+    cfg.blockDim = dim3(32 * kDigitWarps);
+    cfg.dynamicSmemBytes = (size_t)d.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = packed_write_pending(s, /*clear=*/true) ? 0 : 1;      // as in launch_one
+    if (!raised[dev].load(std::memory_order_relaxed)) prefer_common_split(kern);
+    return launch_with_smem(kern, kDigitSmem, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, p); });
+}
+
+template <int BITS, int NB, int NT, bool INT>
+static tman_status launch_digits(const DigitParams &p, int sms, cudaStream_t s)
+{
+    const DigitSplit d = split_digits(p.M, p.K, p.strip0[kGemvMaxGroup], BITS, p.group, NB, INT, sms);
+    if (d.flush < 1) return TMAN_ERR_UNSUPPORTED;
+    return d.depth == 2 ? launch_digits_split<BITS, NB, NT, 2, INT>(p, d, s) : launch_digits_split<BITS, NB, NT, 1, INT>(p, d, s);
+}
+
+template <int BITS>
+static tman_status launch_digit_tiles(const DigitParams &p, int sms, cudaStream_t s)
+{
+    if (p.group == 128) return launch_digits<BITS, 1, 1, false>(p, sms, s);
+    if (p.group == 64) return p.M == 1 ? launch_digits<BITS, 2, 1, false>(p, sms, s) : launch_digits<BITS, 2, 2, false>(p, sms, s);
+    return p.M == 1 ? launch_digits<BITS, 4, 2, false>(p, sms, s) : launch_digits<BITS, 4, 4, false>(p, sms, s);
+}
+
+template <int BITS>
+static tman_status launch_digit_rows(const GemvParams &g, int sms, cudaStream_t s)
+{
+    DigitParams p = {};
+    p.count = g.count;
+    for (int i = 0; i < kGemvMaxGroup; ++i) {
+        p.packed[i] = g.packed[i];
+        p.planes[i] = reinterpret_cast<const uint8_t *>(g.planes[i]);
+        p.scales[i] = reinterpret_cast<const uint8_t *>(g.scales[i]);
+        p.zeros[i] = reinterpret_cast<const uint8_t *>(g.zeros[i]);
+        p.y[i] = g.y[i];
+        p.Ng[i] = g.Ng[i];
+        p.strip0[i + 1] = p.strip0[i] + (i < g.count ? g.Ng[i] / 4 : 0);
+    }
+    p.x = g.x;
+    p.status = g.status;
+    p.M = g.M; p.K = g.K; p.bits = g.bits; p.group = g.group; p.nblk = g.nblk;
+    return launch_digit_tiles<BITS>(p, sms, s);
+}
+
 template <int BITS>
 static tman_status launch_rows(GemvParams p, const GemvPass &ps, int sms, cudaStream_t s)
 {
     p.M = ps.rows;
+    if (ps.digits) return launch_digit_rows<BITS>(p, sms, s);
     const bool pre = p.group >= 64;
     if (ps.mma) return launch_mma_rows<BITS>(p, ps.rows, sms, variant_ws_bytes(kGemvVariants[ps.variant], p.K, p.N), s);
     if (ps.variant == 0) return pre ? launch_mt<BITS, 1, 1, 0>(p, sms, s) : launch_mt<BITS, 1, 0, 0>(p, sms, s);
@@ -1237,6 +1380,15 @@ static tman_status launch_quantize(const void *x, int M, int K, int qmax, OUT *a
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     auto kern = few ? quantize_rows_regs_kernel<OUT, 1> : quantize_rows_regs_kernel<OUT, 4>;
+    if constexpr (sizeof(OUT) == 2) {                                            // (a decode follows)
+        static std::atomic<bool> preferred[2][kMaxDevices];
+        int dev = 0;
+        if (!device_info(&dev)) return TMAN_ERR_CUDA;
+        if (!preferred[few][dev].load(std::memory_order_relaxed)) {
+            prefer_common_split(kern);
+            preferred[few][dev].store(true, std::memory_order_relaxed);
+        }
+    }
     return cudaLaunchKernelEx(&cfg, kern, xh, nvec, qmax, a, s_a) == cudaSuccess ? TMAN_OK : TMAN_ERR_CUDA;
 }
 
@@ -1296,6 +1448,22 @@ tman_status launch_mpgemv_ternary(const void *packed, const int16_t *a, const fl
     p.group_shift = (group == 32) ? 5 : (group == 64) ? 6 : 7;
     p.nblk = K / group;
     const bool pre = group >= 64;
+    if (uses_digits_ternary(M, K, N, group, sms)) {
+        DigitParams d = {};
+        d.count = 1;
+        for (int i = 0; i < kGemvMaxGroup; ++i) {
+            d.packed[i] = p.packed[0];
+            d.planes[i] = reinterpret_cast<const uint8_t *>(p.planes[0]);
+            d.y[i] = static_cast<__half *>(y);
+            d.Ng[i] = N;
+            d.strip0[i + 1] = N / 4;
+        }
+        d.x = a; d.row_scale = s_a; d.w_scale = s_w; d.acc_out = acc_out;
+        d.status = p.status;
+        d.M = M; d.K = K; d.bits = 2; d.group = group; d.nblk = p.nblk;
+        return M <= 2 ? launch_digits<2, 1, 1, true>(d, sms, s) : M <= 4 ? launch_digits<2, 1, 2, true>(d, sms, s)
+             : M <= 6 ? launch_digits<2, 1, 3, true>(d, sms, s) : launch_digits<2, 1, 4, true>(d, sms, s);
+    }
     for (int m0 = 0; m0 < M; m0 += 4) {
         const int rows = (M - m0 < 4) ? (M - m0) : 4;
         int mt = 1, words = 16;

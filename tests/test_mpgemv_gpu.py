@@ -131,6 +131,10 @@ def test_lookup_units_of_one_strip_and_the_line_above_them(M, bits, G, K, N):
 @pytest.mark.parametrize("M,bits,G", [(3, 3, 64), (3, 2, 128), (4, 2, 64), (4, 4, 128), (5, 2, 32), (5, 3, 64), (6, 2, 64), (7, 4, 32), (8, 2, 128), (8, 3, 128), (8, 4, 64)])
 @pytest.mark.parametrize("K,Ns", [(128, (8,)), (640, (32, 40)), (2176, (264,)), (4096, (2056, 8, 40))])
 def test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, Ns):
+    check_grouped_twice(M, bits, G, K, Ns, 5.1e-4)
+
+
+def check_grouped_twice(M, bits, G, K, Ns, bound):
     # one chunk of 128 k; a team with idle warps; a second K-slice of a single chunk; ragged groups of 32 columns and a
     # matrix narrower than one.  Codes and activations are exact operands and sums fp32, so what is left is the rounding of
     # the result to fp16, 2^-11 = 4.9e-4 of it, and fp32 sums of up to 4096 terms, below 1e-5.
@@ -147,7 +151,7 @@ def test_tensor_core_rows_at_the_edges_of_their_split(M, bits, G, K, Ns):
         H.check_guards()
         for c, y in zip(cases, ys):
             ref = orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)
-            assert rel_err(H.to_f64(y), ref) <= 5.1e-4
+            assert rel_err(H.to_f64(y), ref) <= bound
 
 
 @pytest.mark.parametrize("M,bits,G,K,N", [(M, b, G, K, 4104) for K in (2176, 4096) for M, b, G in
@@ -163,9 +167,13 @@ def test_tensor_core_rows_with_two_chunks_a_warp(M, bits, G, K, N):
 
 @pytest.mark.parametrize("M,bits,G,K", [(4, 4, 128, 4096), (8, 3, 64, 4096), (8, 2, 32, 1152), (3, 2, 128, 640)])
 def test_tensor_core_rows_with_a_large_spread_of_activations(M, bits, G, K):
+    check_large_spread(M, bits, G, K, 40)
+
+
+def check_large_spread(M, bits, G, K, N):
     # Activations from 2^-24 to 2^4 side by side (sums of larger ones would leave fp16's range): below 2^-21 of the largest neighbour
     # they lose bits as operands, at most 2^-32 of it each, far below the bound of the tests above
-    c = synth.small_case(M, K, 40, bits, G, seed=700 + M + K)
+    c = synth.small_case(M, K, N, bits, G, seed=700 + M + K)
     rng = np.random.default_rng(M + K)
     x = rng.standard_normal((M, K)) * 2.0 ** rng.integers(-24, 0, size=(M, K))
     big = np.arange(0, K, 37)
@@ -174,6 +182,45 @@ def test_tensor_core_rows_with_a_large_spread_of_activations(M, bits, G, K):
     got, *_ = run_gemv(c)
     ref = orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)
     assert rel_err(got, ref) <= 5.1e-4
+
+
+# (M, K, Ns): one chunk of 128 k and an odd number of them, teams of one to eight warps, ragged groups of eight strips, matrices narrower
+# than one, the longest K, the columns at which the rule changes sides
+DIGIT_CASES = [(1, 128, (64,)), (2, 128, (72,)), (1, 640, (328, 40)), (2, 640, (320,)), (1, 1536, (8, 760, 16)), (2, 2048, (1032,)),
+               (1, 2176, (1096, 8, 40)), (2, 2176, (1088,)), (1, 4096, (2048,)), (1, 4096, (2040,)), (2, 4096, (4096, 1024, 1024)),
+               (1, 5120, (2560, 24)), (2, 5120, (1288,)), (1, 4096, (16392,))]
+
+
+@pytest.mark.parametrize("bits,G", [(2, 32), (2, 64), (2, 128), (3, 32), (3, 64), (3, 128), (4, 32), (4, 64), (4, 128)])
+@pytest.mark.parametrize("M,K,Ns", DIGIT_CASES)
+def test_one_and_two_rows_on_the_integer_tensor_cores(M, K, Ns, bits, G):
+    # Sums are exact up to a block; an activation is rounded by at most 2^-24 of its largest neighbour, so what is left is the rounding of
+    # the result to fp16 and fp32 sums: the bound of test_tensor_core_rows_at_the_edges_of_their_split (calls beyond the rule's limits go to
+    # the lookups, whose fp16 tables for two rows have the bound of test_rows_in_fp16_tables_stay_near_the_predicted_error).
+    plan = B.tman_debug_gemv_plan(M, K, sum(Ns), bits, G)
+    lookup = plan["passes"][0]["words"] != K // 32
+    check_grouped_twice(M, bits, G, K, Ns, 2e-3 if lookup and M > 1 else 5.1e-4)
+
+
+@pytest.mark.parametrize("M,bits,G", [(1, 2, 64), (1, 4, 128), (2, 3, 128), (2, 2, 64), (1, 3, 32), (2, 4, 32)])
+def test_digits_with_a_large_spread_of_activations(M, bits, G):
+    # as above, 2^-24 to 2^4 side by side
+    check_large_spread(M, bits, G, 2048, 1096)
+
+
+@pytest.mark.parametrize("bits,G", [(2, 128), (4, 64), (3, 32)])
+def test_digits_with_an_infinity_and_a_nan(bits, G):
+    # the definition column by column: s (q - z) inf is an infinity of the sign of q - z, NaN where q = z; a NaN reaches every column
+    c = synth.small_case(2, 2048, 1096, bits, G, seed=5)
+    c.x[0, 700] = -np.inf
+    c.x[1, 3] = np.nan
+    dev = H.device_case(c)
+    ws, y = H.alloc_workspace(B.OP_GEMV, 2, c.K, c.N, bits, G), H.alloc_y(2, c.N)
+    B.tman_mpgemv(H.pack_case(c, dev), dev["x"], y, 2, c.K, c.N, bits, G, ws)
+    got = H.to_f64(y)
+    d = c.codes[700].astype(np.int64) - c.zeros[700 // G].astype(np.int64)
+    assert np.all(np.isnan(got[1])) and np.all(np.isnan(got[0, d == 0]))
+    assert np.all(np.isinf(got[0, d != 0])) and np.array_equal(got[0, d != 0] > 0, d[d != 0] < 0)
 
 
 def test_repeat_calls_share_workspace_and_agree():
