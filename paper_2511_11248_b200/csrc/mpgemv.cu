@@ -752,7 +752,8 @@ static tman_status launch_one(GemvParams p, int sms, cudaStream_t s)
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGemvThreads, kSmem) != cudaSuccess)
                 return TMAN_ERR_CUDA;
-            prefer_common_split(kern);
+            // they alternate with decode_digits_kernel in a layer (two rows of group 32 do not, and lose 4 % by it)
+            if constexpr (INT || (MT == 1 && (PRE || !HR))) prefer_common_split(kern);
             f = per_sm >= 1 ? 1 : -1;
             fits[dev].store(f, std::memory_order_relaxed);
         }
@@ -910,8 +911,8 @@ static DigitSplit split_digits(int rows, int K, int strips, int bits, int group,
 // K: every CTA prepares all activations (8192 x 2048 5.14 / 5.66, 14336 x 4096 9.9 / 11.0).  Few columns: the same work for little
 // (4096 x 512 3.25 / 4.82; 4096 x 1024, one row 3.51 / 3.63).  20480 columns are too many for one CTA an SM and fill two badly (4096 x
 // 20480 12.2 / 14.1, 2-bit 8.9 / 9.0; 2048 x 20480 8.0 / 7.6).  Where rows and blocks need more columns of B than the MMA has (more tiles), the
-// work grows with the columns: two rows of group 64 4096 x 4096 6.34 / 5.60, 4096 x 6144 7.68 / 8.16, 2048 x 8192 6.33 / 4.38; group 32 2048
-// x 8192 4.63 / 3.97 and 6.29 / 5.22, 4096 x 6144 5.47 / 6.12.  3 and 4 bits of group 64, one row: 4096 x 4096 4.61 / 4.03, x 20480 10.4 / 11.7.
+// work grows with the columns: two rows of group 64 4096 x 4096 6.34 / 5.60, 4096 x 6144 7.68 / 8.16, 2048 x 8192 6.33 / 4.38; group 32,
+// one row 2048 x 8192 4.63 / 3.97, 4096 x 6144 5.47 / 6.12 (two rows stay with the lookups).  3 and 4 bits of group 64, one row: 4096 x 4096 4.61 / 4.03, x 20480 10.4 / 11.7.
 static bool uses_digits(int bits, int group, int rows, int K, long long columns, int sms)
 {
     if (rows > 2 || K > 5120 || columns * rows < K / 2) return false;
@@ -919,7 +920,7 @@ static bool uses_digits(int bits, int group, int rows, int K, long long columns,
     const bool one_tile = group == 128 || (group == 64 && rows == 1);
     long long most = one_tile && (group == 128 || bits == 2) ? 10ll * K : 8192;
     if (K > 2048 && group == 64 && (rows == 2 || bits == 3)) most = 5120;
-    if (columns > most || (group == 32 && K > 2048)) return false;
+    if (columns > most || (group == 32 && (rows == 2 || K > 2048))) return false;
     if (K > 2048 && columns >= 96ll * sms && columns < 160ll * sms) return false;
     return split_digits(rows, K, (int)(columns / 4), bits, group, blocks, false, sms).flush > 0;
 }
@@ -1015,7 +1016,6 @@ static tman_status launch_mma_split(MmaParams p, const MmaSplit &sp, cudaStream_
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = packed_write_pending(s, /*clear=*/true) ? 0 : 1;      // as in launch_one
-    if (!raised[dev].load(std::memory_order_relaxed)) prefer_common_split(kern);
     return launch_with_smem(kern, smem, dev, raised, [&] { return cudaLaunchKernelEx(&cfg, kern, p); });
 }
 
@@ -1094,7 +1094,7 @@ static tman_status launch_digit_tiles(const DigitParams &p, int sms, cudaStream_
 {
     if (p.group == 128) return launch_digits<BITS, 1, 1, false>(p, sms, s);
     if (p.group == 64) return p.M == 1 ? launch_digits<BITS, 2, 1, false>(p, sms, s) : launch_digits<BITS, 2, 2, false>(p, sms, s);
-    return p.M == 1 ? launch_digits<BITS, 4, 2, false>(p, sms, s) : launch_digits<BITS, 4, 4, false>(p, sms, s);
+    return launch_digits<BITS, 4, 2, false>(p, sms, s);
 }
 
 template <int BITS>
