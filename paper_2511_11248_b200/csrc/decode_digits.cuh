@@ -317,14 +317,22 @@ __global__ void __launch_bounds__(32 * kDigitWarps, 2) decode_digits_kernel(cons
             back_lo = (83u + e) << 23;
             float fac = __uint_as_float((171u - e) << 23);                       // 2^(29 - exponent)
             if (__any_sync(0xffffffffu, e == 31u)) {
-                // Infinities and NaN: a block that holds one counts its infinities (finite values are nothing beside them) and is
-                // multiplied back by infinity, or NaN; the other blocks of the chunk are as if zero.
+                // Infinities and NaN.  A block of one infinity takes it alone (finite values are nothing beside it) and is multiplied
+                // back by infinity: an infinity, or NaN where its code is the zero-point.  More of them may cancel column by column,
+                // which their sum does not show, so that such a block is NaN, as one with a NaN in it; the other blocks of the
+                // chunk are as if zero.
                 uint32_t blk = mine;
+                int infs = 0;
 #pragma unroll
-                for (int mask = 1; mask < 16 / NB; mask <<= 1) blk = max(blk, __shfl_xor_sync(0xffffffffu, blk, mask));
+                for (int i = 0; i < 8; ++i) infs += isinf(f[i]) ? 1 : 0;
+#pragma unroll
+                for (int mask = 1; mask < 16 / NB; mask <<= 1) {
+                    blk = max(blk, __shfl_xor_sync(0xffffffffu, blk, mask));
+                    infs += __shfl_xor_sync(0xffffffffu, infs, mask);
+                }
                 if (e == 31u) {
                     fac = 1.f;
-                    back_hi = blk > 0x7C00u ? 0x7FC00000u : blk == 0x7C00u ? 0x7F800000u : 0u;
+                    back_hi = blk > 0x7C00u || infs > 1 ? 0x7FC00000u : blk == 0x7C00u ? 0x7F800000u : 0u;
                     back_lo = 0u;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) f[i] = isinf(f[i]) ? copysignf(268435456.f, f[i]) : 0.f;

@@ -223,6 +223,27 @@ def test_digits_with_an_infinity_and_a_nan(bits, G):
     assert np.all(np.isinf(got[0, d != 0])) and np.array_equal(got[0, d != 0] > 0, d[d != 0] < 0)
 
 
+@pytest.mark.parametrize("M,bits,G", [(1, 2, 128), (2, 3, 128), (2, 4, 64), (1, 3, 32)])
+@pytest.mark.parametrize("other", [701, 702, 736, 800, 1500])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_digits_with_two_infinities(M, bits, G, other, sign):
+    # two infinities, of one block (the first two, and up to G = 128 the others) or of two: wherever the definition has infinities of both
+    # signs, or an infinity that meets its zero-point, the sum is NaN; nothing finite comes out where it has an infinity
+    c = synth.small_case(M, 2048, 1096, bits, G, seed=6)
+    c.x[M - 1, 700], c.x[M - 1, other] = np.inf, sign * np.inf
+    dev = H.device_case(c)
+    ws, y = H.alloc_workspace(B.OP_GEMV, M, c.K, c.N, bits, G), H.alloc_y(M, c.N)
+    B.tman_mpgemv(H.pack_case(c, dev), dev["x"], y, M, c.K, c.N, bits, G, ws)
+    got = H.to_f64(y)[M - 1]
+    d0 = c.codes[700].astype(np.int64) - c.zeros[700 // G].astype(np.int64)
+    d1 = (c.codes[other].astype(np.int64) - c.zeros[other // G].astype(np.int64)) * int(sign)
+    nan = d0 * d1 <= 0
+    assert nan.any() and not nan.all()
+    assert np.all(np.isnan(got[nan])) and not np.any(np.isfinite(got))
+    if other // G != 700 // G:
+        assert np.array_equal(got[~nan], np.where(d0[~nan] > 0, np.inf, -np.inf))
+
+
 def test_repeat_calls_share_workspace_and_agree():
     c = synth.small_case(2, 2048, 264, 4, 64, seed=21)
     dev = H.device_case(c)
