@@ -121,6 +121,25 @@ inline tman_status launch_with_smem(Kernel kern, int bytes, int dev, std::atomic
     return TMAN_OK;
 }
 
+// ---- loads behind a wait (device) ----------------------------------------------------------
+// What the kernels before this one in the stream wrote (activations, row scales), read after griddepcontrol.wait by a kernel that may
+// have started while they ran: ordinary loads that stay behind the wait.  The read-only path (__ldg) is for data that nobody writes while
+// the kernel is resident: a load by it may be moved above the wait, and it takes a line that an earlier call left in the SM's L1,
+// which the launch of a kernel that starts early does not empty (calls that passed one buffer on to the next read what it held two calls
+// before).
+__device__ __forceinline__ uint4 ld_dependent(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_dependent(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // ---- table building block (device) -------------------------------------------------------
 // The 16 partial sums of four activations: out[p] = sum_{j<4} x_j * bit_j(p), accumulated in
 // increasing j (paper Sec. 2.2: each bit pattern indexes a precomputed sum).

@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(32 * kDigitWarps, 2) decode_digits_kernel(cons
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (j < njobs) {
             const int c = (int)__umulhi((uint32_t)j * 2u, p.by_rows), r = j - c * M;
-            if (c < p.chunks) v = __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(p.x) + (size_t)r * p.K + (size_t)c * 128 + aw * 32 + aph * 8));
+            if (c < p.chunks) v = ld_dependent(reinterpret_cast<const uint4 *>(static_cast<const uint16_t *>(p.x) + (size_t)r * p.K + (size_t)c * 128 + aw * 32 + aph * 8));
         }
         return v;
     };
@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(32 * kDigitWarps, 2) decode_digits_kernel(cons
             if constexpr (INT) {
                 const int4 ia = make_int4(__float_as_int(r0), __float_as_int(r1), __float_as_int(r2), __float_as_int(r3));
                 if (p.acc_out) *reinterpret_cast<int4 *>(p.acc_out + (size_t)row * Ng + groups[gq].n0 + 4 * strip) = ia;
-                const float f = __ldg(p.row_scale + row) * p.w_scale;
+                const float f = ld_dependent(p.row_scale + row) * p.w_scale;
                 r0 = (float)ia.x * f; r1 = (float)ia.y * f; r2 = (float)ia.z * f; r3 = (float)ia.w * f;
             }
             const __half2 h01 = __floats2half2_rn(r0, r1), h23 = __floats2half2_rn(r2, r3);

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) decode_mma_kernel(const MmaPar
                 const int ph = R == 1 ? i : R == 2 ? (tig >> 1) + 2 * (i & 1) : tig;
                 raw[c][i] = make_uint4(0u, 0u, 0u, 0u);
                 if (live && (c ? both : active))
-                    raw[c][i] = __ldg(reinterpret_cast<const uint4 *>(p.x + (size_t)b_row * p.K + (size_t)(chunk + c) * 128 + word * 32 + ph * 8));
+                    raw[c][i] = ld_dependent(reinterpret_cast<const uint4 *>(p.x + (size_t)b_row * p.K + (size_t)(chunk + c) * 128 + word * 32 + ph * 8));
             }
 #pragma unroll
         for (int c = 0; c < CPW; ++c)

@@ -652,7 +652,7 @@ mpgemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant_
                     float sc[8];
                     if constexpr (INT8) {
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) sc[e] = __ldg(p.row_scale + min(m0 + t + 2 * e + (odd ? 1 : 0), p.M - 1)) * p.w_scale;
+                        for (int e = 0; e < 8; ++e) sc[e] = ld_dependent(p.row_scale + min(m0 + t + 2 * e + (odd ? 1 : 0), p.M - 1)) * p.w_scale;
                     }
                     tcgen05_wait_ld();
 #pragma unroll
