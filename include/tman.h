@@ -127,7 +127,7 @@ tman_status tman_unpack_weights(const void *packed, size_t packed_bytes,
  * four in groups of 64 or 128 except long calls of 2-bit weights in groups of 64 (K x N above 48 million): codes exact in fp16, activations
  * in fp16 scaled by a power of two (exact down to 2^-21 of the largest of a row's 128 or 256 neighbours, else off by less than 2^-32 of
  * it), sums in fp32.  One and two rows of short reductions (K <= 5120; by columns, bits and group) are multiplied on the integer tensor
- * cores: activations as 32-bit integers (rounded by at most 2^-24 of the largest of 128 neighbours), a block's sum exact, the rest fp32.
+ * cores: activations as 32-bit integers (rounded by at most 2^-24 of the largest of their block), a block's sum exact, the rest fp32.
  * Precision: one row, and everything on tensor cores -- fp32 table entries or better, fp32 sums.  Two to four rows by
  * lookup -- each row of a K-slice is scaled by a power of two into [1, 2) (exactly
  * undone at the end), table entries are rounded to fp16 and the bits x 4 lookups of a 32-activation word

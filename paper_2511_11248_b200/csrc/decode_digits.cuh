@@ -1,13 +1,13 @@
 // Decode of one and two rows on the warp-level integer tensor cores: codes as bytes against activations cut into 8-bit digits.
 //
-// Arithmetic.  A row's activations of a 128-deep chunk of k become 32-bit integers (a power of two brings the largest to
+// Arithmetic.  A row's activations of a block of k become 32-bit integers (a power of two brings the largest to
 // [2^29, 2^30)) and those four signed 8-bit digits, the columns of the MMA's B operand (mma.sync.m16n8k32, unsigned x signed bytes,
 // 32-bit sums, exact).  The codes' bytes are plane words merged by rotations and bit-selects, two codes of three or four bits (four of two)
 // a byte.  They are not taken apart completely: an operand holds a byte's lowest fields f0, f0 + 16 f1 and so on, and
 // the activations carry the differences, x0 - x1 / 16 for f0 and x1 / 16 for f0 + 16 f1, so that the last operand needs no mask.
 // Zero-point and scale are applied to a block's sum, s * (sum - z * sum of the activations), in fp32.
 // Exactness: an activation of a field is an integer after the field's power of two has been taken out, rounded by at most 2^-26 (3 and 4
-// bits) or 2^-24 (2 bits) of the largest of its 128 neighbours; everything up to a block's sum is exact then, the rest fp32.
+// bits) or 2^-24 (2 bits) of the largest of its block (blocks may have scales of any size); everything up to a block's sum is exact then, the rest fp32.
 //
 // Work split.  A CTA owns all of k for its columns, so that nothing is summed through global memory: its eight warps are teams that
 // have the chunks of k among them and take the groups of 32 columns in turn; the warps' sums meet in shared memory once.  The CTA is
@@ -308,31 +308,25 @@ __global__ void __launch_bounds__(32 * kDigitWarps, 2) decode_digits_kernel(cons
                 f[2 * i] = t.x;
                 f[2 * i + 1] = t.y;
             }
-            big = max(big & 0xFFFFu, big >> 16);
-            const uint32_t mine = big;
+            big = max(big & 0xFFFFu, big >> 16);                                 // of the block: 16 / NB lanes
 #pragma unroll
-            for (int mask = 1; mask < 16; mask <<= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, mask));
-            const uint32_t e = max(big >> 10, 1u);                               // biased exponent of the chunk's largest
+            for (int mask = 1; mask < 16 / NB; mask <<= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, mask));
+            const uint32_t e = max(big >> 10, 1u);                               // biased exponent of the block's largest
             back_hi = (99u + e) << 23;                                           // 2^16 / factor
             back_lo = (83u + e) << 23;
             float fac = __uint_as_float((171u - e) << 23);                       // 2^(29 - exponent)
             if (__any_sync(0xffffffffu, e == 31u)) {
                 // Infinities and NaN.  A block of one infinity takes it alone (finite values are nothing beside it) and is multiplied
                 // back by infinity: an infinity, or NaN where its code is the zero-point.  More of them may cancel column by column,
-                // which their sum does not show, so that such a block is NaN, as one with a NaN in it; the other blocks of the
-                // chunk are as if zero.
-                uint32_t blk = mine;
+                // which their sum does not show, so that such a block is NaN, as one with a NaN in it.
                 int infs = 0;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) infs += isinf(f[i]) ? 1 : 0;
 #pragma unroll
-                for (int mask = 1; mask < 16 / NB; mask <<= 1) {
-                    blk = max(blk, __shfl_xor_sync(0xffffffffu, blk, mask));
-                    infs += __shfl_xor_sync(0xffffffffu, infs, mask);
-                }
+                for (int mask = 1; mask < 16 / NB; mask <<= 1) infs += __shfl_xor_sync(0xffffffffu, infs, mask);
                 if (e == 31u) {
                     fac = 1.f;
-                    back_hi = blk > 0x7C00u || infs > 1 ? 0x7FC00000u : blk == 0x7C00u ? 0x7F800000u : 0u;
+                    back_hi = big > 0x7C00u || infs > 1 ? 0x7FC00000u : 0x7F800000u;
                     back_lo = 0u;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) f[i] = isinf(f[i]) ? copysignf(268435456.f, f[i]) : 0.f;

@@ -208,6 +208,20 @@ def test_digits_with_a_large_spread_of_activations(M, bits, G):
     check_large_spread(M, bits, G, 2048, 1096)
 
 
+@pytest.mark.parametrize("M,bits,G", [(1, 2, 64), (1, 3, 32), (1, 2, 32), (1, 4, 64), (2, 4, 64), (2, 2, 64)])
+def test_digits_with_blocks_of_very_different_size(M, bits, G):
+    # every other block has activations of about 1000 under the smallest scale, 2^-24, its neighbours activations of about 2^-10 under scales
+    # near 1, which make up nearly all of the result.  Rounded to a part of the neighbours' largest (3000 x 2^-25 at 2 bits), they would be off
+    # by percents; rounded to a part of their own block's, by nothing that shows.
+    c = synth.small_case(M, 2048, 1096, bits, G, seed=9 + M)
+    rng = np.random.default_rng(bits * G)
+    small = (np.arange(c.K) // G) % 2 == 1
+    c.x[:] = (rng.standard_normal((M, c.K)) * np.where(small, 2.0 ** -10, 1000.0)).astype(np.float16)
+    c.scales[:] = np.where(small[::G, None], rng.uniform(0.5, 1.0, c.scales.shape), 2.0 ** -24).astype(np.float16)
+    got, *_ = run_gemv(c)
+    assert rel_err(got, orc.mpgemm(c.x, c.codes, c.scales, c.zeros, c.group)) <= 5.1e-4
+
+
 @pytest.mark.parametrize("bits,G", [(2, 128), (4, 64), (3, 64)])
 def test_digits_with_an_infinity_and_a_nan(bits, G):
     # the definition column by column: s (q - z) inf is an infinity of the sign of q - z, NaN where q = z; a NaN reaches every column
