@@ -311,7 +311,8 @@ tman_status tman_debug_gemm_plan_for(int M, int K, int N, int bits, int group, i
  * partial sums fit `ws_limit` bytes (0: no limit); among the admitted ones the passes with the least
  * modelled time (fixed cost per pass + per-megabyte cost of the bit planes, fitted to measurements) are
  * chosen.  out (host, 52 ints): [0] passes (0: none admissible -> TMAN_ERR_UNSUPPORTED), [1] workspace
- * KiB the plan needs, [2] modelled time in ns, then six ints per pass from out[4]: rows carried, rows the
+ * KiB the plan needs, [2] modelled time in ns (of the variants; a pass of one or two rows that goes to the integer tensor cores takes less),
+ * [3] what multiplies, two bits a pass from bit 0 (0: lookups, 1: integer tensor cores, 2: fp16 tensor cores), then six ints per pass from out[4]: rows carried, rows the
  * variant can carry, plane words per K-slice, K-slices, CTAs launched, shared-memory bytes per CTA. */
 tman_status tman_debug_gemv_plan(int M, int K, int N, int bits, int group, int sms, size_t ws_limit,
                                  int *out /*host*/);

@@ -216,7 +216,8 @@ def tman_debug_gemv_plan(M, K, N, bits, group, sms=148, ws_limit=0) -> dict:
     _check(lib().tman_debug_gemv_plan(M, K, N, bits, group, sms, C.c_size_t(ws_limit), out), "tman_debug_gemv_plan")
     keys = ("rows", "variant_rows", "words", "slices", "ctas", "smem_bytes")
     return {"ws_kib": out[1], "cost_us": out[2] / 1000.0,
-            "passes": [dict(zip(keys, out[4 + 6 * i: 10 + 6 * i])) for i in range(out[0])]}
+            "passes": [dict(zip(keys, out[4 + 6 * i: 10 + 6 * i]), kernel=("lookup", "digits", "mma")[out[3] >> 2 * i & 3])
+                       for i in range(out[0])]}
 
 
 def tman_dequant_ternary_int8(packed, K, N, group, w8, ws, stream=None) -> None:

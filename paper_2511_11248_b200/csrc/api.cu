@@ -316,6 +316,7 @@ tman_status tman_debug_gemv_plan(int M, int K, int N, int bits, int group, int s
     for (int i = 0; i < g.npass; ++i) {
         int *o = out + 4 + 6 * i;
         o[0] = g.pass[i].rows; o[1] = g.pass[i].variant_rows; o[2] = g.pass[i].words;
+        out[3] |= (g.pass[i].digits ? 1 : g.pass[i].mma ? 2 : 0) << (2 * i);
         o[3] = g.pass[i].nkappa; o[4] = g.pass[i].nkappa * g.pass[i].ctas_per_slice; o[5] = g.pass[i].smem_bytes;
     }
     return g.npass ? TMAN_OK : TMAN_ERR_UNSUPPORTED;

@@ -197,6 +197,20 @@ def test_decode_plan_choices_and_limits(lib):
     assert B.tman_debug_gemv_plan(4, K, N, 2, G)["cost_us"] < B.tman_debug_gemv_plan(4, K, N, 4, G)["cost_us"]
 
 
+def test_decode_plan_says_what_multiplies(lib):
+    from paper_2511_11248_b200 import binding as B
+    want = {(1, 14336, 4096, 4, 128): "lookup", (1, 4096, 512, 4, 128): "lookup", (2, 4096, 14336, 4, 32): "lookup", (4, 4096, 14336, 4, 32): "lookup",
+            (1, 2048, 2048, 4, 128): "digits", (2, 2048, 8192, 2, 128): "digits", (1, 512, 1024, 2, 64): "digits",
+            (4, 4096, 14336, 4, 128): "mma", (5, 4096, 14336, 2, 32): "mma", (8, 14336, 4096, 3, 64): "mma"}
+    for call, kernel in want.items():
+        assert [q["kernel"] for q in B.tman_debug_gemv_plan(*call)["passes"]] == [kernel], call
+    # several passes: each says its own (rows beyond the integer tensor cores' two go to the other kernels)
+    ws1 = B.tman_workspace_bytes(B.OP_GEMV, 1, 4096, 512, 4, 128)
+    assert [q["kernel"] for q in B.tman_debug_gemv_plan(3, 4096, 512, 4, 128, ws_limit=ws1)["passes"]] == ["lookup"] * 2
+    ws1 = B.tman_workspace_bytes(B.OP_GEMV, 1, 2048, 2048, 4, 128)
+    assert set(q["kernel"] for q in B.tman_debug_gemv_plan(3, 2048, 2048, 4, 128, ws_limit=ws1)["passes"]) == {"digits"}
+
+
 def test_marshalled_calls_report_status_and_bad_arguments(lib):
     """The hot entry points go through the _marshal extension: statuses come back as TmanError, sizes and addresses are
     read from the tensors, and arguments of the wrong kind raise instead of reaching the library."""
