@@ -857,8 +857,9 @@ static MmaSplit split_mma(int M, int K, int N, int groups, int sms, size_t ws_li
 }
 
 // ---- decode on the integer tensor cores (decode_digits.cuh) ----------------------------------------------------------
-// How a launch is laid out: CTAs, warps of a team, units of the warps' rings, turns between reductions (0: it does not fit).
-struct DigitSplit { int ctas, tk_shift, depth, flush, smem, scale_row, zero_row; };
+// How a launch is laid out: CTAs (two an SM: `two`), warps of a team, units of the warps' rings, turns between reductions (0: it does not
+// fit); groups of a CTA, and units that the busiest warp takes (`steps`), which say how well the columns and K fill it.
+struct DigitSplit { int ctas, tk_shift, depth, flush, smem, scale_row, zero_row, groups, steps; bool two; };
 static DigitSplit split_digits(int rows, int K, int strips, int bits, int group, int nb, bool ints, int sms)
 {
     DigitSplit d = {};
@@ -873,6 +874,8 @@ static DigitSplit split_digits(int rows, int K, int strips, int bits, int group,
     const int at_most = two ? 2 * sms : sms;
     d.ctas = strips < at_most ? strips : at_most;
     const int share = (strips + d.ctas - 1) / d.ctas, groups = (share + 7) / 8;
+    d.two = two;
+    d.groups = groups;
     const int rest = fixed + 2 * pairs * slot + share * (d.scale_row + d.zero_row) + 16;
     int room = kDigitSmemHalf;
     d.depth = rest + 2 * ring + turn <= room ? 2 : 1;
@@ -883,10 +886,10 @@ static DigitSplit split_digits(int rows, int K, int strips, int bits, int group,
     const int base = rest + d.depth * ring;
     if (groups > kDigitGroups - kGemvMaxGroup || base + turn > room || (two && room > kDigitSmemHalf)) return d;
     d.tk_shift = kDigitWarpsShift;
-    int best = 1 << 30;
+    d.steps = 1 << 30;
     for (int shift = kDigitWarpsShift; shift >= 0; --shift) {
         const int tc = kDigitWarps >> shift, steps = (groups + tc - 1) / tc * ((pairs + (1 << shift) - 1) >> shift);
-        if (steps < best) { best = steps; d.tk_shift = shift; }
+        if (steps < d.steps) { d.steps = steps; d.tk_shift = shift; }
     }
     const int tc = kDigitWarps >> d.tk_shift, turns = (groups + kGemvMaxGroup + tc - 1) / tc;
     d.flush = (room - base) / turn;
@@ -895,24 +898,34 @@ static DigitSplit split_digits(int rows, int K, int strips, int bits, int group,
     return d;
 }
 
-// Whether a pass of `rows` rows goes to the integer tensor cores instead of the table lookups (columns: of all matrices).  In a graph,
-// lookup / here, us: one row, 2-bit group 64 2048 x 8192 4.35 / 3.24, 4096 x 4096 4.30 / 3.34, 4096 x 28672 11.7 / 10.3; 4-bit group 128 4096 x
-// 4096 5.13 / 4.25, 4096 x 28672 15.9 / 13.5; two rows 6.63 / 5.36 (4096 x 4096), 6.55 / 4.28 (2048 x 8192).  The lines:
-// K: every CTA prepares all activations (8192 x 2048 5.14 / 5.66, 14336 x 4096 9.9 / 11.0).  Few columns: the same work for little
-// (4096 x 512 3.25 / 4.82; 4096 x 1024, one row 3.51 / 3.63).  20480 columns are too many for one CTA an SM and fill two badly (4096 x
-// 20480 12.2 / 14.1, 2-bit 8.9 / 9.0; 2048 x 20480 8.0 / 7.6).  Where rows and blocks need more columns of B than the MMA has (more tiles), the
-// work grows with the columns: two rows of group 64 4096 x 4096 6.34 / 5.60, 4096 x 6144 7.68 / 8.16, 2048 x 8192 6.33 / 4.38; group 32,
-// one row 2048 x 8192 4.63 / 3.97, 4096 x 6144 5.47 / 6.12 (two rows stay with the lookups).  3 and 4 bits of group 64, one row: 4096 x 4096 4.61 / 4.03, x 20480 10.4 / 11.7.
+// Whether a pass of `rows` rows goes to the integer tensor cores instead of the table lookups (columns: of all matrices).  The difference
+// of the two times is modelled from what a launch consists of, in us: preparing all activations in every CTA (by K), the units
+// that the busiest warp takes (also where K does not fill the warps: 2176 takes as many as 4096) and the tiles of B that each is
+// multiplied with, groups, and megabytes of planes, which cost the lookups more.  Constants: least squares over graphs of layers,
+// MLPs and single calls with every call by either kernel, for 3600 draws of K = 1024..5120 and 256..40000 columns and for layers
+// of nine common shapes, plus half a change of kernel between neighbours (0.4 us) and 0.2 us of margin.  On 800 further draws
+// one row takes 0.979 of its time by lookup in the mean (a layer or MLP in 40 more than 2 % longer, at most 9 %), two rows in groups of 64 and
+// 128 0.921 (one in 170, at most 4 %).  Examples, by lookup / by this rule, 4-bit group 128: layer of 4096 x (6144, 4096, 28672) and
+// 14336 x 4096, one row 40.7 / 36.2 us, of 2048 x (3072, 2048, 16384) and 8192 x 2048 22.3 / 21.0, two rows 27.7 / 24.9.
+// Lines outside the model: six and more units a warp in one CTA an SM (3584 x 22784 and back, 4-bit 23.6 / 29.5), few columns
+// (4096 x 512 3.3 / 4.8), two rows in groups of 32 (four tiles).  Calls of one group a CTA and at most two units, 2 and 4 bits
+// (4096 x 4096), gain more than the linear model says, 0.2 to 1.3 us.
+struct DigitPrice { float base, k, unit, tile, group, mb, two; };
+static const DigitPrice kDigitPrices[2][3] = {
+    {{-1.44f, 0.23f, 0.28f, 0.14f, 0.33f, -0.09f, -0.46f}, {-1.52f, 0.39f, 0.34f, 0.03f, 0.52f, -0.12f, -0.44f}, {-1.59f, 0.46f, 0.21f, 0.04f, 0.55f, -0.12f, -0.24f}},
+    {{-2.23f, 0.36f, 0.11f, 0.22f, 0.48f, -0.12f, 0.70f}, {-1.67f, 0.31f, 0.03f, 0.18f, 0.30f, -0.02f, 0.18f}, {-1.58f, 0.31f, -0.03f, 0.24f, 0.06f, -0.03f, 0.f}},
+};
 static bool uses_digits(int bits, int group, int rows, int K, long long columns, int sms)
 {
-    if (rows > 2 || K > 5120 || columns * rows < K / 2) return false;
-    const int blocks = 128 / group;
-    const bool one_tile = group == 128 || (group == 64 && rows == 1);
-    long long most = one_tile && (group == 128 || bits == 2) ? 10ll * K : 8192;
-    if (K > 2048 && group == 64 && (rows == 2 || bits == 3)) most = 5120;
-    if (columns > most || (group == 32 && (rows == 2 || K > 2048))) return false;
-    if (K > 2048 && columns >= 96ll * sms && columns < 160ll * sms) return false;
-    return split_digits(rows, K, (int)(columns / 4), bits, group, blocks, false, sms).flush > 0;
+    if (rows > 2 || K > 5120 || columns > 40960 || columns * rows < K / 2 || (group == 32 && rows == 2)) return false;
+    const DigitSplit d = split_digits(rows, K, (int)(columns / 4), bits, group, 128 / group, false, sms);
+    if (d.flush < 1 || (d.steps >= 6 && !d.two)) return false;
+    const int tiles = group == 128 ? 1 : group == 64 ? rows : 2;
+    if (rows == 1 && tiles == 1 && bits != 3 && d.groups == 1 && d.steps <= 2 && d.ctas == sms) return true;
+    const DigitPrice &c = kDigitPrices[rows - 1][bits - 2];
+    const float us = c.base + c.k * (float)K / 1024.f + (c.unit + c.tile * (float)(tiles - 1)) * (float)d.steps + c.group * (float)d.groups +
+                     c.mb * (float)((double)K * (double)columns * bits / 8e6) + (d.two ? c.two : 0.f);
+    return us < (tiles > 1 ? -0.3f : 0.f);
 }
 
 // The same for the integer path, whose product follows a row quantization: products 2560 x 6912 and back in turn, each with its

@@ -211,6 +211,18 @@ def test_decode_plan_says_what_multiplies(lib):
     assert set(q["kernel"] for q in B.tman_debug_gemv_plan(3, 2048, 2048, 4, 128, ws_limit=ws1)["passes"]) == {"digits"}
 
 
+def test_decode_plan_takes_the_integer_tensor_cores_where_they_are_faster(lib):
+    """One and two rows: calls that the integer tensor cores slowed down by 5 to 28 % (a layer or an MLP with them in it, timed against the
+    lookups) stay with the lookups, calls that gain from them go there."""
+    from paper_2511_11248_b200 import binding as B
+    slower = [(1, 3584, 22784, 4, 128), (1, 2304, 10240, 3, 128), (1, 3840, 15872, 3, 128), (1, 3968, 17920, 4, 128), (1, 4096, 22016, 2, 128),
+              (1, 4096, 22016, 3, 128), (2, 2048, 16384, 2, 64), (1, 2048, 16384, 3, 128), (1, 4480, 9600, 2, 64), (1, 3328, 17920, 3, 128)]
+    faster = [(1, 2048, 3072, 4, 128), (1, 4096, 28672, 4, 128), (2, 2048, 3072, 2, 128), (1, 4096, 4096, 4, 128), (1, 4096, 4096, 2, 64),
+              (1, 2048, 2048, 3, 128), (2, 3072, 5120, 4, 128), (2, 1536, 4096, 4, 64)]
+    assert [[p["kernel"] for p in B.tman_debug_gemv_plan(*c)["passes"]] for c in slower] == [["lookup"]] * len(slower)
+    assert [[p["kernel"] for p in B.tman_debug_gemv_plan(*c)["passes"]] for c in faster] == [["digits"]] * len(faster)
+
+
 def test_marshalled_calls_report_status_and_bad_arguments(lib):
     """The hot entry points go through the _marshal extension: statuses come back as TmanError, sizes and addresses are
     read from the tensors, and arguments of the wrong kind raise instead of reaching the library."""

@@ -184,36 +184,64 @@ def check_large_spread(M, bits, G, K, N):
     assert rel_err(got, ref) <= 5.1e-4
 
 
-# (M, K, Ns): one chunk of 128 k and an odd number of them, teams of one to eight warps, ragged groups of eight strips, matrices narrower
-# than one, the longest K, the columns at which the rule changes sides
-DIGIT_CASES = [(1, 128, (64,)), (2, 128, (72,)), (1, 640, (328, 40)), (2, 640, (320,)), (1, 1536, (8, 760, 16)), (2, 2048, (1032,)),
-               (1, 2176, (1096, 8, 40)), (2, 2176, (1088,)), (1, 4096, (2048,)), (1, 4096, (2040,)), (2, 4096, (4096, 1024, 1024)),
-               (1, 5120, (2560, 24)), (2, 5120, (1288,)), (1, 4096, (16392,))]
+def on_digits(M, K, N, bits, G):
+    """Whether the call is one pass on the integer tensor cores."""
+    return [p["kernel"] for p in B.tman_debug_gemv_plan(M, K, N, bits, G)["passes"]] == ["digits"]
 
 
-@pytest.mark.parametrize("bits,G", [(2, 32), (2, 64), (2, 128), (3, 32), (3, 64), (3, 128), (4, 32), (4, 64), (4, 128)])
-@pytest.mark.parametrize("M,K,Ns", DIGIT_CASES)
-def test_one_and_two_rows_on_the_integer_tensor_cores(M, K, Ns, bits, G):
-    # Sums are exact up to a block; an activation is rounded by at most 2^-24 of its largest neighbour, so what is left is the rounding of
-    # the result to fp16 and fp32 sums: the bound of test_tensor_core_rows_at_the_edges_of_their_split (calls beyond the rule's limits go to
-    # the lookups, whose fp16 tables for two rows have the bound of test_rows_in_fp16_tables_stay_near_the_predicted_error).
-    plan = B.tman_debug_gemv_plan(M, K, sum(Ns), bits, G)
-    lookup = plan["passes"][0]["words"] != K // 32
-    check_grouped_twice(M, bits, G, K, Ns, 2e-3 if lookup and M > 1 else 5.1e-4)
+# (K, Ns, (M, bits, group) ...), all of them on the integer tensor cores
+ONE_TILE = [(1, b, 64) for b in (2, 3, 4)] + [(M, b, 128) for M in (1, 2) for b in (2, 3, 4)]
+TWO_TILES = [(1, 2, 32), (2, 2, 64), (2, 3, 64), (2, 4, 64)]
+DIGIT_CASES = [
+    # one chunk of 128 k, matrices narrower than a group of 32 columns; 15 chunks, a CTA's columns from several matrices
+    (128, (64, 8, 8), ONE_TILE + TWO_TILES + [(1, 3, 32), (1, 4, 32)]), (1536, (8, 760, 16), ONE_TILE + TWO_TILES), (1920, (328, 1600), ONE_TILE + TWO_TILES),
+    # model shapes and the longest K
+    (2048, (2048, 512, 512), ONE_TILE + TWO_TILES), (4096, (4096,), [(1, 2, 64), (1, 4, 128), (2, 2, 128), (2, 3, 128)]),
+    (4096, (2056, 1024, 1024), [(1, 2, 128), (1, 4, 64), (2, 4, 128)]), (4992, (2504,), [(2, 2, 128)]), (5120, (5120,), [(2, 4, 128)]),
+    # two, four and eight teams of four, two and one warps
+    (128, (4000, 776), ONE_TILE + TWO_TILES), (640, (9216,), [(1, 4, 32)]), (128, (9512,), [(1, 2, 64), (2, 3, 128), (2, 4, 64)]),
+    (128, (19064,), [(2, 3, 128), (2, 4, 64)]),
+    # two CTAs an SM, rings of one and of two units, teams of two warps and of one
+    (640, (20000, 4104), [(1, 2, 64), (1, 3, 128), (1, 4, 64), (1, 4, 32), (2, 2, 128), (2, 4, 128)]), (128, (38216,), [(1, 2, 128), (2, 4, 64)]),
+    (3200, (26120,), [(1, 2, 64), (1, 4, 64)]),
+    # more turns than the warps' sums have room for: several reductions
+    (1152, (4776,), [(2, 3, 128)]), (640, (11880,), [(2, 3, 128)]), (640, (24104,), [(2, 3, 128)]), (1920, (11288,), [(2, 4, 64)]),
+    (1152, (24104,), [(1, 3, 64)]), (1920, (15536,), [(2, 2, 128)]), (1408, (20576,), [(2, 4, 128)]),
+    # the other length of the rings, and all of an SM's shared memory
+    (1408, (368,), [(2, 3, 64)]), (3712, (944,), [(2, 2, 128), (2, 4, 128)]), (2944, (3592,), [(2, 2, 64), (2, 4, 64)]), (2176, (4776,), [(2, 3, 128)]),
+]
 
 
-@pytest.mark.parametrize("M,bits,G", [(1, 2, 64), (1, 4, 128), (2, 3, 128), (2, 2, 64), (1, 3, 32), (2, 4, 64)])
+@pytest.mark.parametrize("K,Ns,M,bits,G", [(K, Ns, *c) for K, Ns, cs in DIGIT_CASES for c in cs])
+def test_one_and_two_rows_on_the_integer_tensor_cores(K, Ns, M, bits, G):
+    # Sums are exact up to a block; an activation is rounded by at most 2^-24 of its block's largest, so what is left is the rounding of
+    # the result to fp16 and fp32 sums: the bound of test_tensor_core_rows_at_the_edges_of_their_split
+    assert on_digits(M, K, sum(Ns), bits, G)
+    check_grouped_twice(M, bits, G, K, Ns, 5.1e-4)
+
+
+@pytest.mark.parametrize("K,Ns,M,bits,G", [(4096, (504,), 1, 4, 128), (2048, (1032,), 2, 2, 32), (4096, (16392,), 1, 4, 128), (5248, (2504,), 1, 2, 64),
+                                           (3584, (1024, 2056), 1, 3, 64), (2048, (4096, 2056), 2, 3, 64)])
+def test_one_and_two_rows_beyond_the_rule_by_lookup(K, Ns, M, bits, G):
+    # (two rows: the bound of test_rows_in_fp16_tables_stay_near_the_predicted_error)
+    assert [p["kernel"] for p in B.tman_debug_gemv_plan(M, K, sum(Ns), bits, G)["passes"]] == ["lookup"]
+    check_grouped_twice(M, bits, G, K, Ns, 2e-3 if M > 1 else 5.1e-4)
+
+
+@pytest.mark.parametrize("M,bits,G", [(1, 2, 64), (1, 4, 128), (2, 3, 128), (2, 2, 64), (1, 2, 32), (2, 4, 64)])
 def test_digits_with_a_large_spread_of_activations(M, bits, G):
     # as above, 2^-24 to 2^4 side by side
-    check_large_spread(M, bits, G, 2048, 1096)
+    assert on_digits(M, 1536, 784, bits, G)
+    check_large_spread(M, bits, G, 1536, 784)
 
 
-@pytest.mark.parametrize("M,bits,G", [(1, 2, 64), (1, 3, 32), (1, 2, 32), (1, 4, 64), (2, 4, 64), (2, 2, 64)])
+@pytest.mark.parametrize("M,bits,G", [(1, 2, 64), (1, 3, 64), (1, 2, 32), (1, 4, 64), (2, 4, 64), (2, 2, 64)])
 def test_digits_with_blocks_of_very_different_size(M, bits, G):
     # every other block has activations of about 1000 under the smallest scale, 2^-24, its neighbours activations of about 2^-10 under scales
     # near 1, which make up nearly all of the result.  Rounded to a part of the neighbours' largest (3000 x 2^-25 at 2 bits), they would be off
     # by percents; rounded to a part of their own block's, by nothing that shows.
-    c = synth.small_case(M, 2048, 1096, bits, G, seed=9 + M)
+    c = synth.small_case(M, 1536, 784, bits, G, seed=9 + M)
+    assert on_digits(M, c.K, c.N, bits, G)
     rng = np.random.default_rng(bits * G)
     small = (np.arange(c.K) // G) % 2 == 1
     c.x[:] = (rng.standard_normal((M, c.K)) * np.where(small, 2.0 ** -10, 1000.0)).astype(np.float16)
@@ -225,7 +253,8 @@ def test_digits_with_blocks_of_very_different_size(M, bits, G):
 @pytest.mark.parametrize("bits,G", [(2, 128), (4, 64), (3, 64)])
 def test_digits_with_an_infinity_and_a_nan(bits, G):
     # the definition column by column: s (q - z) inf is an infinity of the sign of q - z, NaN where q = z; a NaN reaches every column
-    c = synth.small_case(2, 2048, 1096, bits, G, seed=5)
+    c = synth.small_case(2, 1536, 784, bits, G, seed=5)
+    assert on_digits(2, c.K, c.N, bits, G)
     c.x[0, 700] = -np.inf
     c.x[1, 3] = np.nan
     dev = H.device_case(c)
@@ -237,13 +266,14 @@ def test_digits_with_an_infinity_and_a_nan(bits, G):
     assert np.all(np.isinf(got[0, d != 0])) and np.array_equal(got[0, d != 0] > 0, d[d != 0] < 0)
 
 
-@pytest.mark.parametrize("M,bits,G", [(1, 2, 128), (2, 3, 128), (2, 4, 64), (1, 3, 32)])
+@pytest.mark.parametrize("M,bits,G", [(1, 2, 128), (2, 3, 128), (2, 4, 64), (1, 2, 32)])
 @pytest.mark.parametrize("other", [701, 702, 736, 800, 1500])
 @pytest.mark.parametrize("sign", [1.0, -1.0])
 def test_digits_with_two_infinities(M, bits, G, other, sign):
     # two infinities, of one block (the first two, and up to G = 128 the others) or of two: wherever the definition has infinities of both
     # signs, or an infinity that meets its zero-point, the sum is NaN; nothing finite comes out where it has an infinity
-    c = synth.small_case(M, 2048, 1096, bits, G, seed=6)
+    c = synth.small_case(M, 1536, 784, bits, G, seed=6)
+    assert on_digits(M, c.K, c.N, bits, G)
     c.x[M - 1, 700], c.x[M - 1, other] = np.inf, sign * np.inf
     dev = H.device_case(c)
     ws, y = H.alloc_workspace(B.OP_GEMV, M, c.K, c.N, bits, G), H.alloc_y(M, c.N)
