@@ -216,8 +216,41 @@ def test_int8_prefill_of_large_tiles_of_odd_units():
 
 
 @pytest.mark.parametrize("M,K,N,group", [(2, 1024, 40, 64), (3, 2560, 264, 128), (4, 6912, 2560, 128), (5, 1152, 72, 32),
-                                         (8, 2560, 6912, 64), (7, 16384, 16, 128)])
+                                         (8, 2560, 6912, 64), (7, 16384, 16, 128), (6, 4992, 1288, 64), (7, 4352, 1920, 128)])
 def test_ternary_decode_with_several_rows(M, K, N, group):
+    check_several_rows(M, K, N, group, prepared=True)
+
+
+# an odd number of 128-deep chunks, ragged columns, an odd row in the last pair of rows; rings of one unit and of two; teams of eight to two
+# warps; two CTAs an SM; several reductions; half an SM's shared memory and all of it
+@pytest.mark.parametrize("M,K,N,group", [(2, 640, 1032, 32), (3, 1152, 1288, 64), (5, 2176, 2568, 128), (6, 1920, 1928, 64), (7, 2176, 2056, 128), (8, 1152, 520, 32),
+                                         (2, 3712, 2456, 128), (4, 2304, 4360, 32), (3, 3456, 5312, 128), (7, 1152, 7488, 64), (6, 1408, 5040, 128),
+                                         (2, 640, 19064, 128), (4, 640, 9512, 64), (8, 640, 4776, 128), (3, 640, 24008, 128), (5, 3968, 1096, 128), (2, 5120, 2568, 64)])
+def test_ternary_decode_with_several_rows_on_the_integer_tensor_cores(M, K, N, group):
+    # the area of partial sums holds zeros, which a lookup kernel would take for its sums: this kernel has none
+    check_several_rows(M, K, N, group, prepared=False)
+
+
+@pytest.mark.parametrize("M,K,N", [(2, 5120, 2568), (3, 1152, 1288), (6, 2176, 1032), (8, 1152, 520)])
+def test_ternary_decode_of_the_largest_integers(M, K, N):
+    # the first columns' weights have the signs of the rows, so that the sums are as large as they can be; -32768 is no quantized value, but
+    # the call takes it
+    _, t, _, s_w = ternary_case(1, K, N, seed=K)
+    rng = np.random.default_rng(N)
+    a = rng.choice(np.array([-32768, -32767, 32767], dtype=np.int16), size=(M, K))
+    for m in range(M):
+        t[:, m] = np.sign(a[m])
+    acc_ref = a.astype(np.int64) @ t.astype(np.int64)
+    packed = pack_ternary((t + 1).astype(np.uint8), 128)
+    ws = H.guarded_bytes(B.tman_workspace_bytes(B.OP_TERNARY, M, K, N, 2, 128), "workspace")
+    B.tman_workspace_init(ws)
+    y, acc = H.alloc_y(M, N), H.guarded_bytes(M * N * 4, "acc_i32").view(torch.int32).view(M, N)
+    B.tman_mpgemv_ternary(packed, torch.from_numpy(a).cuda(), torch.full((8,), 2.0 ** -15, device="cuda"), s_w, y, acc, M, K, N, 128, ws)
+    assert B.tman_read_status(ws) == 0
+    assert np.array_equal(acc.cpu().numpy().astype(np.int64), acc_ref)
+
+
+def check_several_rows(M, K, N, group, prepared):
     x, t, q, s_w = ternary_case(M, K, N, seed=7 * M + K + N, spread=1.5)
     a_ref, s_ref = oi.quantize_rows(x, 32767)
     acc_ref = oi.ternary_lut_matmul(a_ref, q)
@@ -228,7 +261,10 @@ def test_ternary_decode_with_several_rows(M, K, N, group):
     s = H.guarded_bytes(256, "row_scale").view(torch.float32)
     B.tman_quantize_rows(xd, M, K, 32767, a, s)
     ws = H.guarded_bytes(B.tman_workspace_bytes(B.OP_TERNARY, M, K, N, 2, group), "workspace")
-    B.tman_workspace_init(ws)
+    if prepared:
+        B.tman_workspace_init(ws)
+    else:
+        ws.zero_()
     y = H.alloc_y(M, N)
     acc = H.guarded_bytes(M * N * 4, "acc_i32").view(torch.int32).view(M, N)
     for _ in range(2):
