@@ -124,10 +124,12 @@ tman_status tman_unpack_weights(const void *packed, size_t packed_bytes,
  * built in shared memory, packed bit-plane bytes index them, partial sums are
  * shift-accumulated per quantization block, scaled, and summed across blocks in fp32.
  * M in [1, 8], normally in one pass over the weights.  Five rows and more are multiplied on the tensor cores instead, and three and
- * four in groups of 64 or 128 except long calls of 2-bit weights in groups of 64 (K x N above 48 million): codes exact in fp16, activations
- * in fp16 scaled by a power of two (exact down to 2^-21 of the largest of a row's 128 or 256 neighbours, else off by less than 2^-32 of
- * it), sums in fp32.  One and two rows of short reductions (K <= 5120; by columns, bits and group) are multiplied on the integer tensor
- * cores: activations as 32-bit integers (rounded by at most 2^-24 of the largest of their block), a block's sum exact, the rest fp32.
+ * four in groups of 64 or 128 except long calls of 2-bit weights in groups of 64 (K x N above 48 million): codes exact in fp16,
+ * activations in fp16 scaled by a power of two (exact down to 2^-21 of the largest of a row's 128 or 256 neighbours, else off by less
+ * than 2^-32 of it), sums in fp32.  One and two rows of short reductions (K <= 5120) are multiplied on the integer tensor cores where
+ * that is modelled to be faster (see tman_debug_gemv_plan): activations as 32-bit integers (rounded by at most 2^-24 of the largest of
+ * their block), a block's sum exact, the rest fp32.  An infinity in x gives the definition's infinities and NaN there where it is alone
+ * in its block, by lookup and beside others NaN.
  * Precision: one row, and everything on tensor cores -- fp32 table entries or better, fp32 sums.  Two to four rows by
  * lookup -- each row of a K-slice is scaled by a power of two into [1, 2) (exactly
  * undone at the end), table entries are rounded to fp16 and the bits x 4 lookups of a 32-activation word
@@ -165,9 +167,11 @@ tman_status tman_mpgemv_grouped(int count, const void *const *packed /*host*/, c
 tman_status tman_quantize_rows(const void *x_f16, int M, int K, int qmax, int16_t *a_i16, float *row_scale,
                                tman_stream_t stream);
 
-/* Decode of M rows (1 <= M <= 8, in passes of up to four rows; K <= 16384): the bit-serial table lookup of
- * tman_mpgemv on integers (two rows and more with K <= 5120: the integer tensor cores).  Tables hold exact integer sums of activations, lookups are shift-accumulated,
- * the activation sum is subtracted once (zero-point 1), K-slices are added as 32-bit integers;
+/* Decode of M rows (1 <= M <= 8; K <= 16384): the bit-serial table lookup of tman_mpgemv on integers, in passes of up to four
+ * rows.  Tables hold exact integer sums of activations, lookups are shift-accumulated, the activation sum is subtracted once
+ * (zero-point 1), K-slices are added as 32-bit integers.  Two rows and more with K <= 5120 and N >= K / (2 M) are multiplied on the
+ * integer tensor cores instead, all rows in one pass, where their activations fit an SM's shared memory (seven rows of 4352 do
+ * not).  Either way
  *   y[m][n] = fp16( row_scale[m] * w_scale * sum_k a[m][k] * (q[k][n] - 1) ).
  * acc_i32 (device, int32 [M][N], 16-byte aligned, may be NULL) receives the exact integer sums.
  * Workspace: tman_workspace_bytes(3, M, K, N, 2, group), prepared with tman_workspace_init; status word
@@ -311,8 +315,8 @@ tman_status tman_debug_gemm_plan_for(int M, int K, int N, int bits, int group, i
  * partial sums fit `ws_limit` bytes (0: no limit); among the admitted ones the passes with the least
  * modelled time (fixed cost per pass + per-megabyte cost of the bit planes, fitted to measurements) are
  * chosen.  out (host, 52 ints): [0] passes (0: none admissible -> TMAN_ERR_UNSUPPORTED), [1] workspace
- * KiB the plan needs, [2] modelled time in ns (of the variants; a pass of one or two rows that goes to the integer tensor cores takes less),
- * [3] what multiplies, two bits a pass from bit 0 (0: lookups, 1: integer tensor cores, 2: fp16 tensor cores), then six ints per pass from out[4]: rows carried, rows the
+ * KiB the plan needs, [2] modelled time in ns (of the variants: a pass of one or two rows that goes to the integer tensor cores is
+ * counted as by lookup), [3] what multiplies, two bits a pass from bit 0 (0: lookups, 1: integer tensor cores, 2: fp16 tensor cores), then six ints per pass from out[4]: rows carried, rows the
  * variant can carry, plane words per K-slice, K-slices, CTAs launched, shared-memory bytes per CTA. */
 tman_status tman_debug_gemv_plan(int M, int K, int N, int bits, int group, int sms, size_t ws_limit,
                                  int *out /*host*/);

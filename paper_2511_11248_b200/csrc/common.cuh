@@ -94,10 +94,11 @@ inline int sm_count()
     return d ? d->sms.load(std::memory_order_acquire) : 0;
 }
 
-// Asks for the common split, of the decode kernels that alternate in a layer of one or two rows, of an SM's 256 KB between shared memory (132 KB) and L1: an SM changes its split only when it
-// is idle, so that kernels of different splits do not follow one another without a gap (a layer of alternating kernels 76 -> 86 us).
-// 132 KB hold two CTAs of decode_digits_kernel and leave the lookups the L1 that their loads in flight pass through (with 228 KB of shared
-// memory 14336 x 4096, 4-bit, takes 12.3 us instead of 9.8).  A hint: failure changes nothing.
+// Asks for the split of an SM's 256 KB between shared memory (132 KB) and L1 that the decode kernels which alternate in a layer of one or
+// two rows have in common: an SM changes its split only when it is idle, so that kernels of different splits do not follow one another
+// without a gap (a layer of alternating kernels 76 -> 86 us).  132 KB hold two CTAs of decode_digits_kernel and leave the lookups the L1
+// that their loads in flight pass through (with 228 KB of shared memory 14336 x 4096, 4-bit, takes 12.3 us instead of 9.8).  A hint:
+// failure changes nothing.
 constexpr int kSharedPercent = 58;        // of 228 KB
 template <typename Kernel> inline void prefer_common_split(Kernel kern)
 {

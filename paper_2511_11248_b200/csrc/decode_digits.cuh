@@ -7,7 +7,8 @@
 // the activations carry the differences, x0 - x1 / 16 for f0 and x1 / 16 for f0 + 16 f1, so that the last operand needs no mask.
 // Zero-point and scale are applied to a block's sum, s * (sum - z * sum of the activations), in fp32.
 // Exactness: an activation of a field is an integer after the field's power of two has been taken out, rounded by at most 2^-26 (3 and 4
-// bits) or 2^-24 (2 bits) of the largest of its block (blocks may have scales of any size); everything up to a block's sum is exact then, the rest fp32.
+// bits) or 2^-24 (2 bits) of the largest of its block (blocks may have scales of any size); everything up to a block's sum is exact
+// then, the rest fp32.
 //
 // Work split.  A CTA owns all of k for its columns, so that nothing is summed through global memory: its eight warps are teams that
 // have the chunks of k among them and take the groups of 32 columns in turn; the warps' sums meet in shared memory once.  The CTA is
@@ -17,8 +18,8 @@
 // What bounds it: issue slots and integer pipe, about 190 instructions (97 on the half-rate integer pipe, 76 of them the merging) per 32
 // columns x 128 k, and at the ends 0.8 us from the predecessor's last store to this call's activations, 1.0 us until their digits are
 // there, 0.4 us for the sums; HBM at the large end (4096 x 28672, 4-bit group 128 13.5 us, 4.6 TB/s; by lookup 15.9).  Measured and
-// dropped: 16 warps of 64 registers, two CTAs an SM (spills: 19.3), 16 warps of 128 registers, one (14.9; 4096 x 4096 4.5 against 4.2), scales by ordinary loads
-// a unit ahead (4096 x 6144 6.5 against 5.9), rings of 64-byte pieces of eight strips (as fast).
+// dropped: 16 warps of 64 registers, two CTAs an SM (spills: 19.3), 16 warps of 128 registers, one (14.9; 4096 x 4096 4.5 against
+// 4.2), scales by ordinary loads a unit ahead (4096 x 6144 6.5 against 5.9), rings of 64-byte pieces of eight strips (as fast).
 #pragma once
 #include "decode_mma.cuh"
 
@@ -150,7 +151,7 @@ template <int BITS> struct CodeBytes {
 //   NB = 1: four digits of rows 2 t and 2 t + 1 (t = n-tile).   NB = 2: four digits of row t, block 0 and block 1; a word of the other
 //   block meets zeros.   NB = 4: two digits (those of pair t & 1) of row t >> 1, blocks 0..3.
 // NT = n-tiles.  INT: 2-bit codes, zero-point 1, 16-bit integer activations (times 64, 16, 4, 1 by their field, so that three digits hold
-// them): the sums stay 32-bit integers to the end.
+// them): the sums stay 32-bit integers to the end.  (Four tiles of it spill 76 bytes: seven rows 2048 x 2176 and back 16.8 us, by lookup 24.8.)
 template <int BITS, int NB, int NT, int DEPTH, bool INT>
 __global__ void __launch_bounds__(32 * kDigitWarps, 2) decode_digits_kernel(const __grid_constant__ DigitParams p)
 {
@@ -458,64 +459,64 @@ __global__ void __launch_bounds__(32 * kDigitWarps, 2) decode_digits_kernel(cons
                 uint4 b[NT];
 #pragma unroll
                 for (int t = 0; t < NT; ++t) b[t] = lds128(b_at[t] + b_off);
-            CodeBytes<BITS> cb[4];
+                CodeBytes<BITS> cb[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t ww[BITS];
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t ww[BITS];
 #pragma unroll
-                for (int i = 0; i < BITS; ++i) ww[i] = comp(w[i], q);
-                cb[q].prepare(ww);
-            }
-            int acc[NT][2][4];
-            auto step = [&](auto ksc, const uint4 (&b)[NT]) {
-                constexpr int KS = decltype(ksc)::value;
-                uint32_t p0[4], p1[4];
+                    for (int i = 0; i < BITS; ++i) ww[i] = comp(w[i], q);
+                    cb[q].prepare(ww);
+                }
+                int acc[NT][2][4];
+                auto step = [&](auto ksc, const uint4 (&b)[NT]) {
+                    constexpr int KS = decltype(ksc)::value;
+                    uint32_t p0[4], p1[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) cb[q].template operands<KS>(p0[q], p1[q]);
+                    for (int q = 0; q < 4; ++q) cb[q].template operands<KS>(p0[q], p1[q]);
 #pragma unroll
-                for (int t = 0; t < NT; ++t)
+                    for (int t = 0; t < NT; ++t)
 #pragma unroll
-                    for (int s = 0; s < 2; ++s)
-                        mma16832<KS == 0>(acc[t][s], p0[2 * s], p0[2 * s + 1], p1[2 * s], p1[2 * s + 1], (KS & 1) ? b[t].z : b[t].x,
-                                          (KS & 1) ? b[t].w : b[t].y);
-            };
-            step(IntC<0>(), b);
-            step(IntC<1>(), b);
+                        for (int s = 0; s < 2; ++s)
+                            mma16832<KS == 0>(acc[t][s], p0[2 * s], p0[2 * s + 1], p1[2 * s], p1[2 * s + 1], (KS & 1) ? b[t].z : b[t].x,
+                                              (KS & 1) ? b[t].w : b[t].y);
+                };
+                step(IntC<0>(), b);
+                step(IntC<1>(), b);
 #pragma unroll
-            for (int t = 0; t < NT; ++t) b[t] = lds128(b_at[t] + b_off + 256u);
-            step(IntC<2>(), b);
-            step(IntC<3>(), b);
-            if constexpr (INT) {
+                for (int t = 0; t < NT; ++t) b[t] = lds128(b_at[t] + b_off + 256u);
+                step(IntC<2>(), b);
+                step(IntC<3>(), b);
+                if constexpr (INT) {
 #pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const int S = (int)lds32(s_at[t] + s_off + (low_pair ? 0u : 4u));      // (the low pair: no sum)
+                    for (int t = 0; t < NT; ++t) {
+                        const int S = (int)lds32(s_at[t] + s_off + (low_pair ? 0u : 4u));      // (the low pair: no sum)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int v = acc[t][q >> 1][2 * (q & 1)] * 256 + acc[t][q >> 1][2 * (q & 1) + 1];
-                        const int add = low_pair ? v >> 6 : v * 1024 - S;
-                        out[t][q] = __int_as_float(__float_as_int(out[t][q]) + add);
+                        for (int q = 0; q < 4; ++q) {
+                            const int v = acc[t][q >> 1][2 * (q & 1)] * 256 + acc[t][q >> 1][2 * (q & 1) + 1];
+                            const int add = low_pair ? v >> 6 : v * 1024 - S;
+                            out[t][q] = __int_as_float(__float_as_int(out[t][q]) + add);
+                        }
+                    }
+                } else {
+                    const uint32_t zp = __byte_perm(z, 0u, 0x4140);
+                    const uint32_t ze = zp & 0x000F000Fu, zo = zp & 0x00F000F0u;    // as fp16 subnormals; columns 1 and 3 sixteen-fold
+                    const float2 zef = __half22float2(*reinterpret_cast<const __half2 *>(&ze));
+                    const float2 zof = __half22float2(*reinterpret_cast<const __half2 *>(&zo));
+                    const float2 s01 = __half22float2(*reinterpret_cast<const __half2 *>(&sc.x));
+                    const float2 s23 = __half22float2(*reinterpret_cast<const __half2 *>(&sc.y));
+                    const float zf[4] = {-zef.x, -zof.x, -zef.y, -zof.y}, sf[4] = {s01.x, s01.y, s23.x, s23.y};
+#pragma unroll
+                    for (int t = 0; t < NT; ++t) {
+                        const uint2 bs = lds64(s_at[t] + s_off);
+                        const float back = __uint_as_float(bs.x), S = __uint_as_float(bs.y), S16 = S * 0.0625f;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int v = acc[t][q >> 1][2 * (q & 1)] * 256 + acc[t][q >> 1][2 * (q & 1) + 1];
+                            const float u = fmaf(zf[q], (q & 1) ? S16 : S, (float)v);
+                            out[t][q] = fmaf(sf[q] * back, u, out[t][q]);
+                        }
                     }
                 }
-            } else {
-                const uint32_t zp = __byte_perm(z, 0u, 0x4140);
-                const uint32_t ze = zp & 0x000F000Fu, zo = zp & 0x00F000F0u;    // as fp16 subnormals; columns 1 and 3 sixteen-fold
-                const float2 zef = __half22float2(*reinterpret_cast<const __half2 *>(&ze));
-                const float2 zof = __half22float2(*reinterpret_cast<const __half2 *>(&zo));
-                const float2 s01 = __half22float2(*reinterpret_cast<const __half2 *>(&sc.x));
-                const float2 s23 = __half22float2(*reinterpret_cast<const __half2 *>(&sc.y));
-                const float zf[4] = {-zef.x, -zof.x, -zef.y, -zof.y}, sf[4] = {s01.x, s01.y, s23.x, s23.y};
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const uint2 bs = lds64(s_at[t] + s_off);
-                    const float back = __uint_as_float(bs.x), S = __uint_as_float(bs.y), S16 = S * 0.0625f;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int v = acc[t][q >> 1][2 * (q & 1)] * 256 + acc[t][q >> 1][2 * (q & 1) + 1];
-                        const float u = fmaf(zf[q], (q & 1) ? S16 : S, (float)v);
-                        out[t][q] = fmaf(sf[q] * back, u, out[t][q]);
-                    }
-                }
-            }
             };
             chunk(IntC<0>(), w2[0]);
             if (!(odd && u + 1 == np)) chunk(IntC<1>(), w2[1]);

@@ -1,8 +1,8 @@
 // Decode path: bit-serial table-lookup mpGEMV (paper Sec. 2.2 "Bit-serial table lookup", Fig. 2;
 // Sec. 4.3 "Mapping of LUT-based Decoding").
 //
-// One and two activation rows (and three and four where that is faster, uses_mma below) by table lookup, described here, short reductions
-// of them on the integer tensor cores (decode_digits.cuh, uses_digits below); more rows on the tensor cores (decode_mma.cuh).
+// One and two activation rows (and three and four where that is faster, uses_mma below) by table lookup, described here, or, short
+// reductions, on the integer tensor cores (decode_digits.cuh) where uses_digits says so; more rows on the tensor cores (decode_mma.cuh).
 //
 // Work split.  The reduction dimension is cut into K-slices of 16 or 32 plane words (16 for one
 // activation row; 32, 16 for 2, 3-4 rows, whose table entries carry the rows as fp16 pairs).  One
@@ -883,6 +883,9 @@ static DigitSplit split_digits(int rows, int K, int strips, int bits, int group,
         room = kDigitSmem;
         d.depth = rest + 2 * ring + turn <= room ? 2 : 1;
     }
+    // (on 148 SMs no call that comes here has one row of 4 bits in short groups with room for two units, or 2 bits in groups of 32 without)
+    if (bits == 4 && nb > 1 && rows == 1) d.depth = 1;
+    if (bits == 2 && nb == 4 && d.depth == 1) return d;
     const int base = rest + d.depth * ring;
     if (groups > kDigitGroups - kGemvMaxGroup || base + turn > room || (two && room > kDigitSmemHalf)) return d;
     d.tk_shift = kDigitWarpsShift;
@@ -907,13 +910,15 @@ static DigitSplit split_digits(int rows, int K, int strips, int bits, int group,
 // one row takes 0.979 of its time by lookup in the mean (a layer or MLP in 40 more than 2 % longer, at most 9 %), two rows in groups of 64 and
 // 128 0.921 (one in 170, at most 4 %).  Examples, by lookup / by this rule, 4-bit group 128: layer of 4096 x (6144, 4096, 28672) and
 // 14336 x 4096, one row 40.7 / 36.2 us, of 2048 x (3072, 2048, 16384) and 8192 x 2048 22.3 / 21.0, two rows 27.7 / 24.9.
-// Lines outside the model: six and more units a warp in one CTA an SM (3584 x 22784 and back, 4-bit 23.6 / 29.5), few columns
+// Lines outside the model: six and more units a warp in one CTA an SM (3584 x 22784 and back, 4-bit 22.6 / 28.3), few columns
 // (4096 x 512 3.3 / 4.8), two rows in groups of 32 (four tiles).  Calls of one group a CTA and at most two units, 2 and 4 bits
 // (4096 x 4096), gain more than the linear model says, 0.2 to 1.3 us.
 struct DigitPrice { float base, k, unit, tile, group, mb, two; };
 static const DigitPrice kDigitPrices[2][3] = {
-    {{-1.44f, 0.23f, 0.28f, 0.14f, 0.33f, -0.09f, -0.46f}, {-1.52f, 0.39f, 0.34f, 0.03f, 0.52f, -0.12f, -0.44f}, {-1.59f, 0.46f, 0.21f, 0.04f, 0.55f, -0.12f, -0.24f}},
-    {{-2.23f, 0.36f, 0.11f, 0.22f, 0.48f, -0.12f, 0.70f}, {-1.67f, 0.31f, 0.03f, 0.18f, 0.30f, -0.02f, 0.18f}, {-1.58f, 0.31f, -0.03f, 0.24f, 0.06f, -0.03f, 0.f}},
+    {{-1.44f, 0.23f, 0.28f, 0.14f, 0.33f, -0.09f, -0.46f}, {-1.52f, 0.39f, 0.34f, 0.03f, 0.52f, -0.12f, -0.44f},
+     {-1.59f, 0.46f, 0.21f, 0.04f, 0.55f, -0.12f, -0.24f}},
+    {{-2.23f, 0.36f, 0.11f, 0.22f, 0.48f, -0.12f, 0.70f}, {-1.67f, 0.31f, 0.03f, 0.18f, 0.30f, -0.02f, 0.18f},
+     {-1.58f, 0.31f, -0.03f, 0.24f, 0.06f, -0.03f, 0.f}},
 };
 static bool uses_digits(int bits, int group, int rows, int K, long long columns, int sms)
 {
@@ -1089,7 +1094,9 @@ static tman_status launch_digits(const DigitParams &p, int sms, cudaStream_t s)
 {
     const DigitSplit d = split_digits(p.M, p.K, p.strip0[kGemvMaxGroup], BITS, p.group, NB, INT, sms);
     if (d.flush < 1) return TMAN_ERR_UNSUPPORTED;
-    return d.depth == 2 ? launch_digits_split<BITS, NB, NT, 2, INT>(p, d, s) : launch_digits_split<BITS, NB, NT, 1, INT>(p, d, s);
+    if constexpr (BITS == 4 && NB > 1 && NT == NB / 2) return launch_digits_split<BITS, NB, NT, 1, INT>(p, d, s);     // (split_digits)
+    else if constexpr (BITS == 2 && NB == 4) return launch_digits_split<BITS, NB, NT, 2, INT>(p, d, s);
+    else return d.depth == 2 ? launch_digits_split<BITS, NB, NT, 2, INT>(p, d, s) : launch_digits_split<BITS, NB, NT, 1, INT>(p, d, s);
 }
 
 template <int BITS>
