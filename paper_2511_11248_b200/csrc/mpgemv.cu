@@ -906,10 +906,12 @@ static DigitSplit split_digits(int rows, int K, int strips, int bits, int group,
 // that the busiest warp takes (also where K does not fill the warps: 2176 takes as many as 4096) and the tiles of B that each is
 // multiplied with, groups, and megabytes of planes, which cost the lookups more.  Constants: least squares over graphs of layers,
 // MLPs and single calls with every call by either kernel, for 3600 draws of K = 1024..5120 and 256..40000 columns and for layers
-// of nine common shapes, plus half a change of kernel between neighbours (0.4 us) and 0.2 us of margin.  On 800 further draws
-// one row takes 0.979 of its time by lookup in the mean (a layer or MLP in 40 more than 2 % longer, at most 9 %), two rows in groups of 64 and
-// 128 0.921 (one in 170, at most 4 %).  Examples, by lookup / by this rule, 4-bit group 128: layer of 4096 x (6144, 4096, 28672) and
-// 14336 x 4096, one row 40.7 / 36.2 us, of 2048 x (3072, 2048, 16384) and 8192 x 2048 22.3 / 21.0, two rows 27.7 / 24.9.
+// of nine common shapes, plus half a change of kernel between neighbours (0.4 us) and 0.2 us of margin.  On 400 further draws
+// one row takes 0.979 of its time by lookup in the mean (a layer or MLP in 40 more than 2 % longer, at most 9 %).  Two rows go by it only
+// beyond the lines within which they come here in any case, because the lookups' fp16 sums are three times further from the exact product
+// (6.5e-4 of it against 2.1e-4): 0.905 in the mean, one layer or MLP in 30 more than 2 % longer (1920 x 9728 and back, 2-bit group 64 12 %).
+// Examples, by lookup / by this rule, 4-bit group 128: layer of 4096 x (6144, 4096, 28672) and 14336 x 4096, one row 40.7 / 36.2 us,
+// of 2048 x (3072, 2048, 16384) and 8192 x 2048 22.3 / 21.0, two rows 27.7 / 24.9.
 // Lines outside the model: six and more units a warp in one CTA an SM (3584 x 22784 and back, 4-bit 22.6 / 28.3), few columns
 // (4096 x 512 3.3 / 4.8), two rows in groups of 32 (four tiles).  Calls of one group a CTA and at most two units, 2 and 4 bits
 // (4096 x 4096), gain more than the linear model says, 0.2 to 1.3 us.
@@ -924,7 +926,10 @@ static bool uses_digits(int bits, int group, int rows, int K, long long columns,
 {
     if (rows > 2 || K > 5120 || columns > 40960 || columns * rows < K / 2 || (group == 32 && rows == 2)) return false;
     const DigitSplit d = split_digits(rows, K, (int)(columns / 4), bits, group, 128 / group, false, sms);
-    if (d.flush < 1 || (d.steps >= 6 && !d.two)) return false;
+    if (d.flush < 1) return false;
+    const bool badly_filled = K > 2048 && columns >= 96ll * sms && columns < 160ll * sms;
+    if (rows == 2 && columns <= (group == 128 ? 10 * K : K > 2048 ? 5120 : 8192) && !badly_filled) return true;
+    if (d.steps >= 6 && !d.two) return false;
     const int tiles = group == 128 ? 1 : group == 64 ? rows : 2;
     if (rows == 1 && tiles == 1 && bits != 3 && d.groups == 1 && d.steps <= 2 && d.ctas == sms) return true;
     const DigitPrice &c = kDigitPrices[rows - 1][bits - 2];

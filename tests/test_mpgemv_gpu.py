@@ -221,7 +221,7 @@ def test_one_and_two_rows_on_the_integer_tensor_cores(K, Ns, M, bits, G):
 
 
 @pytest.mark.parametrize("K,Ns,M,bits,G", [(4096, (504,), 1, 4, 128), (2048, (1032,), 2, 2, 32), (4096, (16392,), 1, 4, 128), (5248, (2504,), 1, 2, 64),
-                                           (3584, (1024, 2056), 1, 3, 64), (2048, (4096, 2056), 2, 3, 64)])
+                                           (3584, (1024, 2056), 1, 3, 64), (2304, (4096, 2056), 2, 3, 64)])
 def test_one_and_two_rows_beyond_the_rule_by_lookup(K, Ns, M, bits, G):
     # (two rows: the bound of test_rows_in_fp16_tables_stay_near_the_predicted_error)
     assert [p["kernel"] for p in B.tman_debug_gemv_plan(M, K, sum(Ns), bits, G)["passes"]] == ["lookup"]
