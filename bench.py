@@ -14,7 +14,7 @@ replay and the replay count.
 
 Also reported on the same JSON line: under roofline.prefill the prefill mpGEMM rate (M = 1024,
 K = 4096, N in {4096, 14336}, 4-bit, group 128) with its tensor roofline; under roofline.ceilings the
-lookup-rate and instruction-issue ceilings of the decode kernel; under config one-line digests of
+lookup-rate ceiling of the lookup kernel and the instruction-issue ceiling of the step's two kernels; under config one-line digests of
 configs 1, 3 and 5 measured in the same run; the end-to-end rate through the C ABI with host
 buffers; the CPU oracle's rate on a bounded sample; clocks sampled during the timed region.
 
@@ -421,7 +421,10 @@ def run_ours(args):
     }
     avg_launch_s = sec_step / launches_per_step
     ach = (abytes_step / launches_per_step) / avg_launch_s / 1e9
-    line["roofline"] = {"bound": "hbm", "kernel": "mpgemv_kernel (2-bit, M=1: BITS=2, MT=1, S=4, PRE, HALF, ROLL; grouped and single launches averaged)", "achieved": ach, "peak": peaks["hbm"],
+    (_, kx, ng), _, (_, kd, nd) = MLP
+    kernels = [KERNEL_NAMES[B.tman_debug_gemv_plan(1, K, N, BITS, GROUP)["passes"][0]["kernel"]] for K, N in ((kx, 2 * ng), (kd, nd))]
+    line["roofline"] = {"bound": "hbm", "kernel": f"{kernels[0]} (gate and up, one grouped call) and {kernels[1]} (down), 2-bit, one row; "
+                                                  "mean of the two launches", "achieved": ach, "peak": peaks["hbm"],
                         "unit": "GB/s", "frac": ach / peaks["hbm"], "traffic": TRAFFIC_BYTES_PER_LAUNCH,
                         "peak_source": f"of {peaks['src']}", "algorithmic_bytes_per_launch": abytes_step / launches_per_step}
 
@@ -441,25 +444,24 @@ def run_ours(args):
         print(json.dumps(line))
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch, from the ncu captures summarised under
-# profiles/.  mpGEMV: one gate/up-sized launch moved 17.04 MB for 16.78 MB of algorithmic bytes
-# (+1.5 %; counters re-taken on the present kernel build); traffic grows with the bytes streamed, so the step's mean launch (25.17 MB) is scaled
-# by the same ratio.
-TRAFFIC_BYTES_PER_LAUNCH = 25171968.0 * (17.04 / 16.78)
+KERNEL_NAMES = {"lookup": "mpgemv_kernel", "digits": "decode_digits_kernel", "mma": "decode_mma_kernel"}
+
+# dram__bytes_read.sum + dram__bytes_write.sum, from the ncu captures summarised under profiles/: the gate and up launch
+# (decode_digits_kernel) moved 33.98 MB, the down launch (mpgemv_kernel) 17.03 MB; the mean of the two, for 25.17 MB of algorithmic bytes.
+TRAFFIC_BYTES_PER_LAUNCH = (33984256.0 + 17032704.0) / 2
 
 
-# Warp instructions the decode kernel executes for one gate/up-sized launch (16.78 MB of algorithmic
-# bytes), from the ncu capture summarised under profiles/ (smsp__inst_executed.sum).
-DECODE_WARP_INSTRUCTIONS_PER_BYTE = 3.56e6 / 16.78e6
+# Warp instructions of the same two launches per algorithmic byte (smsp__inst_executed.sum).
+DECODE_WARP_INSTRUCTIONS_PER_BYTE = (6.409e6 + 3.461e6) / 50.34e6
 SCHEDULERS_PER_SM = 4
 
 
 def decode_ceilings(torch, B, clocks, bytes_per_launch, achieved_gbs):
-    """Two ceilings of the decode kernel other than HBM, in the units of roofline.achieved.
-    lookup: the rate at which one SM performs the kernel's lookup (8-bit index, 256-entry fp32 table in
+    """Two ceilings of the decode step other than HBM, in the units of roofline.achieved.
+    lookup: of the down call's kernel: the rate at which one SM performs its lookup (8-bit index, 256-entry fp32 table in
     shared memory, one add), measured now by the lookup microbenchmark; a lookup consumes one byte of a
     bit plane, and planes are 8/9 (2-bit, group 64) of the bytes streamed.
-    issue: the kernel's warp instructions per byte (from its ncu capture) at one instruction per clock
+    issue: both kernels' warp instructions per byte (from their ncu captures) at one instruction per clock
     per scheduler."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     mhz = clocks.get("sm_mhz") or clocks.get("sm_max_mhz") or 1965.0
@@ -474,8 +476,7 @@ def decode_ceilings(torch, B, clocks, bytes_per_launch, achieved_gbs):
     lookup_gbs = lookups_per_clk * sms * mhz * 1e6 / plane_share / 1e9
     issue_gbs = SCHEDULERS_PER_SM * sms * mhz * 1e6 / DECODE_WARP_INSTRUCTIONS_PER_BYTE / 1e9
     return {"unit": "GB/s", "sm_mhz": mhz,
-            "lookup": {"lookups_per_clk_per_sm": round(lookups_per_clk, 2), "GBs": round(lookup_gbs, 1),
-                       "achieved_frac": round(achieved_gbs / lookup_gbs, 3)},
+            "lookup": {"lookups_per_clk_per_sm": round(lookups_per_clk, 2), "GBs": round(lookup_gbs, 1)},
             "issue": {"warp_instructions_per_byte": round(DECODE_WARP_INSTRUCTIONS_PER_BYTE, 4),
                       "GBs": round(issue_gbs, 1), "achieved_frac": round(achieved_gbs / issue_gbs, 3)}}
 
