@@ -169,9 +169,9 @@ tman_status tman_quantize_rows(const void *x_f16, int M, int K, int qmax, int16_
 
 /* Decode of M rows (1 <= M <= 8; K <= 16384): the bit-serial table lookup of tman_mpgemv on integers, in passes of up to four
  * rows.  Tables hold exact integer sums of activations, lookups are shift-accumulated, the activation sum is subtracted once
- * (zero-point 1), K-slices are added as 32-bit integers.  Two rows and more with K <= 5120 and N >= K / (2 M) are multiplied on the
- * integer tensor cores instead, all rows in one pass, where their activations fit an SM's shared memory (seven rows of 4352 do
- * not).  Either way
+ * (zero-point 1), K-slices are added as 32-bit integers.  With K <= 5120 and N >= K / (2 M) two rows and more, and one row of few columns, are
+ * multiplied on the integer tensor cores instead, all rows in one pass, where their activations fit an SM's shared memory (seven
+ * rows of 4352 do not).  Either way
  *   y[m][n] = fp16( row_scale[m] * w_scale * sum_k a[m][k] * (q[k][n] - 1) ).
  * acc_i32 (device, int32 [M][N], 16-byte aligned, may be NULL) receives the exact integer sums.
  * Workspace: tman_workspace_bytes(3, M, K, N, 2, group), prepared with tman_workspace_init; status word

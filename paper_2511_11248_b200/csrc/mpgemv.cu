@@ -938,12 +938,15 @@ static bool uses_digits(int bits, int group, int rows, int K, long long columns,
     return us < (tiles > 1 ? -0.3f : 0.f);
 }
 
-// The same for the integer path, whose product follows a row quantization: products 2560 x 6912 and back in turn, each with its
-// quantization, two rows 13.8 / 13.6 us, six 28.9 / 23.1, eight (which the lookups take in two passes) 32.0 / 27.0; 4096 x 4096 two rows
-// 13.3 / 12.7, three 16.1 / 13.7.  One row stays with the lookups (ternary_decode of one row 47.1 / 48.4).
+// The same for the integer path, whose product follows a row quantization (sums are exact either way): products 2560 x 6912 and back in
+// turn, each with its quantization, two rows 13.8 by lookup / 13.6 us, six 28.9 / 23.1, eight (which the lookups take in two passes)
+// 32.0 / 27.0.  One row as far as the busiest warp has three units at most: of 250 drawn pairs of products none loses more than 1 %, 0.912 of the
+// time by lookup in the mean; with four units 10 % of them lose up to 7 % (3584 x 5504 and back 12.1 / 13.0).
 static bool uses_digits_ternary(int rows, int K, int N, int group, int sms)
 {
-    return rows >= 2 && K <= 5120 && (long long)N * rows >= K / 2 && split_digits(rows, K, N / 4, 2, group, 1, true, sms).flush > 0;
+    if (K > 5120 || (long long)N * rows < K / 2) return false;
+    const DigitSplit d = split_digits(rows, K, N / 4, 2, group, 1, true, sms);
+    return d.flush > 0 && (rows >= 2 || d.steps <= 3);
 }
 
 GemvPlan plan_gemv(int M, int K, int N, int bits, int group, int sms, size_t ws_limit)

@@ -223,7 +223,8 @@ def test_ternary_decode_with_several_rows(M, K, N, group):
 
 # an odd number of 128-deep chunks, ragged columns, an odd row in the last pair of rows; rings of one unit and of two; teams of eight to two
 # warps; two CTAs an SM; several reductions; half an SM's shared memory and all of it
-@pytest.mark.parametrize("M,K,N,group", [(2, 640, 1032, 32), (3, 1152, 1288, 64), (5, 2176, 2568, 128), (6, 1920, 1928, 64), (7, 2176, 2056, 128), (8, 1152, 520, 32),
+@pytest.mark.parametrize("M,K,N,group", [(1, 640, 328, 64), (1, 2176, 2568, 32), (1, 2560, 6912, 128), (1, 5120, 2568, 64), (1, 640, 19064, 128),
+                                         (2, 640, 1032, 32), (3, 1152, 1288, 64), (5, 2176, 2568, 128), (6, 1920, 1928, 64), (7, 2176, 2056, 128), (8, 1152, 520, 32),
                                          (2, 3712, 2456, 128), (4, 2304, 4360, 32), (3, 3456, 5312, 128), (7, 1152, 7488, 64), (6, 1408, 5040, 128),
                                          (2, 640, 19064, 128), (4, 640, 9512, 64), (8, 640, 4776, 128), (3, 640, 24008, 128), (5, 3968, 1096, 128), (2, 5120, 2568, 64)])
 def test_ternary_decode_with_several_rows_on_the_integer_tensor_cores(M, K, N, group):
@@ -231,7 +232,7 @@ def test_ternary_decode_with_several_rows_on_the_integer_tensor_cores(M, K, N, g
     check_several_rows(M, K, N, group, prepared=False)
 
 
-@pytest.mark.parametrize("M,K,N", [(2, 5120, 2568), (3, 1152, 1288), (6, 2176, 1032), (8, 1152, 520)])
+@pytest.mark.parametrize("M,K,N", [(1, 2560, 2568), (2, 5120, 2568), (3, 1152, 1288), (6, 2176, 1032), (8, 1152, 520)])
 def test_ternary_decode_of_the_largest_integers(M, K, N):
     # the first columns' weights have the signs of the rows, so that the sums are as large as they can be; -32768 is no quantized value, but
     # the call takes it
