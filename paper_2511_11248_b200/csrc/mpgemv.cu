@@ -806,6 +806,9 @@ static const GemvVariant kGemvVariants[kGemvVariantCount] = {
 // there (three rows, 18944 x 3584: 2-bit, group 128 12.0 / 13.3, 3-bit, group 64 14.1 / 15.0; 2-bit, group 64, 11008 x 4096 9.6 / 10.5); such
 // calls stay on the tensor cores, whose sums are fp32 throughout: the lookups' fp16 ones are three times further from the exact product.
 // One and two rows are cheaper by lookup (4-bit, group 128, two rows: 17.2 / 18.4).
+// (Lookup times from before activations came by ordinary loads; they take 0.5 to 1 us a call more now.  Over 450 drawn layers, MLPs and calls
+// every class of three and four rows in groups of 64 and 128 is still faster here in the mean, by 0.5 to 3 us a call, two rows are not, by up
+// to 1.7, nor groups of 32 above about 10 million weights.)
 static bool uses_mma(int bits, int group, int rows, long long weights)
 {
     return rows >= 5 || (rows >= 3 && group >= 64 && (bits >= 3 || group == 128 || weights <= 48000000ll));
